@@ -351,21 +351,49 @@ cudaError_t launch_onetime(const Group &g, int p0, int np, const uint64_t *P, in
 // chi_lin = C(0) + 2 sum_{0 < tau < L_tau/2} C(tau) + C(L_tau/2), C averaged
 // over replicas.  Per k: disorder averages over the group's samples and
 // xi = sqrt(chi / F - 1) / (2 sin(pi / L)), B = mean q4 / (mean q2)^2.
+//
+// A warp per (sample, k): the lanes sum the int64 correlator sums of chi_lin
+// over the lags (coalesced, exact integers) and one division normalises their
+// total.  The work is the read of the correlator sums; with one thread per
+// (sample, k) and a division per lag it was a chain of R L_tau / 2 dependent
+// FP64 divisions and adds on at most n_samples K threads (64 samples, 8 k,
+// R = 4, L_tau = 2048: 3,280 us; this form 14 us).
 // ---------------------------------------------------------------------------
-__global__ void k_onetime_finish(Group g, double nm, int triples) {
+constexpr int kFinishWarps = 8;
+
+__global__ void __launch_bounds__(32 * kFinishWarps) k_onetime_finish(Group g, double nm, int triples) {
     const int H = g.L / 2, R = g.R, K = g.K, nl = g.nlag;
     const double LD = (double)(g.L * g.L), Lt = (double)g.Ltau;
     const double npair = (double)(R * (R - 1) / 2), ntrip = (double)(R * (R - 1) * (R - 2) / 6);
     const bool has3 = triples && R >= 3 && R <= kMaxTripleR;
+    const int lane = threadIdx.x & 31;
     const int total = g.n_samples * K;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * kFinishWarps + (int)(threadIdx.x >> 5); i < total; i += gridDim.x * kFinishWarps) {
         const int s = i / K, j = i % K;
         const size_t c = (size_t)s * K + j;  // the sample index equals the bit index w * 64 + b
+        // chi_lin: per lane an exact integer sum per replica; the total is
+        // exact in FP64 too while it stays below 2^53
+        double cl = 0.0;
+        for (int r = 0; r < R; ++r) {
+            const long long *Cr = g.Cacc + (((size_t)r * g.W * 64 + s) * K + j) * nl;
+            long long part = 0;
+            for (int lag = lane; lag < nl; lag += 32) part += (lag == 0 || lag == nl - 1) ? Cr[lag] : 2 * Cr[lag];
+            cl = __dadd_rn(cl, (double)part);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) cl = __dadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, o));
+        // momentum sums: lane d holds the term of lag d, added in increasing d
+        double tG = 0.0, tF = 0.0;
+        if (lane <= H) {
+            tG = __dmul_rn(g.wcos[lane], (double)g.Gacc[c * (H + 1) + lane]);
+            tF = __dmul_rn(g.wcos[lane], (double)g.F3acc[c * (H + 1) + lane]);
+        }
         double G = 0.0, F3 = 0.0;
         for (int d = 0; d <= H; ++d) {
-            G = __dadd_rn(G, __dmul_rn(g.wcos[d], (double)g.Gacc[c * (H + 1) + d]));
-            F3 = __dadd_rn(F3, __dmul_rn(g.wcos[d], (double)g.F3acc[c * (H + 1) + d]));
+            G = __dadd_rn(G, __shfl_sync(0xffffffffu, tG, d));
+            F3 = __dadd_rn(F3, __shfl_sync(0xffffffffu, tF, d));
         }
+        if (lane != 0) continue;
         const double p4 = __dadd_rn(__dmul_rn((double)g.P4acc[2 * c + 1], 4294967296.0), (double)g.P4acc[2 * c]);
         double *o = g.outO + c * 7;
         o[0] = __ddiv_rn((double)g.Pacc[c], nm * npair * LD * LD * Lt);
@@ -374,28 +402,22 @@ __global__ void k_onetime_finish(Group g, double nm, int triples) {
         o[3] = __ddiv_rn(G, 2.0 * nm * npair * Lt * LD);
         o[4] = has3 ? __ddiv_rn((double)g.T3acc[c], nm * ntrip * Lt * LD) : __longlong_as_double(0x7ff8000000000000LL);
         o[5] = has3 ? __ddiv_rn(F3, 6.0 * nm * ntrip * Lt * LD) : __longlong_as_double(0x7ff8000000000000LL);
-        double cl = 0.0;
-        for (int r = 0; r < R; ++r) {
-            const long long *Cr = g.Cacc + (((size_t)r * g.W * 64 + s) * K + j) * nl;
-            double sr = 0.0;
-            for (int lag = 0; lag < nl; ++lag) {
-                const double v = __ddiv_rn((double)Cr[lag], __dmul_rn(__dmul_rn(nm, LD), Lt));
-                sr = __dadd_rn(sr, (lag == 0 || lag == nl - 1) ? v : __dmul_rn(2.0, v));
-            }
-            cl = __dadd_rn(cl, sr);
-        }
-        o[6] = __ddiv_rn(cl, (double)R);
+        o[6] = __ddiv_rn(__ddiv_rn(cl, __dmul_rn(__dmul_rn(nm, LD), Lt)), (double)R);
     }
 }
 
-__global__ void k_onetime_average(Group g) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= g.K) return;
+// Disorder averages of one k per block, a warp per observable.
+__global__ void __launch_bounds__(224) k_onetime_average(Group g) {
+    __shared__ double m[7];
+    const int j = blockIdx.x, f = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = g.K, ns = g.n_samples;
-    double m[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int s = 0; s < ns; ++s)
-        for (int f = 0; f < 7; ++f) m[f] = __dadd_rn(m[f], g.outO[((size_t)s * K + j) * 7 + f]);
-    for (int f = 0; f < 7; ++f) m[f] = __ddiv_rn(m[f], (double)ns);
+    double v = 0.0;
+    for (int s = lane; s < ns; s += 32) v = __dadd_rn(v, g.outO[((size_t)s * K + j) * 7 + f]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) m[f] = __ddiv_rn(v, (double)ns);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     const double s2 = g.xi_norm;  // 2 sin(pi / L), host FP64
     double *o = g.outK + (size_t)j * 8;
     o[0] = m[2];
@@ -410,13 +432,13 @@ __global__ void k_onetime_average(Group g) {
 
 cudaError_t launch_onetime_finish(const Group &g, long long n_meas, int triples, cudaStream_t st) {
     const int total = g.n_samples * g.K;
-    int blocks = (total + 255) / 256;
+    int blocks = (total + kFinishWarps - 1) / kFinishWarps;
     if (blocks > 152 * 8) blocks = 152 * 8;
     count_launches(2);
-    k_onetime_finish<<<blocks, 256, 0, st>>>(g, (double)n_meas, triples);
+    k_onetime_finish<<<blocks, 32 * kFinishWarps, 0, st>>>(g, (double)n_meas, triples);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_onetime_average<<<(g.K + 127) / 128, 128, 0, st>>>(g);
+    k_onetime_average<<<g.K, 224, 0, st>>>(g);
     return cudaGetLastError();
 }
 
