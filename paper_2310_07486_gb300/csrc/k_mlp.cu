@@ -5,13 +5,19 @@
 // Loss of a batch: mean over its samples of the cross-entropy between
 // softmax(y[0:32]) and the target fractions t[0:32], plus (y[32] - t[32])^2.
 //
-// A training step is two launches: k_mlp_grad (one block per tile of 16
-// samples: forward, loss, backward, the tile's gradient written to its own
-// slice of a partial-gradient buffer) and k_mlp_adam (one thread per
-// parameter: the tiles' partial gradients summed in tile order, then Adam).
-// Every sum runs in a fixed order, so training is deterministic.  The layer
-// products are a few MFLOP per step; they run on the FP32 pipes from shared
-// memory, where the launch latency, not the arithmetic, sets the time.
+// Training is one cooperative launch per call of qsg_mlp_train (up to 256
+// steps): per step, the blocks compute the gradients of the batch's tiles of 16
+// samples (forward, loss, backward) into a partial-gradient buffer, meet at a
+// grid barrier, sum the tiles' partial gradients in tile order and apply Adam
+// (one thread per parameter), and meet again.  Every sum runs in a fixed
+// order, so training is deterministic.  A step is a few MFLOP on 29k
+// parameters, so what counts is latency: the weights are staged in shared
+// memory once per tile with 16-byte loads, in rows padded so that both the
+// forward products (16-byte reads along a row, one row per lane) and the
+// backward ones (4-byte reads along a column index, one column per lane) are
+// free of bank conflicts, and 512 threads share a tile.  With one thread per
+// hidden unit, weights read from global memory for every sample and two
+// launches per step, a step of 128 samples took 280 us; it takes 28 us now.
 #include <cmath>
 
 #include <cuda_bf16.h>
@@ -25,227 +31,426 @@ constexpr int oW1 = 0, oB1 = oW1 + kH * kIn, oW2 = oB1 + kH, oB2 = oW2 + kH * kH
               oB3 = oW3 + kOut * kH, kParams = oB3 + kOut;
 static_assert(kParams == 29089, "parameter layout");
 
+constexpr int kMlpThreads = 512;
+// rows padded by 16 bytes: a quarter warp's eight 16-byte reads of eight
+// consecutive rows fall into different banks
+constexpr int kP1 = kIn + 4, kPH = kH + 4;
+
+// The weights in shared memory.
+struct Weights {
+    float W1[kH][kP1];
+    float W2[kH][kPH];
+    float W3[kOut][kPH];
+    float b1[kH], b2[kH], b3[kOut + 3];
+};
+
+// Activations and gradients of one tile.
+struct Tile {
+    float x[kTile][kP1];
+    float z1[kTile][kPH], z2[kTile][kPH];  // before the ReLU
+    float y[kTile][kOut + 3];
+    float dyT[kOut + 3][kTile], d2T[kH][kTile], d1T[kH][kTile];  // dL/dy, dL/dz2, dL/dz1 by unit
+    float lsum[kTile];
+};
+
 int mlp_param_count() { return kParams; }
 
-// One tile of samples idx[t0 .. t0+nt): forward, loss, backward.
-__global__ void __launch_bounds__(128) k_mlp_grad(const float *__restrict__ P, const float *__restrict__ X,
-                                                  const float *__restrict__ T, const int *__restrict__ idx,
-                                                  int batch, float *__restrict__ partial,
-                                                  float *__restrict__ loss_partial) {
-    __shared__ float x[kTile][kIn];
-    __shared__ float z1[kTile][kH], z2[kTile][kH];
-    __shared__ float y[kTile][kOut], dy[kTile][kOut];
-    __shared__ float d2[kTile][kH], d1[kTile][kH];
-    __shared__ float lsum[kTile];
-    const int tid = threadIdx.x, t0 = blockIdx.x * kTile;
-    const int nt = min(kTile, batch - t0);
-    const float inv_b = 1.0f / (float)batch;
-    for (int i = tid; i < kTile * kIn; i += 128) {
-        const int s = i / kIn, f = i % kIn;
-        x[s][f] = s < nt ? X[(size_t)idx[t0 + s] * kIn + f] : 0.0f;
+// Copy the parameters to shared memory, asynchronously (every load in flight
+// at once) and past L1 (the previous step of the same launch wrote them). The
+// caller's next barrier follows stage_wait.
+__device__ __forceinline__ void stage_weights(const float *P, Weights &w) {
+    const int tid = threadIdx.x;
+    auto rows = [&](const float *src, float *dst, int n, int len, int pitch) {
+        const int q = len / 4;
+#pragma unroll 8
+        for (int e = tid; e < n * q; e += kMlpThreads)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(dst + (e / q) * pitch + 4 * (e % q))),
+                         "l"(src + 4 * e)
+                         : "memory");
+    };
+    rows(P + oW1, &w.W1[0][0], kH, kIn, kP1);
+    rows(P + oW2, &w.W2[0][0], kH, kH, kPH);
+    rows(P + oW3, &w.W3[0][0], kOut, kH, kPH);
+    if (tid < kH) {
+        w.b1[tid] = __ldcg(P + oB1 + tid);
+        w.b2[tid] = __ldcg(P + oB2 + tid);
+        if (tid < kOut) w.b3[tid] = __ldcg(P + oB3 + tid);
     }
-    __syncthreads();
-    // layer 1 and 2: thread = hidden unit
-    {
-        const int j = tid;
-        for (int s = 0; s < nt; ++s) {
-            float a = P[oB1 + j];
-            for (int i = 0; i < kIn; ++i) a = fmaf(P[oW1 + j * kIn + i], x[s][i], a);
-            z1[s][j] = a;
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// acc[k] += row . a[k] over n (a multiple of 4) terms in increasing order; `in`
+// maps an activation before it is used.
+template <int S, class In>
+__device__ __forceinline__ void dots(const float *row, const float *const (&a)[S], int n, float (&acc)[S], In &&in) {
+#pragma unroll 4
+    for (int i = 0; i < n; i += 4) {
+        const float4 w = *reinterpret_cast<const float4 *>(row + i);
+#pragma unroll
+        for (int k = 0; k < S; ++k) {
+            const float4 v = *reinterpret_cast<const float4 *>(a[k] + i);
+            acc[k] = fmaf(w.x, in(v.x), acc[k]);
+            acc[k] = fmaf(w.y, in(v.y), acc[k]);
+            acc[k] = fmaf(w.z, in(v.z), acc[k]);
+            acc[k] = fmaf(w.w, in(v.w), acc[k]);
         }
     }
-    __syncthreads();
-    {
-        const int j = tid;
-        for (int s = 0; s < nt; ++s) {
-            float a = P[oB2 + j];
-            for (int i = 0; i < kH; ++i) a = fmaf(P[oW2 + j * kH + i], fmaxf(z1[s][i], 0.0f), a);
-            z2[s][j] = a;
-        }
+}
+
+__device__ __forceinline__ float relu(float v) { return fmaxf(v, 0.0f); }
+
+// Forward, loss and backward of samples idx[t0 .. t0 + nt) (nt <= 16); the
+// tile's gradient goes to G, its loss to *loss.  Units of the padding samples
+// are computed from zeros and never written.
+__device__ void tile_gradient(const Weights &w, Tile &t, const float *__restrict__ X, const float *__restrict__ T,
+                              const int *__restrict__ idx, int t0, int nt, float inv_b, float *__restrict__ G,
+                              float *loss) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < kTile * (kIn / 4); e += kMlpThreads) {
+        const int s = e / (kIn / 4), q = e % (kIn / 4);
+        const float4 v = s < nt ? __ldg(reinterpret_cast<const float4 *>(X + (size_t)idx[t0 + s] * kIn) + q)
+                                : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        *reinterpret_cast<float4 *>(&t.x[s][4 * q]) = v;
     }
     __syncthreads();
-    for (int e = tid; e < nt * kOut; e += 128) {
+    // layers 1 and 2: thread = (hidden unit, four samples)
+    const int j = tid & (kH - 1), s0 = 4 * (tid >> 7);
+    {
+        float a[4] = {w.b1[j], w.b1[j], w.b1[j], w.b1[j]};
+        const float *const in[4] = {t.x[s0], t.x[s0 + 1], t.x[s0 + 2], t.x[s0 + 3]};
+        dots<4>(w.W1[j], in, kIn, a, [](float v) { return v; });
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t.z1[s0 + k][j] = a[k];
+    }
+    __syncthreads();
+    {
+        float a[4] = {w.b2[j], w.b2[j], w.b2[j], w.b2[j]};
+        const float *const in[4] = {t.z1[s0], t.z1[s0 + 1], t.z1[s0 + 2], t.z1[s0 + 3]};
+        dots<4>(w.W2[j], in, kH, a, relu);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t.z2[s0 + k][j] = a[k];
+    }
+    __syncthreads();
+    // layer 3: thread = (output, sample); 33 outputs x 16 samples
+    for (int e = tid; e < kOut * kTile; e += kMlpThreads) {
         const int s = e / kOut, o = e % kOut;
-        float a = P[oB3 + o];
-        for (int i = 0; i < kH; ++i) a = fmaf(P[oW3 + o * kH + i], fmaxf(z2[s][i], 0.0f), a);
-        y[s][o] = a;
+        float a[1] = {w.b3[o]};
+        const float *const in[1] = {t.z2[s]};
+        dots<1>(w.W3[o], in, kH, a, relu);
+        t.y[s][o] = a[0];
     }
     __syncthreads();
-    // loss and dL/dy per sample (thread = sample)
-    if (tid < nt) {
-        const int s = tid;
-        const float *t = T + (size_t)idx[t0 + s] * kOut;
-        float mx = y[s][0];
-        for (int o = 1; o < 32; ++o) mx = fmaxf(mx, y[s][o]);
-        float se = 0.0f, tsum = 0.0f;
-        for (int o = 0; o < 32; ++o) {
-            se += expf(y[s][o] - mx);
-            tsum += t[o];
+    // loss and dL/dy: warp = sample, lane = output; sums in output order
+    {
+        const int s = warp;
+        if (s < nt) {
+            const float *tt = T + (size_t)idx[t0 + s] * kOut;
+            const float yo = t.y[s][lane], to = __ldg(tt + lane);
+            float mx = yo;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            const float ex = expf(yo - mx);
+            float se = 0.0f, tsum = 0.0f;
+#pragma unroll
+            for (int o = 0; o < 32; ++o) {
+                se += __shfl_sync(0xffffffffu, ex, o);
+                tsum += __shfl_sync(0xffffffffu, to, o);
+            }
+            const float lse = logf(se);
+            const float logp = yo - mx - lse;
+            float ce = 0.0f;
+#pragma unroll
+            for (int o = 0; o < 32; ++o)
+                ce -= __shfl_sync(0xffffffffu, to, o) * __shfl_sync(0xffffffffu, logp, o);
+            t.dyT[lane][s] = (expf(logp) * tsum - to) * inv_b;
+            if (lane == 0) {
+                const float r = t.y[s][32] - __ldg(tt + 32);
+                t.dyT[32][s] = 2.0f * r * inv_b;
+                t.lsum[s] = ce + r * r;
+            }
+        } else {
+            t.dyT[lane][s] = 0.0f;
+            if (lane == 0) t.dyT[32][s] = 0.0f;
         }
-        const float lse = logf(se);
-        float ce = 0.0f;
-        for (int o = 0; o < 32; ++o) {
-            const float logp = y[s][o] - mx - lse;
-            ce -= t[o] * logp;
-            dy[s][o] = (expf(logp) * tsum - t[o]) * inv_b;
-        }
-        const float r = y[s][32] - t[32];
-        dy[s][32] = 2.0f * r * inv_b;
-        lsum[s] = ce + r * r;
     }
     __syncthreads();
     if (tid == 0) {
         float l = 0.0f;
-        for (int s = 0; s < nt; ++s) l += lsum[s];
-        loss_partial[blockIdx.x] = l * inv_b;
+        for (int s = 0; s < nt; ++s) l += t.lsum[s];
+        *loss = l * inv_b;
     }
-    float *G = partial + (size_t)blockIdx.x * kParams;
-    // layer 3 gradients; dL/dz2
-    for (int e = tid; e < kOut * kH; e += 128) {
-        const int o = e / kH, i = e % kH;
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a = fmaf(dy[s][o], fmaxf(z2[s][i], 0.0f), a);
-        G[oW3 + e] = a;
-    }
-    if (tid < kOut) {
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a += dy[s][tid];
-        G[oB3 + tid] = a;
-    }
+    // dL/dz2: thread = (unit, four samples)
     {
-        const int j = tid;
-        for (int s = 0; s < nt; ++s) {
+        float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 3
+        for (int o = 0; o < kOut; ++o) {
+            const float4 d = *reinterpret_cast<const float4 *>(&t.dyT[o][s0]);
+            const float wv = w.W3[o][j];
+            a[0] = fmaf(d.x, wv, a[0]);
+            a[1] = fmaf(d.y, wv, a[1]);
+            a[2] = fmaf(d.z, wv, a[2]);
+            a[3] = fmaf(d.w, wv, a[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = t.z2[s0 + k][j] > 0.0f ? a[k] : 0.0f;
+        *reinterpret_cast<float4 *>(&t.d2T[j][s0]) = make_float4(a[0], a[1], a[2], a[3]);
+    }
+    // weight gradient rows [0, n) of a layer: thread = (input i, every step-th
+    // row); the inputs of the sixteen samples stay in registers
+    auto weight_grad = [&](const float (*dT)[kTile], int n, const float (&v)[kTile], int i, int r0, int step, int len,
+                           float *Gw) {
+        for (int r = r0; r < n; r += step) {
             float a = 0.0f;
-            for (int o = 0; o < kOut; ++o) a = fmaf(dy[s][o], P[oW3 + o * kH + j], a);
-            d2[s][j] = z2[s][j] > 0.0f ? a : 0.0f;
+            const float4 *d = reinterpret_cast<const float4 *>(dT[r]);
+#pragma unroll
+            for (int q = 0; q < kTile / 4; ++q) {
+                const float4 dv = d[q];
+                if (4 * q + 0 < nt) a = fmaf(dv.x, v[4 * q + 0], a);
+                if (4 * q + 1 < nt) a = fmaf(dv.y, v[4 * q + 1], a);
+                if (4 * q + 2 < nt) a = fmaf(dv.z, v[4 * q + 2], a);
+                if (4 * q + 3 < nt) a = fmaf(dv.w, v[4 * q + 3], a);
+            }
+            Gw[r * len + i] = a;
         }
-    }
-    __syncthreads();
-    // layer 2 gradients; dL/dz1
-    for (int e = tid; e < kH * kH; e += 128) {
-        const int j = e / kH, i = e % kH;
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a = fmaf(d2[s][j], fmaxf(z1[s][i], 0.0f), a);
-        G[oW2 + e] = a;
-    }
-    {
-        const int j = tid;
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a += d2[s][j];
-        G[oB2 + j] = a;
-        for (int s = 0; s < nt; ++s) {
-            float c = 0.0f;
-            for (int k = 0; k < kH; ++k) c = fmaf(d2[s][k], P[oW2 + k * kH + j], c);
-            d1[s][j] = z1[s][j] > 0.0f ? c : 0.0f;
+    };
+    auto bias_grad = [&](const float (*dT)[kTile], int n, float *Gb) {
+        if (tid < n) {
+            float a = 0.0f;
+            for (int s = 0; s < nt; ++s) a += dT[tid][s];
+            Gb[tid] = a;
         }
-    }
+    };
+    float v[kTile];
+#pragma unroll
+    for (int s = 0; s < kTile; ++s) v[s] = relu(t.z2[s][j]);
+    weight_grad(t.dyT, kOut, v, j, tid >> 7, kMlpThreads / kH, kH, G + oW3);
+    bias_grad(t.dyT, kOut, G + oB3);
     __syncthreads();
-    // layer 1 gradients
-    for (int e = tid; e < kH * kIn; e += 128) {
-        const int j = e / kIn, i = e % kIn;
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a = fmaf(d1[s][j], x[s][i], a);
-        G[oW1 + e] = a;
-    }
+    // dL/dz1
     {
-        const int j = tid;
-        float a = 0.0f;
-        for (int s = 0; s < nt; ++s) a += d1[s][j];
-        G[oB1 + j] = a;
+        float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+        for (int k = 0; k < kH; ++k) {
+            const float4 d = *reinterpret_cast<const float4 *>(&t.d2T[k][s0]);
+            const float wv = w.W2[k][j];
+            a[0] = fmaf(d.x, wv, a[0]);
+            a[1] = fmaf(d.y, wv, a[1]);
+            a[2] = fmaf(d.z, wv, a[2]);
+            a[3] = fmaf(d.w, wv, a[3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = t.z1[s0 + k][j] > 0.0f ? a[k] : 0.0f;
+        *reinterpret_cast<float4 *>(&t.d1T[j][s0]) = make_float4(a[0], a[1], a[2], a[3]);
     }
+#pragma unroll
+    for (int s = 0; s < kTile; ++s) v[s] = relu(t.z1[s][j]);
+    weight_grad(t.d2T, kH, v, j, tid >> 7, kMlpThreads / kH, kH, G + oW2);
+    bias_grad(t.d2T, kH, G + oB2);
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < kTile; ++s) v[s] = t.x[s][tid & (kIn - 1)];
+    weight_grad(t.d1T, kH, v, tid & (kIn - 1), tid >> 6, kMlpThreads / kIn, kIn, G + oW1);
+    bias_grad(t.d1T, kH, G + oB1);
 }
 
-// Sum the tiles' partial gradients (tile order) and apply one Adam step
-// (Kingma & Ba 2015) at step number t, or only write the gradient (adam = 0).
-__global__ void k_mlp_adam(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V,
-                           const float *__restrict__ partial, int ntiles, float *__restrict__ grad_out,
-                           int adam, float lr, float c1, float c2, const float *__restrict__ loss_partial,
-                           float *__restrict__ loss_out) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && loss_out) {
-        float l = 0.0f;
-        for (int b = 0; b < ntiles; ++b) l += loss_partial[b];
-        *loss_out = l;
+// Barrier over the blocks of a cooperative launch: `count` is the number of
+// arrivals so far of the launch (a multiple of the grid before the first).
+// False, and *status set, when the wait gives up after `limit` polls.
+__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned goal, int *status, unsigned limit) {
+    __shared__ int ok;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(count, 1u);
+        int got = 0;
+        for (unsigned it = 0; it < limit && !got; ++it) got = *(volatile unsigned *)count >= goal;
+        if (!got) atomicExch(status, (int)DEVERR_TIMEOUT);
+        ok = got;
     }
-    if (p >= kParams) return;
-    float g = 0.0f;
-    for (int b = 0; b < ntiles; ++b) g += partial[(size_t)b * kParams + p];
-    if (grad_out) grad_out[p] = g;
-    if (!adam) return;
-    const float m = 0.9f * M[p] + 0.1f * g;
-    const float v = 0.999f * V[p] + 0.001f * g * g;
-    M[p] = m;
-    V[p] = v;
-    // c1 = 1 - 0.9^t, c2 = 1 - 0.999^t (host FP64, rounded once)
-    P[p] -= lr * (m / c1) / (sqrtf(v / c2) + 1e-8f);
+    __syncthreads();
+    __threadfence();
+    return ok != 0;
 }
 
-cudaError_t launch_mlp_step(float *P, float *M, float *V, const float *X, const float *T, const int *idx, int batch,
-                            float *partial, float *loss_partial, float *grad_out, int adam, float lr, int t,
-                            float *loss_out, cudaStream_t st) {
+// `steps` training steps (adam != 0) or one gradient (adam = 0, grad_out).
+// idx: [steps][batch] sample indices; corr: [steps][2] Adam's 1 - 0.9^t and
+// 1 - 0.999^t (host FP64, rounded once); sync: {barrier count, status}, zero
+// at launch.
+__global__ void __launch_bounds__(kMlpThreads, 1)
+    k_mlp_train(float *P, float *__restrict__ M, float *__restrict__ V, const float *__restrict__ X,
+                const float *__restrict__ T, const int *__restrict__ idx, int steps, int batch, float *partial,
+                float *loss_partial, float *grad_out, int adam, float lr, const float *__restrict__ corr,
+                float *loss_out, unsigned *sync, unsigned wait_limit) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    Weights &w = *reinterpret_cast<Weights *>(mlp_smem);
+    Tile &t = *reinterpret_cast<Tile *>(mlp_smem + sizeof(Weights));
     const int ntiles = (batch + kTile - 1) / kTile;
-    count_launches(2);
-    k_mlp_grad<<<ntiles, 128, 0, st>>>(P, X, T, idx, batch, partial, loss_partial);
-    cudaError_t e = cudaGetLastError();
+    const float inv_b = 1.0f / (float)batch;
+    unsigned goal = 0;
+    for (int step = 0; step < steps; ++step) {
+        const int *ix = idx + (size_t)step * batch;
+        if ((int)blockIdx.x < ntiles) {
+            stage_weights(P, w);
+            stage_wait();  // the barrier after the tile's inputs follows
+            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+                const int t0 = tile * kTile;
+                tile_gradient(w, t, X, T, ix, t0, min(kTile, batch - t0), inv_b, partial + (size_t)tile * kParams,
+                              loss_partial + tile);
+                __syncthreads();  // the tile's buffers are reused
+            }
+        }
+        goal += gridDim.x;
+        if (!grid_barrier(sync, goal, reinterpret_cast<int *>(sync + 1), wait_limit)) return;
+        const float c1 = corr[2 * step], c2 = corr[2 * step + 1];
+        for (int p = blockIdx.x * kMlpThreads + threadIdx.x; p < kParams; p += gridDim.x * kMlpThreads) {
+            float g = 0.0f;
+#pragma unroll 8
+            for (int b = 0; b < ntiles; ++b) g += __ldcg(partial + (size_t)b * kParams + p);
+            if (grad_out) grad_out[p] = g;
+            if (adam) {
+                // Adam (Kingma & Ba 2015)
+                const float m = 0.9f * M[p] + 0.1f * g;
+                const float v = 0.999f * V[p] + 0.001f * g * g;
+                M[p] = m;
+                V[p] = v;
+                P[p] -= lr * (m / c1) / (sqrtf(v / c2) + 1e-8f);
+            }
+        }
+        if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+            float l = 0.0f;
+            for (int b = 0; b < ntiles; ++b) l += __ldcg(loss_partial + b);
+            loss_out[step] = l;
+        }
+        if (step + 1 == steps) break;
+        goal += gridDim.x;
+        if (!grid_barrier(sync, goal, reinterpret_cast<int *>(sync + 1), wait_limit)) return;
+    }
+}
+
+cudaError_t launch_mlp_steps(float *P, float *M, float *V, const float *X, const float *T, const int *idx, int steps,
+                             int batch, float *partial, float *loss_partial, float *grad_out, int adam, float lr,
+                             const float *corr, float *loss_out, unsigned *sync, cudaStream_t st) {
+    constexpr int sm = (int)(sizeof(Weights) + sizeof(Tile));
+    static_assert(sm <= 227 * 1024, "one block per SM");
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
-    const float c1 = (float)(1.0 - std::pow(0.9, (double)t)), c2 = (float)(1.0 - std::pow(0.999, (double)t));
-    k_mlp_adam<<<(kParams + 255) / 256, 256, 0, st>>>(P, M, V, partial, ntiles, grad_out, adam, lr, c1, c2,
-                                                       loss_partial, loss_out);
-    return cudaGetLastError();
+    // a block per tile, and enough for one parameter per thread (57 blocks);
+    // one block per SM at most (the blocks wait for one another)
+    const int ntiles = (batch + kTile - 1) / kTile, nparam = (kParams + kMlpThreads - 1) / kMlpThreads;
+    int blocks = ntiles > nparam ? ntiles : nparam;
+    if (blocks > nsm) blocks = nsm;
+    unsigned limit = kDefaultWaitLimit;
+    void *args[] = {&P, &M, &V, &X, &T, &idx, &steps, &batch, &partial, &loss_partial, &grad_out, &adam, &lr, &corr,
+                    &loss_out, &sync, &limit};
+    count_launches(1);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_mlp_train), dim3((unsigned)blocks),
+                                       dim3(kMlpThreads), args, (size_t)sm, st);
 }
 
 // ---------------------------------------------------------------------------
 // Inference.  FP32: plain forward.  BF16: weights, inputs and hidden
 // activations rounded to bfloat16 (nearest even), products and sums in FP32.
-// One block per sample.
+// A block stages the weights once (rounding them on the way) and runs tiles
+// of 4 S samples, one hidden unit and S samples per thread; with a block and a
+// pass over the weights in global memory per sample, 256 samples took 33 us.
 // ---------------------------------------------------------------------------
-__global__ void k_mlp_to_bf16(const float *__restrict__ P, __nv_bfloat16 *__restrict__ Pb) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < kParams) Pb[p] = __float2bfloat16_rn(P[p]);
+template <int S>
+struct InferTile {
+    float x[4 * S][kP1], h1[4 * S][kPH], h2[4 * S][kPH];
+};
+
+template <bool BF16, int S>
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_infer(const float *P, const float *__restrict__ X,
+                                                              float *__restrict__ Y, long long n) {
+    extern __shared__ __align__(16) unsigned char mlp_smem[];
+    Weights &w = *reinterpret_cast<Weights *>(mlp_smem);
+    InferTile<S> &t = *reinterpret_cast<InferTile<S> *>(mlp_smem + sizeof(Weights));
+    constexpr int TS = 4 * S;
+    const int tid = threadIdx.x;
+    auto act = [](float v) { return BF16 ? __bfloat162float(__float2bfloat16_rn(v)) : v; };
+    auto same = [](float v) { return v; };
+    stage_weights(P, w);
+    stage_wait();
+    if (BF16) {
+        // round in place: every thread its share of all of it
+        __syncthreads();
+        float *all = reinterpret_cast<float *>(mlp_smem);
+        for (int e = tid; e < (int)(sizeof(Weights) / sizeof(float)); e += kMlpThreads) all[e] = act(all[e]);
+    }
+    const int j = tid & (kH - 1), s0 = S * (tid >> 7);
+    for (long long base = (long long)blockIdx.x * TS; base < n; base += (long long)gridDim.x * TS) {
+        const int nt = (int)(n - base < TS ? n - base : TS);
+        for (int e = tid; e < TS * (kIn / 4); e += kMlpThreads) {
+            const int s = e / (kIn / 4), q = e % (kIn / 4);
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (s < nt) v = __ldg(reinterpret_cast<const float4 *>(X + (size_t)(base + s) * kIn) + q);
+            *reinterpret_cast<float4 *>(&t.x[s][4 * q]) = make_float4(act(v.x), act(v.y), act(v.z), act(v.w));
+        }
+        __syncthreads();
+        {
+            float a[S];
+            const float *in[S];
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+                a[k] = w.b1[j];
+                in[k] = t.x[s0 + k];
+            }
+            dots<S>(w.W1[j], in, kIn, a, same);
+#pragma unroll
+            for (int k = 0; k < S; ++k) t.h1[s0 + k][j] = act(relu(a[k]));
+        }
+        __syncthreads();
+        {
+            float a[S];
+            const float *in[S];
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+                a[k] = w.b2[j];
+                in[k] = t.h1[s0 + k];
+            }
+            dots<S>(w.W2[j], in, kH, a, same);
+#pragma unroll
+            for (int k = 0; k < S; ++k) t.h2[s0 + k][j] = act(relu(a[k]));
+        }
+        __syncthreads();
+        for (int e = tid; e < nt * kOut; e += kMlpThreads) {
+            const int s = e / kOut, o = e % kOut;
+            float a[1] = {w.b3[o]};
+            const float *const in[1] = {t.h2[s]};
+            dots<1>(w.W3[o], in, kH, a, same);
+            Y[(size_t)base * kOut + e] = a[0];
+        }
+        __syncthreads();
+    }
 }
 
-template <bool BF16>
-__global__ void __launch_bounds__(128) k_mlp_infer(const float *__restrict__ P, const __nv_bfloat16 *__restrict__ Pb,
-                                                   const float *__restrict__ X, float *__restrict__ Y) {
-    __shared__ float h0[kIn], h1[kH], h2[kH];
-    const int s = blockIdx.x, tid = threadIdx.x;
-    auto w = [&](int i) { return BF16 ? __bfloat162float(Pb[i]) : P[i]; };
-    auto act = [&](float v) { return BF16 ? __bfloat162float(__float2bfloat16_rn(v)) : v; };
-    if (tid < kIn) h0[tid] = act(X[(size_t)s * kIn + tid]);
-    __syncthreads();
-    {
-        float a = w(oB1 + tid);
-        for (int i = 0; i < kIn; ++i) a = fmaf(w(oW1 + tid * kIn + i), h0[i], a);
-        h1[tid] = act(fmaxf(a, 0.0f));
-    }
-    __syncthreads();
-    {
-        float a = w(oB2 + tid);
-        for (int i = 0; i < kH; ++i) a = fmaf(w(oW2 + tid * kH + i), h1[i], a);
-        h2[tid] = act(fmaxf(a, 0.0f));
-    }
-    __syncthreads();
-    if (tid < kOut) {
-        float a = w(oB3 + tid);
-        for (int i = 0; i < kH; ++i) a = fmaf(w(oW3 + tid * kH + i), h2[i], a);
-        Y[(size_t)s * kOut + tid] = a;
-    }
-}
-
-cudaError_t launch_mlp_infer(const float *P, __nv_bfloat16 *Pb, const float *X, float *Y, long long n, int bf16,
-                             cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    if (bf16) {
-        count_launches(2);
-        k_mlp_to_bf16<<<(kParams + 255) / 256, 256, 0, st>>>(P, Pb);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_mlp_infer<true><<<(unsigned)n, 128, 0, st>>>(P, Pb, X, Y);
-    } else {
-        count_launches(1);
-        k_mlp_infer<false><<<(unsigned)n, 128, 0, st>>>(P, Pb, X, Y);
-    }
+template <bool BF16, int S>
+static cudaError_t launch_infer(const float *P, const float *X, float *Y, long long n, int nsm, cudaStream_t st) {
+    constexpr int sm = (int)(sizeof(Weights) + sizeof(InferTile<S>));
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_infer<BF16, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e != cudaSuccess) return e;
+    const long long tiles = (n + 4 * S - 1) / (4 * S);
+    count_launches(1);
+    k_mlp_infer<BF16, S><<<(unsigned)(tiles < nsm ? tiles : nsm), kMlpThreads, sm, st>>>(P, X, Y, n);
     return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_infer(const float *P, const float *X, float *Y, long long n, int bf16, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // one sample per thread while every tile of four has an SM of its own,
+    // else four (a weight read then serves four products)
+    const bool wide = n > 4LL * nsm;
+    if (bf16) return wide ? launch_infer<true, 4>(P, X, Y, n, nsm, st) : launch_infer<true, 1>(P, X, Y, n, nsm, st);
+    return wide ? launch_infer<false, 4>(P, X, Y, n, nsm, st) : launch_infer<false, 1>(P, X, Y, n, nsm, st);
 }
 
 }  // namespace qsg

@@ -19,9 +19,9 @@ constexpr int kMaxBatch = 4096;
 size_t up(size_t v) { return (v + kAlignM - 1) / kAlignM * kAlignM; }
 
 struct Layout {
-    float *P, *M, *V, *grad, *partial, *lossp, *losses, *X, *T, *Xp, *Yp;
-    __nv_bfloat16 *Pb;
+    float *P, *M, *V, *grad, *partial, *lossp, *losses, *corr, *X, *T, *Xp, *Yp;
     int *idx;
+    unsigned *sync;  // grid-barrier count and status of the training launch
 };
 
 size_t carve_mlp(char *base, long long n_data, int max_batch, Layout *l) {
@@ -38,10 +38,11 @@ size_t carve_mlp(char *base, long long n_data, int max_batch, Layout *l) {
     t.M = (float *)take(np * 4);
     t.V = (float *)take(np * 4);
     t.grad = (float *)take(np * 4);
-    t.Pb = (__nv_bfloat16 *)take(np * 2);
     t.partial = (float *)take(tiles * np * 4);
     t.lossp = (float *)take(tiles * 4);
     t.losses = (float *)take((size_t)kChunk * 4);
+    t.corr = (float *)take((size_t)kChunk * 2 * 4);
+    t.sync = (unsigned *)take(2 * sizeof(unsigned));
     t.idx = (int *)take((size_t)kChunk * max_batch * 4);
     t.X = (float *)take((size_t)n_data * 64 * 4);
     t.T = (float *)take((size_t)n_data * 33 * 4);
@@ -130,18 +131,27 @@ static qsg_status upload_idx(qsg_mlp *m, const int32_t *idx, size_t count) {
     return QSG_OK;
 }
 
+// Reads the status word of the last training launch (with the stream drained).
+static qsg_status finish_steps(qsg_mlp *m) {
+    unsigned status = 0;
+    MLP_CUDA(cudaMemcpyAsync(&status, m->l.sync + 1, sizeof(status), cudaMemcpyDeviceToHost, m->st));
+    MLP_CUDA(cudaStreamSynchronize(m->st));
+    return status == DEVERR_NONE ? QSG_OK : QSG_ERR_TIMEOUT;
+}
+
 qsg_status qsg_mlp_grad(qsg_mlp *m, const int32_t *idx, int32_t batch, float *loss, float *grad_host) {
     if (!m || !idx || batch < 1 || batch > m->max_batch) return QSG_ERR_ARG;
     if (!m->has_params || m->n_loaded == 0) return QSG_ERR_STATE;
     qsg_status s = upload_idx(m, idx, (size_t)batch);
     if (s != QSG_OK) return s;
-    MLP_CUDA(launch_mlp_step(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, batch, m->l.partial, m->l.lossp,
-                             m->l.grad, 0, 0.0f, 1, m->l.losses, m->st));
+    MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, 1, batch, m->l.partial, m->l.lossp,
+                              m->l.grad, 0, 0.0f, m->l.corr, m->l.losses, m->l.sync, m->st));
     if (grad_host)
         MLP_CUDA(cudaMemcpyAsync(grad_host, m->l.grad, (size_t)mlp_param_count() * 4, cudaMemcpyDeviceToHost, m->st));
     float l = 0.0f;
     MLP_CUDA(cudaMemcpyAsync(&l, m->l.losses, 4, cudaMemcpyDeviceToHost, m->st));
-    MLP_CUDA(cudaStreamSynchronize(m->st));
+    s = finish_steps(m);
+    if (s != QSG_OK) return s;
     if (loss) *loss = l;
     return QSG_OK;
 }
@@ -149,18 +159,23 @@ qsg_status qsg_mlp_grad(qsg_mlp *m, const int32_t *idx, int32_t batch, float *lo
 qsg_status qsg_mlp_train(qsg_mlp *m, const int32_t *idx, int32_t steps, int32_t batch, float lr, float *losses) {
     if (!m || !idx || steps < 0 || batch < 1 || batch > m->max_batch || !(lr > 0.0f)) return QSG_ERR_ARG;
     if (!m->has_params || m->n_loaded == 0) return QSG_ERR_STATE;
+    float corr[2 * kChunk];
     for (int c0 = 0; c0 < steps; c0 += kChunk) {
         const int nc = steps - c0 < kChunk ? steps - c0 : kChunk;
         qsg_status s = upload_idx(m, idx + (size_t)c0 * batch, (size_t)nc * batch);
         if (s != QSG_OK) return s;
         for (int i = 0; i < nc; ++i) {
             ++m->step;
-            MLP_CUDA(launch_mlp_step(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx + (size_t)i * batch, batch,
-                                     m->l.partial, m->l.lossp, nullptr, 1, lr, m->step, m->l.losses + i, m->st));
+            corr[2 * i] = (float)(1.0 - std::pow(0.9, (double)m->step));
+            corr[2 * i + 1] = (float)(1.0 - std::pow(0.999, (double)m->step));
         }
+        MLP_CUDA(cudaMemcpyAsync(m->l.corr, corr, sizeof(float) * 2 * nc, cudaMemcpyHostToDevice, m->st));
+        MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, nc, batch, m->l.partial,
+                                  m->l.lossp, nullptr, 1, lr, m->l.corr, m->l.losses, m->l.sync, m->st));
         if (losses) MLP_CUDA(cudaMemcpyAsync(losses + c0, m->l.losses, (size_t)nc * 4, cudaMemcpyDeviceToHost, m->st));
         // the index buffer is reused by the next chunk
-        MLP_CUDA(cudaStreamSynchronize(m->st));
+        s = finish_steps(m);
+        if (s != QSG_OK) return s;
     }
     return QSG_OK;
 }
@@ -169,7 +184,7 @@ qsg_status qsg_mlp_predict(qsg_mlp *m, const float *X, int64_t n, int32_t bf16, 
     if (!m || !X || !Y || n < 1 || n > m->n_data || (bf16 != 0 && bf16 != 1)) return QSG_ERR_ARG;
     if (!m->has_params) return QSG_ERR_STATE;
     MLP_CUDA(cudaMemcpyAsync(m->l.Xp, X, (size_t)n * 64 * 4, cudaMemcpyHostToDevice, m->st));
-    MLP_CUDA(launch_mlp_infer(m->l.P, m->l.Pb, m->l.Xp, m->l.Yp, n, bf16, m->st));
+    MLP_CUDA(launch_mlp_infer(m->l.P, m->l.Xp, m->l.Yp, n, bf16, m->st));
     MLP_CUDA(cudaMemcpyAsync(Y, m->l.Yp, (size_t)n * 33 * 4, cudaMemcpyDeviceToHost, m->st));
     MLP_CUDA(cudaStreamSynchronize(m->st));
     return QSG_OK;

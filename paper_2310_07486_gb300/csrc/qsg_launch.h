@@ -1,7 +1,6 @@
 // qsg_launch.h -- host-side launchers of the sm_103a kernels (internal).
 #pragma once
 #include <cstdint>
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "qsg_device.cuh"
@@ -99,14 +98,15 @@ size_t measure_scratch_words_per_pair(const Group &g);
 cudaError_t launch_features(const Group &g, float *out, cudaStream_t st);
 
 // Learned-ladder MLP (k_mlp.cu).  P: FP32 parameters, M, V: Adam moments;
-// one step = gradient of the batch idx[0..batch) (tiles of 16 samples into
-// `partial`), then Adam at step number t if adam != 0; grad_out and loss_out
-// (device) may be null.
+// `steps` steps over the batches idx[steps][batch] (tiles of 16 samples into
+// `partial`), Adam's bias corrections in corr[steps][2]; adam = 0 only writes
+// the gradient to grad_out (device, may be null).  loss_out: [steps] (device);
+// sync: two device words, the second a status (DEVERR_TIMEOUT after a bounded
+// grid wait gave up).  X, T and P are 16-byte aligned.
 int mlp_param_count();
-cudaError_t launch_mlp_step(float *P, float *M, float *V, const float *X, const float *T, const int *idx, int batch,
-                            float *partial, float *loss_partial, float *grad_out, int adam, float lr, int t,
-                            float *loss_out, cudaStream_t st);
-cudaError_t launch_mlp_infer(const float *P, __nv_bfloat16 *Pb, const float *X, float *Y, long long n, int bf16,
-                             cudaStream_t st);
+cudaError_t launch_mlp_steps(float *P, float *M, float *V, const float *X, const float *T, const int *idx, int steps,
+                             int batch, float *partial, float *loss_partial, float *grad_out, int adam, float lr,
+                             const float *corr, float *loss_out, unsigned *sync, cudaStream_t st);
+cudaError_t launch_mlp_infer(const float *P, const float *X, float *Y, long long n, int bf16, cudaStream_t st);
 
 }  // namespace qsg
