@@ -7,32 +7,46 @@
 // a dense contraction over the L^2 sites.  The spins are +-1, exact in FP8
 // E4M3, and every partial sum is an integer of magnitude <= L^2 < 2^24, so a
 // tcgen05.mma (kind::f8f6f4, FP32 accumulation in tensor memory) computes G
-// exactly.  Only the upper triangle of 128 x 128 tiles (i, j >= i) is formed
-// (G is symmetric), and every element is folded into per-lag bins: pairs with
-// offset o = t2 - t1 feed lag o when o < L_tau/2 and lag L_tau - o (the
-// forward pair from t2, which wraps, so it carries the APBC sign) when
-// o > L_tau/2; o = L_tau/2 counts twice.
+// exactly.
+//
+// Order of the work.  A 128 x 128 tile (i, e) holds the rows t1 = 128 i + m and
+// the columns t2 = 128 (i + e) + q (mod L_tau), so its element (m, q) has the
+// offset d = 128 e + q - m whatever i is.  A work unit is one sample and one
+// column offset e, or two neighbouring ones (e, e + 1), and runs over every row
+// block i: the epilogue keeps the sums of G and of G^2 over i in registers, one
+// FP32 add and one FP32 multiply-add per element straight on the accumulator
+// values (integers below 2^24, exact), and folds them into per-lag bins once
+// per unit.  With the tensor-memory loads in the 16 x 256 bit shape a thread's
+// elements lie in rows r, r + 8, r + 16, r + 24 and the same columns of every
+// octet, so elements of equal offset meet in one thread and 38 sums of each
+// kind cover its 128 elements of a tile.  (The form before this one ordered
+// the tiles by row block and folded every tile with two shared-memory atomics
+// per element: 3.92 ms for 2,048 sample bits at L = 24, L_tau = 2048, where
+// this one takes 2.57 ms.)  The wrap past L_tau is taken where the rows
+// are loaded: the row of t2 >= L_tau is that of t2 - L_tau, with its sign
+// flipped under APBC, so C needs no sign in the epilogue.
 //
 // One persistent CTA per SM, specialised warps:
-//   producers (8 warps) load the x-packed bit rows of the transposed scratch
-//     one block ahead into registers and expand them to E4M3 +-1 (0 for
-//     padding) in shared memory, K-major with the 128-byte swizzle, sites in a
-//     bit-interleaved order shared by A and B: the row block A of an item in
-//     128-site chunks, each with its own full/empty barrier pair (so the next
-//     item's A is written chunk by chunk as the last tile of the current one
-//     releases it), and B two column blocks at a time in 32 KB stages (256
-//     rows x 128 sites);
-//   one thread issues the MMAs: the diagonal tile (i, i) with N = 128 and
-//     B = A, then the column-block pairs (i, j), (i, j + 1) as one N = 256
-//     MMA per 32-site step (a single block when the count is odd), into two
-//     256-column tensor-memory accumulators, so the next tile is multiplied
-//     while the last one is folded.  Issue is nearly synchronous with the
-//     tensor pipe, so the issuing thread does nothing between MMAs but wait
-//     for a stage every four of them;
-//   the epilogue (8 warps, two per TMEM lane quadrant) folds the tiles into
-//     shared-memory lag bins and flushes them to the int64 sums.
-// The work unit is one sample's row blocks i and nb - 1 - i: nb + 1 tiles for
-// every unit, so a static round robin over the units balances the SMs.
+//   producers (8 warps, a thread per row of A or of B) load the x-packed bit
+//     rows of the transposed scratch one step ahead into registers and expand
+//     them to E4M3 in shared memory, +-1 (0 for padding) in A and +-1/2 in B (G
+//     is even, so the accumulators hold the integers G / 2 and the running sums
+//     of squares stay exact four times as long), K-major with the 128-byte
+//     swizzle, sites in a bit-interleaved order shared by A and B;
+//   one thread issues the MMAs of a step (one i) in 128-site chunks, two tiles
+//     as one N = 256 MMA per 32 sites.  In a unit of two offsets the column
+//     block i + e + 1 of one step is the block i + e of the next: it stays in
+//     shared memory (slots used in turn), so a step expands two blocks for two
+//     tiles;
+//   the epilogue (8 warps, two per TMEM lane quadrant, one per tile of the
+//     step) reads the accumulators, double-buffered in tensor memory.
+// Per step of two tiles at L = 24 the MMAs read 216 KB and the producers write 144
+// KB of shared memory (2,880 cycles at 128 B per cycle) beside 2,304 cycles of
+// tensor work; measured, a step takes 5,200: the producers' expansion (470 cycles a
+// chunk, 740 with its fences and hand-over) and the MMA thread's waits alternate
+// more than they overlap in the three chunks that fit in flight.  Lattices of L > 22..24 whose two
+// resident column blocks do not fit (more than five chunks) take every offset
+// as a unit of its own, both operands streamed.
 #include "qsg_launch.h"
 
 namespace qsg {
@@ -42,15 +56,26 @@ namespace {
 constexpr int kTile = 128;                   // rows of A (t1) and of B (t2) per tile
 constexpr int kChunk = 128;                  // sites (bytes) per K chunk = one swizzled row
 constexpr int kChunkBytes = kTile * kChunk;  // 16 KB per operand chunk
-constexpr int kMaxNc = 8;                    // 128-site chunks of a row at most (L <= 32)
-constexpr int kStageBytes = 2 * kChunkBytes; // 32 KB per B stage (two column blocks)
-constexpr int kMaxStages = 6;                // B stages at most
-constexpr int kProducers = 256;              // warps 0-7: one thread per B stage row
+constexpr int kPairNc = 5;                   // chunks up to which column blocks stay resident
+// Slots of resident column blocks: two, or more for rows of few chunks, whose
+// steps are so short that the hand-over of a stage (about 1,500 cycles from the
+// wait for it to its release) needs several steps in flight.
+__host__ __device__ constexpr int block_slots(int nc) { return nc == 1 ? 6 : (nc == 2 ? 4 : 2); }
+constexpr int kMaxStages = 6;                // chunks in flight at most
+constexpr int kProducers = 256;              // warps 0-7: threads 0-127 A rows, 128-255 B rows
 constexpr int kProducerWarps = kProducers / 32;
 constexpr int kEpilogueWarps = 8;
-constexpr int kEpilogue = 256;               // warps 8-15: two per TMEM lane quadrant
+constexpr int kEpilogue = 256;               // warps 8-15: quadrant = warp & 3, tile = (warp >> 2) & 1
 constexpr int kMmaWarp = 16;
 constexpr int kThreads = 17 * 32;
+// registers: 17 warps put five on one scheduler, so the launch gets 96 a
+// thread; the epilogue's 76 running sums and 32 loaded values want more, which
+// the producers give up (256 x 80 + 256 x 112 + 32 x 96 = 544 x 96)
+constexpr int kLaunchRegs = 96, kProducerRegs = 80, kEpilogueRegs = 112;
+static_assert(kProducers * kProducerRegs + kEpilogue * kEpilogueRegs + 32 * kLaunchRegs == kThreads * kLaunchRegs,
+              "register shares");
+constexpr int kBins = 384;                   // lags of a unit: 128 e - 127 .. 128 e + 255
+constexpr int kOct = kTile / 8 + 3;          // distinct octet offsets of a thread's elements
 constexpr unsigned kSpinLimit = 1u << 22;    // polls of the wait for issued MMAs before TMEM is freed
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -72,10 +97,9 @@ __device__ __forceinline__ uint32_t idesc_e4m3(int n) {
 }
 
 struct Ctl {
-    uint64_t bfull[kMaxStages], bempty[kMaxStages];  // B stage written / multiplied
-    uint64_t afull[kMaxNc], aempty[kMaxNc];          // A chunk written / multiplied
-    uint64_t accfull[2], accempty[2];                // accumulator computed / folded
-    uint64_t done;                                   // every MMA of the CTA completed
+    uint64_t full[kMaxStages], empty[kMaxStages];  // chunk written / multiplied
+    uint64_t accfull[2], accempty[2];              // accumulator computed / read
+    uint64_t done;                                 // every MMA of the CTA completed
     uint32_t tmem;
     int abort;  // a wait gave up: every role skips its work and runs out its loops
 };
@@ -108,12 +132,14 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
                  : "memory");
 }
 
-// 32 spin bits -> 32 E4M3 bytes (+1 = 0x38, -1 = 0xB8; a set bit is spin -1)
-// in the site order of the contraction: byte k of output word j is bit
-// 8k + j.  The Gram sums over sites, so any order serves that A and B share;
-// this one takes one shift and one mask per output word.
-__device__ __forceinline__ uint32_t spread_e4m3(uint32_t b, int j) {
-    return ((b << (7 - j)) & 0x80808080u) | 0x38383838u;
+// 32 spin bits -> 32 E4M3 bytes (`one` = four bytes of the magnitude; a set bit
+// is spin -1, the sign bit) in the site order of the contraction: byte k of
+// output word j is bit 8k + j.  The Gram sums over sites, so any order serves
+// that A and B share; this one takes one shift and one mask per output word.
+// The shift is a multiplication by unit << (7 - j), unit = 1 unknown to the
+// compiler: the multiplier's pipe is idle here and the integer one is not.
+__device__ __forceinline__ uint32_t spread_e4m3(uint32_t b, int j, uint32_t one, uint32_t unit) {
+    return ((b * (unit << (7 - j))) & 0x80808080u) | one;
 }
 
 // Bytes of spread_e4m3's output word j whose bits are set in the site mask vm
@@ -126,7 +152,7 @@ __device__ __forceinline__ uint32_t spread_mask(uint32_t vm, int j) {
 // 128-byte row `row` at rowp; sites >= valid (outside the lattice, or every
 // site of a row past L_tau) become 0.  Output words 8 e + j (e = half of the
 // word) fill granules 4 hh + 2 e + (j >> 2).
-__device__ __forceinline__ void expand_full(uint8_t *rowp, uint64_t wv, int hh, int row) {
+__device__ __forceinline__ void expand_full(uint8_t *rowp, uint64_t wv, int hh, int row, uint32_t one, uint32_t unit) {
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         const uint32_t b = (uint32_t)(wv >> (32 * e));
@@ -134,13 +160,13 @@ __device__ __forceinline__ void expand_full(uint8_t *rowp, uint64_t wv, int hh, 
         for (int hq = 0; hq < 2; ++hq) {
             const int gr = 4 * hh + 2 * e + hq;
             *reinterpret_cast<uint4 *>(rowp + ((gr ^ (row & 7)) << 4)) =
-                make_uint4(spread_e4m3(b, 4 * hq), spread_e4m3(b, 4 * hq + 1), spread_e4m3(b, 4 * hq + 2),
-                           spread_e4m3(b, 4 * hq + 3));
+                make_uint4(spread_e4m3(b, 4 * hq, one, unit), spread_e4m3(b, 4 * hq + 1, one, unit),
+                           spread_e4m3(b, 4 * hq + 2, one, unit), spread_e4m3(b, 4 * hq + 3, one, unit));
         }
     }
 }
 
-__device__ __noinline__ void expand_part(uint8_t *rowp, uint64_t wv, int valid, int hh, int row) {
+__device__ __noinline__ void expand_part(uint8_t *rowp, uint64_t wv, int valid, int hh, int row, uint32_t one) {
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         const uint32_t b = (uint32_t)(wv >> (32 * e));
@@ -151,26 +177,19 @@ __device__ __noinline__ void expand_part(uint8_t *rowp, uint64_t wv, int valid, 
             const int gr = 4 * hh + 2 * e + hq;
             uint32_t o[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) o[k] = spread_e4m3(b, 4 * hq + k) & spread_mask(vm, 4 * hq + k);
+            for (int k = 0; k < 4; ++k) o[k] = spread_e4m3(b, 4 * hq + k, one, 1u) & spread_mask(vm, 4 * hq + k);
             *reinterpret_cast<uint4 *>(rowp + ((gr ^ (row & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
 }
 
-__device__ __forceinline__ void expand_word(uint8_t *rowp, uint64_t wv, int valid, int hh, int row) {
+__device__ __forceinline__ void expand_word(uint8_t *rowp, uint64_t wv, int valid, int hh, int row, uint32_t one,
+                                            uint32_t unit) {
     if (valid >= 64)
-        expand_full(rowp, wv, hh, row);
+        expand_full(rowp, wv, hh, row, one, unit);
     else
-        expand_part(rowp, wv, valid, hh, row);
+        expand_part(rowp, wv, valid, hh, row, one);
 }
-
-// FP32 accumulator holding an integer |x| < 2^22 -> int32 with one add: in
-// [2^23, 2^24) the FP32 spacing is 1, so x + 1.5 * 2^23 is exact and its bit
-// pattern is that of 1.5 * 2^23 plus x.
-__device__ __forceinline__ int exact_f32_to_int(uint32_t bits) {
-    return __float_as_int(__uint_as_float(bits) + 12582912.0f) - 0x4B400000;
-}
-
 
 __device__ __forceinline__ void mma_f8(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
     asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
@@ -178,149 +197,130 @@ __device__ __forceinline__ void mma_f8(uint32_t d, uint64_t da, uint64_t db, uin
                  "l"(da), "l"(db), "r"(idesc), "r"(acc));
 }
 
-// The work of one CTA: units u = blockIdx.x + n gridDim.x; unit u is sample
-// u / nhalf, row blocks h = u % nhalf and nb - 1 - h (one block when equal).
-// Within a unit the blocks are items; item i has the diagonal tile (i, i) and
-// the column-block pairs (i, jp), (i, jp + 1), jp = i + 1, i + 3, ...
-__device__ __forceinline__ int item_block(int h, int item, int nb) { return item ? nb - 1 - h : h; }
-__device__ __forceinline__ int unit_items(int h, int nb) { return nb - 1 - h != h ? 2 : 1; }
-
-// The producers' block sequence: per item the A block i, then the pairs.
-struct Seq {
-    int u, sidx, h, item, i, jp;
-    bool isA, valid;
+// How the offsets of one sample are cut into units and steps.
+struct GramPlan {
+    int nsamples;
+    int nb;       // row blocks
+    int npair;    // units of two offsets per sample: e = 0, 2, ..
+    int nsingle;  // units of one offset per sample, the first of them e = e_single
+    int e_single;
+    int e_mirror;  // offset whose steps stop at nb / 2 (each tile is the transpose of another), or -1
+    int nstages;
+    int flush;     // steps after which the FP32 sums must be folded
+    uint32_t unit;  // 1 (see spread_e4m3)
 };
 
-__device__ __forceinline__ void seq_unit(Seq &c, int nunits, int nhalf) {
-    c.valid = c.u < nunits;
-    c.sidx = c.u / nhalf;
-    c.h = c.u - c.sidx * nhalf;
-    c.item = 0;
-    c.i = c.h;
-    c.isA = true;
-    c.jp = c.h;
-}
+struct Unit {
+    int sample, e, steps;
+    bool pair, mirror;
+};
 
-__device__ __forceinline__ void seq_next(Seq &c, int nunits, int nhalf, int nb) {
-    if (c.isA) {
-        c.isA = false;
-        c.jp = c.i + 1;
-        if (c.jp < nb) return;
+// Units of two offsets of every sample first (a sample's units on neighbouring
+// SMs at the same time, so that they share its rows in L2), then the others;
+// a static round robin over each kind keeps the SMs balanced.
+__device__ __forceinline__ Unit unit_of(const GramPlan &pl, int u) {
+    Unit r;
+    const int np = pl.nsamples * pl.npair;
+    r.pair = u < np;
+    if (r.pair) {
+        r.sample = u / pl.npair;
+        r.e = 2 * (u - r.sample * pl.npair);
+        r.mirror = false;
     } else {
-        c.jp += 2;
-        if (c.jp < nb) return;
+        r.sample = (u - np) / pl.nsingle;
+        r.e = pl.e_single + (u - np) - r.sample * pl.nsingle;
+        r.mirror = r.e == pl.e_mirror;
     }
-    if (++c.item >= unit_items(c.h, nb)) {
-        c.u += gridDim.x;
-        seq_unit(c, nunits, nhalf);
-        return;
-    }
-    c.i = item_block(c.h, c.item, nb);
-    c.isA = true;
-    c.jp = c.i;
+    r.steps = r.mirror ? pl.nb / 2 : pl.nb;
+    return r;
+}
+__device__ __forceinline__ int unit_count(const GramPlan &pl) { return pl.nsamples * (pl.npair + pl.nsingle); }
+
+// The steps a CTA runs, in order: of every unit the steps 0 .. steps - 1, before
+// them (i = -1) the load of the first column block in a unit of two offsets.
+struct Cursor {
+    int u, i;
+    bool valid;
+    Unit un;
+};
+__device__ __forceinline__ void cursor_unit(const GramPlan &pl, Cursor &c) {
+    c.valid = c.u < unit_count(pl);
+    if (!c.valid) return;
+    c.un = unit_of(pl, c.u);
+    c.i = c.un.pair ? -1 : 0;
+}
+__device__ __forceinline__ void cursor_next(const GramPlan &pl, Cursor &c) {
+    if (!c.valid || ++c.i < c.un.steps) return;
+    c.u += gridDim.x;
+    cursor_unit(pl, c);
 }
 
-// Bit words of producer thread pt for block c, 0 outside the lattice and past
-// L_tau.  A block: w[kc] = word 2 kc + (pt >> 7) of row (pt & 127) of block
-// i.  Pair: w[2 kc + hh] = word 2 kc + hh of stage row pt (rows 0..127 are
-// block jp, rows 128..255 block jp + 1).
-template <int NC>
-__device__ __forceinline__ void load_seq(const Seq &c, const uint64_t *__restrict__ P, int Lt, int nwx, int pt,
-                                         uint64_t (&w)[2 * NC]) {
-    const size_t sbase = (size_t)(c.valid ? c.sidx : 0) * Lt;
-    if (c.isA) {
-        const int row = pt & 127, hh = pt >> 7;
-        const int t = c.i * kTile + row;
-        const bool in = c.valid && t < Lt;
-        const uint64_t *src = P + (sbase + (in ? t : 0)) * nwx + hh;
-#pragma unroll
-        for (int kc = 0; kc < NC; ++kc) w[kc] = (in && 2 * kc + hh < nwx) ? __ldg(src + 2 * kc) : 0ull;
-    } else {
-        const int t = (c.jp + (pt >> 7)) * kTile + (pt & 127);
-        const bool in = c.valid && t < Lt;
-        const uint64_t *src = P + (sbase + (in ? t : 0)) * nwx;
-#pragma unroll
-        for (int kc = 0; kc < NC; ++kc)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh)
-                w[2 * kc + hh] = (in && 2 * kc + hh < nwx) ? __ldg(src + 2 * kc + hh) : 0ull;
+// Source row of a producer thread at a step: row `row` of the A block
+// (t1 = 128 i + row) or of the column block the step brings in (t2 =
+// 128 (i + e [+ 1]) + row, wrapped).
+struct Row {
+    const uint64_t *src;
+    uint64_t flip;  // all ones where B's row wraps under APBC
+    bool live;      // B, or an A row that exists (t1 < L_tau)
+};
+__device__ __forceinline__ Row row_of(const Cursor &c, const uint64_t *__restrict__ P, int Lt, int nwx, int apbc,
+                                      bool isB, int row) {
+    Row r;
+    int t = c.valid ? kTile * (c.i + (isB ? c.un.e + (c.un.pair ? 1 : 0) : 0)) + row : 0;
+    r.flip = 0ull;
+    r.live = true;
+    if (isB) {
+        if (t >= Lt) {
+            t = t < 2 * Lt ? t - Lt : t % Lt;  // beyond 2 L_tau: no lag of this row is used
+            if (apbc) r.flip = ~0ull;
+        }
+    } else if (c.i < 0 || t >= Lt) {
+        r.live = false;
+        t = 0;
     }
+    r.src = P + ((size_t)(c.valid ? c.un.sample : 0) * Lt + t) * nwx;
+    return r;
+}
+// 64 accumulator columns of 16 TMEM lanes: octet o of the columns is v[4 o ..
+// 4 o + 3] = (row r, columns 2 c, 2 c + 1), (row r + 8, the same), with r =
+// lane / 4 and c = lane % 4
+__device__ __forceinline__ void tmem_ld_oct8(uint32_t taddr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
 }
 
-// Fold the 64 columns cbase .. cbase + 63 of row m of tile (i, jb) into the
-// lag bins.  Most tiles map every element to lag o (all o < L_tau/2) or to
-// lag L_tau - o (all o > L_tau/2); only the tiles around L_tau/2 and those
-// past L_tau need the per-element choice.
-__device__ __forceinline__ void fold_slice(const uint32_t (&v)[64], int i, int jb, int m, int cbase, int Lt, int half,
-                                           int boundary, int *binC, unsigned *binQ) {
-    const int whigh = boundary == 1 ? -1 : 1;
-    const int t1 = i * kTile + m;
-    const int obase = (jb - i) * kTile;
-    const int omin = jb == i ? 1 : obase - (kTile - 1), omax = obase + kTile - 1;
-    const bool full = (jb + 1) * kTile <= Lt && (i + 1) * kTile <= Lt;
-    const int cls = (omax < half) ? 0 : (omin > half ? 1 : 2);
-    const int o0 = obase + cbase - m;  // offset of column q is o0 + q
-    if (full && cls == 0 && jb != i) {
-        int *bc = binC + o0;
-        unsigned *bq = binQ + o0;
+// Shift the sums v[0 .. N) of a warp one level down a tree over its lanes: add to
+// every lane the sums `from` of lane `src`, whose elements lie at offsets 8 higher
+// where that lane's row wrapped (then its sum k belongs to k + 1).  v[N] is new.
+template <int N, class T>
+__device__ __forceinline__ void fold_level(T (&v)[22], const T (&from)[22], bool wraps, int src) {
 #pragma unroll
-        for (int q = 0; q < 64; ++q) {
-            const int gv = exact_f32_to_int(v[q]);
-            atomicAdd(bc + q, gv);
-            atomicAdd(bq + q, (unsigned)(gv * gv));
-        }
-    } else if (full && cls == 1) {
-        // the wrapped forward pair: lag L_tau - o0 - q (APBC: C takes the minus sign)
-        int *bc = binC + (Lt - o0);
-        unsigned *bq = binQ + (Lt - o0);
-        if (whigh == 1) {
-#pragma unroll
-            for (int q = 0; q < 64; ++q) {
-                const int gv = exact_f32_to_int(v[q]);
-                atomicAdd(bc - q, gv);
-                atomicAdd(bq - q, (unsigned)(gv * gv));
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 64; ++q) {
-                const int gv = exact_f32_to_int(v[q]);
-                atomicAdd(bc - q, -gv);
-                atomicAdd(bq - q, (unsigned)(gv * gv));
-            }
-        }
-    } else if (t1 < Lt) {
-#pragma unroll
-        for (int q = 0; q < 64; ++q) {
-            const int t2 = jb * kTile + cbase + q;
-            const int o = o0 + q;
-            if (t2 < Lt && o > 0) {
-                const int gv = exact_f32_to_int(v[q]);
-                int lag, wc, wq;
-                if (o < half) {
-                    lag = o; wc = 1; wq = 1;
-                } else if (o == half) {
-                    lag = half; wc = boundary == 1 ? 0 : 2; wq = 2;
-                } else {
-                    lag = Lt - o; wc = whigh; wq = 1;
-                }
-                atomicAdd(&binC[lag], wc * gv);
-                atomicAdd(&binQ[lag], (unsigned)(wq * gv * gv));
-            }
-        }
+    for (int k = N; k >= 0; --k) {
+        const T same = k < N ? from[k < N ? k : 0] : T(0), lower = k > 0 ? from[k > 0 ? k - 1 : 0] : T(0);
+        v[k] = (k < N ? v[k] : T(0)) + __shfl_sync(0xffffffffu, wraps ? lower : same, src);
     }
 }
 
-// 64 consecutive accumulator columns of the warp's 32 lanes
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&v)[64]) {
-#pragma unroll
-    for (int c = 0; c < 64; c += 16)
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-            : "=r"(v[c + 0]), "=r"(v[c + 1]), "=r"(v[c + 2]), "=r"(v[c + 3]), "=r"(v[c + 4]), "=r"(v[c + 5]),
-              "=r"(v[c + 6]), "=r"(v[c + 7]), "=r"(v[c + 8]), "=r"(v[c + 9]), "=r"(v[c + 10]), "=r"(v[c + 11]),
-              "=r"(v[c + 12]), "=r"(v[c + 13]), "=r"(v[c + 14]), "=r"(v[c + 15])
-            : "r"(taddr + (uint32_t)c));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+// The warp's sums of one kind, v[kappa] of column 2 c and w[kappa] of column 2 c + 1
+// of every lane (row r = lane / 4, c = lane % 4), element offset 8 kappa + 2 c + q -
+// r, summed over lanes of equal offset: lane 4 r then holds in v[k] the sum of offset
+// 8 k - r.
+template <class T>
+__device__ __forceinline__ void fold_lanes(T (&v)[22], const T (&w)[22], int lane) {
+    static_assert(kOct == 19, "levels of 19, 20 and 21 sums");
+    const int r = lane >> 2, c = lane & 3;
+    fold_level<19>(v, w, r < 1, (((r + 1) & 7) << 2) | c);              // q = 1 into q = 0
+    fold_level<20>(v, v, r < 2, (((r + 2) & 7) << 2) | ((c + 1) & 3));  // c odd into c even
+    fold_level<21>(v, v, r < 4, (((r + 4) & 7) << 2) | ((c + 2) & 3));  // c = 2 into c = 0
 }
 
 }  // namespace
@@ -329,28 +329,24 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&v)[64]) {
 // NC = 128-site chunks of a row (L^2 / 128 rounded up).
 template <int NC>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_gram_tc(Group g, int p0, const uint64_t *__restrict__ P, int nsamples, int nstages, int *status,
-              unsigned wait_limit) {
+    k_gram_tc(Group g, int p0, const uint64_t *__restrict__ P, const GramPlan pl, int *status, unsigned wait_limit) {
+    constexpr bool RESIDENT = NC <= kPairNc;  // column blocks in resident slots, else streamed with A
+    constexpr int NS = block_slots(NC);
     extern __shared__ __align__(16) uint8_t dyn_raw[];
     uint8_t *dyn = dyn_raw + ((1024u - (smem_u32(dyn_raw) & 1023u)) & 1023u);
     __shared__ Ctl ctl;
+    __shared__ int binC[kBins];
+    __shared__ unsigned binQ[kBins];
     const int Lt = g.Ltau, L2 = g.L * g.L, half = Lt / 2, nl = g.nlag, nwx = g.nwx;
-    const int nb = (Lt + kTile - 1) / kTile, nhalf = (nb + 1) / 2;
-    const int nunits = nsamples * nhalf;
-    uint8_t *sA = dyn;                            // NC chunks of 128 rows x 128 sites
-    uint8_t *sB = sA + (size_t)NC * kChunkBytes;  // stages of 256 rows x 128 sites
-    int *binC = reinterpret_cast<int *>(sB + (size_t)nstages * kStageBytes);
-    unsigned *binQ = reinterpret_cast<unsigned *>(binC + nl);
+    const int nunits = unit_count(pl), nst = pl.nstages;
+    uint8_t *sA = dyn;                               // nst chunks of 128 rows x 128 sites
+    uint8_t *sB = sA + (size_t)nst * kChunkBytes;  // RESIDENT: [chunk][slot], else nst chunks
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         for (int s = 0; s < kMaxStages; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&ctl.bfull[s])), "r"(kProducerWarps));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&ctl.bempty[s])));
-        }
-        for (int k = 0; k < kMaxNc; ++k) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&ctl.afull[k])), "r"(kProducerWarps));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&ctl.aempty[k])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&ctl.full[s])), "r"(kProducerWarps));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&ctl.empty[s])));
         }
         for (int a = 0; a < 2; ++a) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&ctl.accfull[a])));
@@ -364,7 +360,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_u32(&ctl.tmem)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
-    for (int l = tid; l < nl; l += kThreads) {
+    for (int l = tid; l < kBins; l += kThreads) {
         binC[l] = 0;
         binQ[l] = 0u;
     }
@@ -375,132 +371,195 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp < kProducerWarps) {
         // ------------------------------------------------------------ producers
-        // the bit words of the next block are loaded into registers while the
-        // current one is expanded; one chunk loop serves both kinds of block:
-        // an A block's thread writes word tid >> 7 of row tid & 127, a pair
-        // block's thread both words of stage row tid (none past a single
-        // last block)
-        Seq cur, nxt;
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kProducerRegs));
+        const bool isB = tid >= kTile;
+        const int row = tid & (kTile - 1);
+        Cursor cur, ahead;
         cur.u = blockIdx.x;
-        seq_unit(cur, nunits, nhalf);
-        uint64_t wc[2 * NC], wn[2 * NC];
-        load_seq<NC>(cur, P, Lt, nwx, tid, wc);
-        // the first use of a buffer waits for the phase before the first
+        cursor_unit(pl, cur);
+        ahead = cur;
+        Row now = row_of(cur, P, Lt, nwx, g.boundary, isB, row);
+        uint64_t w[2 * NC];
+#pragma unroll
+        for (int k = 0; k < 2 * NC; ++k) w[k] = k < nwx ? __ldg(now.src + k) : 0ull;
+        const uint32_t one = isB ? 0x30303030u : 0x38383838u, unit = pl.unit;
+        // the first use of a stage waits for the phase before the first
         // (complete at initialisation)
-        uint32_t a_ph = 1u, b_par = 1u;
-        int s = 0;
+        uint32_t par = 1u;
+        int st = 0, slot = 0;  // slot: of the column block a step brings in, in turn over all steps
         while (cur.valid) {
-            nxt = cur;
-            seq_next(nxt, nunits, nhalf, nb);
-            load_seq<NC>(nxt, P, Lt, nwx, tid, wn);
-            const bool isA = cur.isA;
-            const bool pair = cur.jp + 1 < nb;
-            const int row = isA ? (tid & 127) : tid, hh0 = isA ? (tid >> 7) : 0;
-            const int nw = isA ? 1 : ((pair || tid < kTile) ? 2 : 0);
-            const int t = isA ? cur.i * kTile + row : (cur.jp + (tid >> 7)) * kTile + (tid & 127);
-            // the chunk loop stays rolled (the three roles' code shares the
-            // instruction cache): the words of chunk kc are always in wc[0],
-            // wc[1] (an A block's in wc[0]), and the array shifts after a chunk
-#pragma unroll 1
+            cursor_next(pl, ahead);
+            const Row next = row_of(ahead, P, Lt, nwx, g.boundary, isB, row);
+            const bool write = isB || cur.i >= 0;  // no A block before the first step
+            const uint64_t flip = now.flip;
+            // unrolled, so that a chunk's words are replaced by those of the
+            // next step as soon as they are used: the loads have a whole step
+            // to land and need no registers of their own (in a rolled loop
+            // they were waited for before its first pass, 1,900 cycles a step)
+#pragma unroll
             for (int kc = 0; kc < NC; ++kc) {
-                const bool ok = isA ? mbar_wait(&ctl.aempty[kc], a_ph, &ctl.abort, wait_limit)
-                                    : mbar_wait(&ctl.bempty[s], b_par, &ctl.abort, wait_limit);
-                uint8_t *rowp = isA ? sA + (size_t)kc * kChunkBytes + row * kChunk
-                                    : sB + (size_t)s * kStageBytes + row * kChunk;
-                const uint64_t w0 = wc[0], w1 = wc[1];
-                if (ok) {
-#pragma unroll 1
-                    for (int k = 0; k < nw; ++k) {
-                        const int hh = hh0 + k;
-                        // a word past the lattice's last site is never read (the
-                        // MMAs of the last chunk stop at its last word with a site)
-                        if (L2 - kc * kChunk - 64 * hh > 0)
-                            expand_word(rowp, k ? w1 : w0, t < Lt ? L2 - kc * kChunk - 64 * hh : 0, hh, row);
-                    }
+                const bool ok = mbar_wait(&ctl.empty[st], par, &ctl.abort, wait_limit);
+                uint8_t *rowp = (!isB ? sA + (size_t)st * kChunkBytes
+                                      : (RESIDENT ? sB + (size_t)(NS * kc + slot) * kChunkBytes
+                                                  : sB + (size_t)st * kChunkBytes)) +
+                                row * kChunk;
+                if (ok && write) {
+                    // a word past the lattice's last site is never read (the
+                    // MMAs of the last chunk stop at its last word with a
+                    // site); zeros in A alone blank the sites past L^2 and
+                    // the rows past L_tau
+                    const int left = L2 - kc * kChunk;
+                    const int valid = isB ? kChunk : (now.live ? left : 0);
+                    expand_word(rowp, w[2 * kc] ^ flip, valid, 0, row, one, unit);
+                    if (left > 64) expand_word(rowp, w[2 * kc + 1] ^ flip, valid - 64, 1, row, one, unit);
                 }
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 __syncwarp();  // the warp's rows are written: one arrival per warp
-                if (lane == 0) mbar_arrive(isA ? &ctl.afull[kc] : &ctl.bfull[s]);
-                if (!isA && ++s == nstages) {
-                    s = 0;
-                    b_par ^= 1u;
+                if (lane == 0) mbar_arrive(&ctl.full[st]);
+                if (++st == nst) {
+                    st = 0;
+                    par ^= 1u;
                 }
-                const int sh = isA ? 1 : 2;  // words per chunk of this kind of block
-#pragma unroll
-                for (int k = 0; k < 2 * NC - 2; ++k) wc[k] = sh == 1 ? wc[k + 1] : wc[k + 2];
+                w[2 * kc] = __ldg(next.src + 2 * kc);
+                if (2 * kc + 1 < nwx) w[2 * kc + 1] = __ldg(next.src + 2 * kc + 1);
             }
-            if (isA) a_ph ^= 1u;
-#pragma unroll
-            for (int k = 0; k < 2 * NC; ++k) wc[k] = wn[k];
-            cur = nxt;
+            now = next;
+            cur = ahead;
+            if (++slot == NS) slot = 0;
         }
     } else if (warp < kMmaWarp) {
         // ------------------------------------------------------------- epilogue
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kEpilogueRegs));
         const int etid = tid - kProducers;
-        const int quad = warp & 3;                                  // TMEM lanes 32 quad .. 32 quad + 31
-        const int cbase = ((warp - kProducerWarps) >> 2) * 64;     // column half of a 128-column tile
-        const int m = quad * 32 + lane;                             // tile row
+        const int quad = warp & 3;                       // TMEM lanes 32 quad .. 32 quad + 31
+        const int half_w = (warp >> 2) & 1;              // of two tiles of a step, or of two steps
+        const int r = lane >> 2;                         // the thread's row of an octet pair
         uint32_t n_t = 0;
+        int parity = 0;  // of the step, the loads of a unit's first column block counted
         for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-            const int sidx = u / nhalf, h = u % nhalf;
-            for (int item = 0; item < unit_items(h, nb); ++item) {
-                const int i = item_block(h, item, nb);
-                // the MMA's tile order: (i, i), then the pairs from jp = i + 1
-                for (int jp = i; jp < nb; jp = (jp == i ? i + 1 : jp + 2), ++n_t) {
-                    const int nsub = (jp != i && jp + 1 < nb) ? 2 : 1;
-                    const int a = (int)(n_t & 1u);
-                    // warp-uniform: the tensor-memory loads below are .sync.aligned
-                    const bool ok =
-                        __all_sync(0xFFFFFFFFu, mbar_wait(&ctl.accfull[a], (n_t >> 1) & 1u, &ctl.abort, wait_limit));
-                    asm volatile("tcgen05.fence::after_thread_sync;\n");
-                    if (ok) {
-                        for (int sub = 0; sub < nsub; ++sub) {
-                            uint32_t v[64];
-                            tmem_ld64(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(a * 256 + sub * kTile + cbase),
-                                      v);
-                            if (sub == nsub - 1) {
-                                // the accumulator is free for the tile after next
-                                asm volatile("tcgen05.fence::before_thread_sync;\n");
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(&ctl.accempty[a]);
-                            }
-                            fold_slice(v, i, jp + sub, m, cbase, Lt, half, g.boundary, binC, binQ);
+            const Unit un = unit_of(pl, u);
+            if (un.pair) parity ^= 1;
+            const int e = un.pair ? un.e + half_w : un.e;
+            const int lag0 = max(0, kTile * un.e - (kTile - 1));  // lag of bin 0
+            const int sb = un.sample / 64, bit = un.sample % 64;
+            const int pb = sb / g.R, rr = sb % g.R;
+            const int pidx = p0 + pb, w = pidx / g.K, j = pidx % g.K;
+            const size_t gbase = ((((size_t)rr * g.W * 64) + (size_t)w * 64 + bit) * g.K + j) * nl;
+            float accC[kOct][2], accQ[kOct][2];
+#pragma unroll
+            for (int k = 0; k < kOct; ++k) accC[k][0] = accC[k][1] = accQ[k][0] = accQ[k][1] = 0.0f;
+            int in_flush = 0, in_push = 0;
+            for (int i = 0; i < un.steps; ++i, ++n_t, parity ^= 1) {
+                const int a = (int)(n_t & 1u);
+                // warp-uniform: the tensor-memory loads below are .sync.aligned
+                const bool ok =
+                    __all_sync(0xFFFFFFFFu, mbar_wait(&ctl.accfull[a], (n_t >> 1) & 1u, &ctl.abort, wait_limit));
+                asm volatile("tcgen05.fence::after_thread_sync;\n");
+                // the tile of this warp: the columns of the slot that holds its
+                // offset (two offsets), or every second step (one offset)
+                const bool mine = un.pair || (i & 1) == half_w;
+                // (of two slots, the step's new block, offset e + 1, is in slot `parity`)
+                const int slot = !un.pair ? 0 : (NS == 2 ? (half_w ? parity : parity ^ 1) : half_w);
+                if (ok && mine) {
+                    const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(a * 256 + slot * kTile);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int kg = 0; kg < 2; ++kg) {
+                            uint32_t v[32];
+                            tmem_ld_oct8(ta + ((uint32_t)(h * 16) << 16) + (uint32_t)(kg * 64), v);
+#pragma unroll
+                            for (int o = 0; o < 8; ++o)
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    const int k = kg * 8 + o - (2 * h + (q >> 1)) + 3;
+                                    const float x = __uint_as_float(v[4 * o + q]);
+                                    accC[k][q & 1] += x;
+                                    accQ[k][q & 1] = fmaf(x, x, accQ[k][q & 1]);
+                                }
                         }
-                    } else {
-                        asm volatile("tcgen05.fence::before_thread_sync;\n");
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&ctl.accempty[a]);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;\n");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl.accempty[a]);
+                // fold the sums before they could leave FP32's exact integers,
+                // and add the 32-bit bins to the int64 sums before they wrap
+                const bool last = i + 1 == un.steps;
+                if (++in_flush == pl.flush || last) {
+                    in_flush = 0;
+                    // sums of G over lanes stay exact in FP32 (magnitudes
+                    // below 2^24), those of squares need integers
+                    const int dbase = kTile * e - 32 * quad - 24 - r;
+                    const bool owner = (lane & 3) == 0;
+                    {
+                        float v[22], w[22];
+#pragma unroll
+                        for (int k = 0; k < 22; ++k) {
+                            v[k] = k < kOct ? accC[k < kOct ? k : 0][0] : 0.0f;
+                            w[k] = k < kOct ? accC[k < kOct ? k : 0][1] : 0.0f;
+                        }
+                        fold_lanes(v, w, lane);
+#pragma unroll
+                        for (int k = 0; k < 22; ++k) {
+                            const int d = dbase + 8 * k;
+                            int cv = __float2int_rn(v[k]), lag = d;
+                            if (un.mirror && d >= half) {
+                                // half the row blocks: an element past L_tau / 2 is
+                                // the wrapped pair of lag L_tau - d, and one at
+                                // L_tau / 2 stands for both directions
+                                lag = Lt - d;
+                                cv = d == half ? (g.boundary == 1 ? 0 : 2 * cv) : (g.boundary == 1 ? -cv : cv);
+                            }
+                            if (owner && d >= 0 && lag >= lag0 && lag <= half) atomicAdd(&binC[lag - lag0], cv);
+                        }
+                    }
+                    {
+                        int v[22], w[22];
+#pragma unroll
+                        for (int k = 0; k < 22; ++k) {
+                            v[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][0]) : 0;
+                            w[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][1]) : 0;
+                        }
+                        fold_lanes(v, w, lane);
+#pragma unroll
+                        for (int k = 0; k < 22; ++k) {
+                            const int d = dbase + 8 * k;
+                            unsigned qv = (unsigned)v[k];
+                            int lag = d;
+                            if (un.mirror && d >= half) {
+                                lag = Lt - d;
+                                if (d == half) qv *= 2u;
+                            }
+                            if (owner && d >= 0 && lag >= lag0 && lag <= half) atomicAdd(&binQ[lag - lag0], qv);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < kOct; ++k) accC[k][0] = accC[k][1] = accQ[k][0] = accQ[k][1] = 0.0f;
+                    if (++in_push == 2 || last) {
+                        in_push = 0;
+                        asm volatile("bar.sync 1, %0;\n" ::"n"(kEpilogue) : "memory");
+                        const bool write = !*(volatile int *)&ctl.abort;
+                        for (int l = etid; l < kBins; l += kEpilogue) {
+                            // sums of G / 2 and of its square
+                            const long long cs = 2LL * binC[l];
+                            const unsigned long long qs = 4ull * binQ[l];
+                            if (write && cs)
+                                atomicAdd(reinterpret_cast<unsigned long long *>(&g.Cacc[gbase + lag0 + l]),
+                                          (unsigned long long)cs);
+                            if (write && qs)
+                                atomicAdd(reinterpret_cast<unsigned long long *>(&g.Qacc[gbase + lag0 + l]), qs);
+                            binC[l] = 0;
+                            binQ[l] = 0u;
+                        }
+                        asm volatile("bar.sync 1, %0;\n" ::"n"(kEpilogue) : "memory");
                     }
                 }
             }
-            // the unit's bins are complete: add them to the sample's int64 sums;
-            // a CTA's t1 span two row blocks, so a bin holds at most 2 x 256
-            // products G^2 <= 2^20 (L <= 32): 2^29, exact in 32 bits
-            asm volatile("bar.sync 1, %0;\n" ::"n"(kEpilogue) : "memory");
-            const int sb = sidx / 64, bit = sidx % 64;
-            const int pb = sb / g.R, r = sb % g.R;
-            const int pidx = p0 + pb, w = pidx / g.K, j = pidx % g.K;
-            const size_t gbase = ((((size_t)r * g.W * 64) + (size_t)w * 64 + bit) * g.K + j) * nl;
-            const bool write = !*(volatile int *)&ctl.abort;
-            for (int l = etid; l < nl; l += kEpilogue) {
-                long long c = binC[l];
-                unsigned long long qv = binQ[l];
-                // the diagonal (lag 0) is G(t, t) = L^2 for every t: once per sample
-                if (l == 0 && h == 0) {
-                    c += (long long)Lt * L2;
-                    qv += (unsigned long long)Lt * L2 * L2;
-                }
-                if (write && c) atomicAdd(reinterpret_cast<unsigned long long *>(&g.Cacc[gbase + l]), (unsigned long long)c);
-                if (write && qv) atomicAdd(reinterpret_cast<unsigned long long *>(&g.Qacc[gbase + l]), qv);
-                binC[l] = 0;
-                binQ[l] = 0u;
-            }
-            asm volatile("bar.sync 1, %0;\n" ::"n"(kEpilogue) : "memory");
         }
     } else {
         // ------------------------------------------------------------------ MMA
-        // one thread issues every MMA; after the last tile of an item uses an
-        // A chunk, a commit frees that chunk for the next item's A block
+        // one thread issues every MMA; a commit after a chunk's MMAs frees its
+        // stage (and the older column block's slot of that chunk)
         if (lane == 0) {
             const uint32_t id128 = idesc_e4m3(128), id256 = idesc_e4m3(256);
             // 32-site steps of the last chunk: those of its 64-site words that
@@ -508,70 +567,58 @@ __global__ void __launch_bounds__(kThreads, 1)
             // sites over its whole 64-byte span)
             const int nk_last = min(kChunk / 32, 2 * ((L2 - (NC - 1) * kChunk + 63) / 64));
             const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
-            uint32_t a_par = 0u, b_par = 0u, n_t = 0;
-            int bs = 0;
+            uint32_t par = 0u, n_t = 0;
+            int st = 0, slot = 0, older = NS - 1;  // slots of the step's new column block and of the one before
             bool issued = false;
             for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-                const int h = u % nhalf;
-                for (int item = 0; item < unit_items(h, nb); ++item) {
-                    const int i = item_block(h, item, nb);
-                    {  // the diagonal tile: B = A, 128 columns
-                        const bool last = i + 1 >= nb;
-                        const int a = (int)(n_t & 1u);
-                        bool ok = mbar_wait(&ctl.accempty[a], ((n_t >> 1) & 1u) ^ 1u, &ctl.abort, wait_limit);
+                const Unit un = unit_of(pl, u);
+                for (int i = un.pair ? -1 : 0; i < un.steps; ++i) {
+                    const int a = (int)(n_t & 1u);
+                    bool ok = true;
+                    if (i >= 0) {
+                        ok = mbar_wait(&ctl.accempty[a], ((n_t >> 1) & 1u) ^ 1u, &ctl.abort, wait_limit);
                         asm volatile("tcgen05.fence::after_thread_sync;\n");
-                        const uint32_t d = tmem + (uint32_t)(a * 256);
+                    }
+                    const uint32_t d = tmem + (uint32_t)(a * 256);
+                    // two slots: both column blocks as one N = 256 MMA; more: one
+                    // N = 128 MMA per column block, the older block's first
+                    const uint32_t idesc = un.pair && NS == 2 ? id256 : id128;
+                    const uint32_t b0 =
+                        un.pair ? (NS == 2 ? 0u : (uint32_t)(older * kChunkBytes)) : (uint32_t)(slot * kChunkBytes);
+                    const uint32_t b1 = (uint32_t)(slot * kChunkBytes);
+                    const bool second = un.pair && NS > 2;
 #pragma unroll 1  // rolled: the three roles' code shares the instruction cache
-                        for (int kc = 0; kc < NC; ++kc) {
-                            ok = mbar_wait(&ctl.afull[kc], a_par, &ctl.abort, wait_limit) && ok;
-                            asm volatile("tcgen05.fence::after_thread_sync;\n");
-                            if (ok) {
-                                const uint32_t ab = sA0 + kc * kChunkBytes;
-                                const int nk = kc == NC - 1 ? nk_last : kChunk / 32;
+                    for (int kc = 0; kc < NC; ++kc) {
+                        ok = mbar_wait(&ctl.full[st], par, &ctl.abort, wait_limit) && ok;
+                        asm volatile("tcgen05.fence::after_thread_sync;\n");
+                        if (ok && i >= 0) {
+                            const uint32_t ab = sA0 + st * kChunkBytes;
+                            const uint32_t bb = RESIDENT ? sB0 + NS * kc * kChunkBytes : sB0 + st * kChunkBytes;
+                            const uint32_t bb0 = RESIDENT ? bb + b0 : bb;
+                            const int nk = kc == NC - 1 ? nk_last : kChunk / 32;
 #pragma unroll
-                                for (int kk = 0; kk < kChunk / 32; ++kk)
-                                    if (kk < nk)
-                                        mma_f8(d, sdesc_sw128(ab + kk * 32), sdesc_sw128(ab + kk * 32), id128,
-                                               (kc > 0 || kk > 0) ? 1u : 0u);
-                                issued = true;
-                            }
-                            if (last) mma_commit(&ctl.aempty[kc]);
+                            for (int kk = 0; kk < kChunk / 32; ++kk)
+                                if (kk < nk) {
+                                    mma_f8(d, sdesc_sw128(ab + kk * 32), sdesc_sw128(bb0 + kk * 32), idesc,
+                                           (kc > 0 || kk > 0) ? 1u : 0u);
+                                    if (NS > 2 && second)
+                                        mma_f8(d + kTile, sdesc_sw128(ab + kk * 32), sdesc_sw128(bb + b1 + kk * 32),
+                                               id128, (kc > 0 || kk > 0) ? 1u : 0u);
+                                }
+                            issued = true;
                         }
+                        mma_commit(&ctl.empty[st]);
+                        if (++st == nst) {
+                            st = 0;
+                            par ^= 1u;
+                        }
+                    }
+                    if (i >= 0) {
                         mma_commit(&ctl.accfull[a]);
                         ++n_t;
                     }
-                    for (int jp = i + 1; jp < nb; jp += 2) {  // column blocks jp and jp + 1
-                        const bool pair = jp + 1 < nb, last = jp + 2 >= nb;
-                        const int a = (int)(n_t & 1u);
-                        bool ok = mbar_wait(&ctl.accempty[a], ((n_t >> 1) & 1u) ^ 1u, &ctl.abort, wait_limit);
-                        asm volatile("tcgen05.fence::after_thread_sync;\n");
-                        const uint32_t d = tmem + (uint32_t)(a * 256);
-                        const uint32_t idesc = pair ? id256 : id128;
-#pragma unroll 1  // rolled: the three roles' code shares the instruction cache
-                        for (int kc = 0; kc < NC; ++kc) {
-                            ok = mbar_wait(&ctl.bfull[bs], b_par, &ctl.abort, wait_limit) && ok;
-                            asm volatile("tcgen05.fence::after_thread_sync;\n");
-                            if (ok) {
-                                const uint32_t ab = sA0 + kc * kChunkBytes, bb = sB0 + bs * kStageBytes;
-                                const int nk = kc == NC - 1 ? nk_last : kChunk / 32;
-#pragma unroll
-                                for (int kk = 0; kk < kChunk / 32; ++kk)
-                                    if (kk < nk)
-                                        mma_f8(d, sdesc_sw128(ab + kk * 32), sdesc_sw128(bb + kk * 32), idesc,
-                                               (kc > 0 || kk > 0) ? 1u : 0u);
-                                issued = true;
-                            }
-                            mma_commit(&ctl.bempty[bs]);
-                            if (last) mma_commit(&ctl.aempty[kc]);
-                            if (++bs == nstages) {
-                                bs = 0;
-                                b_par ^= 1u;
-                            }
-                        }
-                        mma_commit(&ctl.accfull[a]);
-                        ++n_t;
-                    }
-                    a_par ^= 1u;
+                    older = slot;
+                    if (++slot == NS) slot = 0;
                 }
             }
             // every MMA issued has completed before the tensor memory is released
@@ -598,57 +645,73 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 namespace {
 
-constexpr size_t kSmemLimit = 227 * 1024 - 256;  // dynamic + the static control block
+constexpr size_t kSmemLimit = 227 * 1024 - 4096;  // dynamic, beside the static control block and bins
 
-size_t gram_tc_smem_bytes(const Group &g, int nc, int nstages) {
-    return 1024 + (size_t)nc * kChunkBytes + (size_t)nstages * kStageBytes + 2 * sizeof(int) * (size_t)g.nlag;
-}
-
-// As many B stages as fit, up to six; at least two.
-int gram_tc_stages(const Group &g) {
-    const int nc = (g.L * g.L + kChunk - 1) / kChunk;
-    if (nc < 1 || nc > kMaxNc) return 0;
-    for (int s = kMaxStages; s >= 2; --s)
-        if (gram_tc_smem_bytes(g, nc, s) <= kSmemLimit) return s;
-    return 0;
+GramPlan gram_plan(const Group &g, int nsamples) {
+    GramPlan pl;
+    const int nc = (g.L * g.L + kChunk - 1) / kChunk, half = g.Ltau / 2;
+    const int mmax = g.Ltau < kTile ? g.Ltau - 1 : kTile - 1;
+    const int ne = (mmax + half + kTile) / kTile;  // column offsets that hold a lag <= L_tau / 2
+    pl.nsamples = nsamples;
+    pl.nb = (g.Ltau + kTile - 1) / kTile;
+    pl.npair = nc <= kPairNc ? ne / 2 : 0;
+    pl.nsingle = ne - 2 * pl.npair;
+    pl.e_single = 2 * pl.npair;
+    // where L_tau / 2 is a whole number of blocks, the tiles (i, e) and
+    // (i + nb / 2, e) of the last offset are each other's transpose
+    pl.e_mirror = half % kTile == 0 && pl.nb > 1 ? half / kTile : -1;
+    // resident: the slots' chunks, and no more stages than a stage's release
+    // can stand for (it must imply that of the slot to be overwritten, block_slots
+    // - 1 steps back); streamed: A and B chunks
+    const int ns = block_slots(nc);
+    const size_t fixed = 1024 + (nc <= kPairNc ? (size_t)ns * nc * kChunkBytes : 0);
+    const size_t per = (nc <= kPairNc ? 1 : 2) * (size_t)kChunkBytes;
+    int s = kMaxStages;
+    if (nc <= kPairNc && s > (ns - 1) * nc) s = (ns - 1) * nc;
+    while (s > 1 && fixed + s * per > kSmemLimit) --s;
+    pl.nstages = s;
+    // a thread's sum takes up to four squares (G / 2)^2 <= L^4 / 4 per step
+    // (exact in FP32 up to 2^24); two flushes of 256 squares per step stay
+    // below 2^31
+    const long long l4 = (long long)g.L * g.L * g.L * g.L;
+    const long long f = (1LL << 24) / l4;
+    pl.flush = (int)(f < 1 ? 1 : (f > 1024 ? 1024 : f));
+    pl.unit = 1u;
+    return pl;
 }
 
 template <int NC>
-cudaError_t launch_nc(const Group &g, int p0, int nsamples, int nstages, const uint64_t *P, int *status,
-                      unsigned wait_limit, int nsm, cudaStream_t st) {
-    const size_t sm = gram_tc_smem_bytes(g, NC, nstages);
+cudaError_t launch_nc(const Group &g, int p0, const GramPlan &pl, const uint64_t *P, int *status, unsigned wait_limit,
+                      int nsm, cudaStream_t st) {
+    const size_t sm =
+        1024 + (NC <= kPairNc ? (size_t)(block_slots(NC) * NC + pl.nstages) : (size_t)(2 * pl.nstages)) * kChunkBytes;
     cudaError_t e = cudaFuncSetAttribute(k_gram_tc<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    const int nb = (g.Ltau + kTile - 1) / kTile;
-    const long long nunits = (long long)nsamples * ((nb + 1) / 2);
+    const long long nunits = (long long)pl.nsamples * (pl.npair + pl.nsingle);
     const int grid = (int)(nunits < nsm ? nunits : nsm);
     count_launches(1);
-    k_gram_tc<NC><<<grid, kThreads, sm, st>>>(g, p0, P, nsamples, nstages, status, wait_limit);
+    k_gram_tc<NC><<<grid, kThreads, sm, st>>>(g, p0, P, pl, status, wait_limit);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-bool gram_tc_fits(const Group &g) { return gram_tc_stages(g) >= 2; }
-
 cudaError_t launch_gram_tc(const Group &g, int p0, int npairs, const uint64_t *P, int *status, unsigned wait_limit,
                            cudaStream_t st) {
-    const int nstages = gram_tc_stages(g);
-    if (nstages < 2) return cudaErrorInvalidValue;
     int dev = 0, nsm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int nsamples = npairs * g.R * 64;
+    const GramPlan pl = gram_plan(g, npairs * g.R * 64);
     switch ((g.L * g.L + kChunk - 1) / kChunk) {
-        case 1: return launch_nc<1>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 2: return launch_nc<2>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 3: return launch_nc<3>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 4: return launch_nc<4>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 5: return launch_nc<5>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 6: return launch_nc<6>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        case 7: return launch_nc<7>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
-        default: return launch_nc<8>(g, p0, nsamples, nstages, P, status, wait_limit, nsm, st);
+        case 1: return launch_nc<1>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 2: return launch_nc<2>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 3: return launch_nc<3>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 4: return launch_nc<4>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 5: return launch_nc<5>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 6: return launch_nc<6>(g, p0, pl, P, status, wait_limit, nsm, st);
+        case 7: return launch_nc<7>(g, p0, pl, P, status, wait_limit, nsm, st);
+        default: return launch_nc<8>(g, p0, pl, P, status, wait_limit, nsm, st);
     }
 }
 

@@ -86,7 +86,6 @@ cudaError_t launch_onetime_finish(const Group &g, long long n_meas, int triples,
 // 128 x 128 tile of the Gram matrices into the lag sums.
 cudaError_t launch_gram_tc(const Group &g, int p0, int npairs, const uint64_t *P, int *status, unsigned wait_limit,
                            cudaStream_t st);
-bool gram_tc_fits(const Group &g);  // the tensor-core path's shared memory fits one CTA
 
 // FP64 finish into g.outC / g.outQ / g.outP.
 cudaError_t launch_finish(const Group &g, long long n_meas, cudaStream_t st);
