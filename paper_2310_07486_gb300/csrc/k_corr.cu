@@ -122,7 +122,144 @@ __global__ void __launch_bounds__(256) k_gram(Group g, int p0, const uint64_t *P
     }
 }
 
-// Equal-time overlap of every replica pair at one ladder position.
+// Short extents of tau: all lags of a few samples per block on the integer pipes.
+// A 128 x 128 tensor tile has (L_tau / 128)^2 of its elements in use, and a unit of
+// one step leaves its fold to the lag bins unhidden, so small lattices spent 8,000
+// cycles per sample where XOR and popcount take a few hundred: L = 8, L_tau = 48,
+// 81,920 samples 2,110 us with tensor tiles, 72 us here.
+//
+// The rows of kShortSamples(..) samples are staged in shared memory, followed by
+// the first L_tau / 2 + 1 of them again as t >= L_tau (complemented under APBC: an
+// overlap with them then has its sign flipped), so a lag is a plain row offset.  A
+// thread owns the lags l, l + ng, l + 2 ng, l + 3 ng of one sample and walks the
+// rows: one read of row t1 serves four lags, consecutive lanes read consecutive
+// rows (an odd pitch keeps the banks apart).  Words are joined three at a time by a
+// full adder (two popcounts for three words), the popcount's rate being a quarter
+// of the logic's.  With n differing sites of L^2, c = L^2 - 2 n: the sums of n and
+// n^2 give those of c and c^2.
+constexpr int kShortThreads = 256;
+constexpr int kShortWords = 4;  // 64-site words of a slice at most (L <= 16)
+
+struct ShortShape {
+    int ng;       // lag groups (threads) per sample
+    int rows;     // rows staged per sample
+    int samples;  // samples per block
+    size_t bytes;
+};
+static ShortShape short_shape(const Group &g) {
+    ShortShape s;
+    s.ng = (g.nlag + 3) / 4;
+    s.rows = g.Ltau + g.nlag;
+    const int pitch = g.nwx | 1;
+    const size_t per = ((size_t)s.rows * pitch | 1) * sizeof(uint64_t);
+    s.samples = kShortThreads / s.ng;
+    while (s.samples > 1 && s.samples * per > 40 * 1024) --s.samples;
+    s.bytes = s.samples * per;
+    return s;
+}
+
+template <int NX>
+__device__ __forceinline__ int differing(const uint64_t (&x)[NX], const uint64_t *y) {
+    uint32_t d[2 * NX];
+#pragma unroll
+    for (int k = 0; k < NX; ++k) {
+        const uint64_t v = x[k] ^ y[k];
+        d[2 * k] = (uint32_t)v;
+        d[2 * k + 1] = (uint32_t)(v >> 32);
+    }
+    int one = 0, two = 0;
+    constexpr int T = 2 * NX / 3;
+#pragma unroll
+    for (int k = 0; k < T; ++k) {
+        one += __popc(d[3 * k] ^ d[3 * k + 1] ^ d[3 * k + 2]);
+        two += __popc(maj3(d[3 * k], d[3 * k + 1], d[3 * k + 2]));
+    }
+#pragma unroll
+    for (int k = 3 * T; k < 2 * NX; ++k) one += __popc(d[k]);
+    return one + 2 * two;
+}
+
+template <int NX>
+__global__ void __launch_bounds__(kShortThreads) k_gram_short(Group g, int p0, const uint64_t *__restrict__ P,
+                                                              int nsamples, ShortShape sh) {
+    extern __shared__ uint64_t rows[];
+    constexpr int pitch = NX | 1;
+    const int Lt = g.Ltau, L2 = g.L * g.L, nl = g.nlag;
+    const int per = sh.rows * pitch | 1;
+    const int s0 = blockIdx.x * sh.samples, ns = min(sh.samples, nsamples - s0);
+    const uint64_t *src = P + (size_t)s0 * Lt * NX;
+    const int n = Lt * NX;
+    for (int i = threadIdx.x; i < ns * n; i += kShortThreads) {
+        const int s = i / n, rk = i - s * n, t = rk / NX, k = rk - t * NX;
+        uint64_t v = src[i];
+        uint64_t *d = rows + (size_t)s * per + k;
+        d[t * pitch] = v;
+        if (t < nl) {
+            if (g.boundary == 1) {
+                const int left = L2 - 64 * k;  // sites of the lattice in this word
+                v ^= left >= 64 ? ~0ull : (1ull << left) - 1;
+            }
+            d[(t + Lt) * pitch] = v;
+        }
+    }
+    __syncthreads();
+    const int sl = threadIdx.x / sh.ng, lg = threadIdx.x - sl * sh.ng;
+    if (sl >= ns) return;
+    const uint64_t *base = rows + (size_t)sl * per;
+    unsigned sn[4] = {0u, 0u, 0u, 0u}, sq[4] = {0u, 0u, 0u, 0u};
+    const uint64_t *y[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) y[j] = base + min(lg + j * sh.ng, nl - 1) * pitch;
+#pragma unroll 2
+    for (int t = 0; t < Lt; ++t) {
+        uint64_t x[NX];
+#pragma unroll
+        for (int k = 0; k < NX; ++k) x[k] = base[t * pitch + k];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned d = (unsigned)differing<NX>(x, y[j] + t * pitch);
+            sn[j] += d;
+            sq[j] += d * d;
+        }
+    }
+    const int sample = s0 + sl, sb = sample / 64, b = sample % 64;
+    const int pb = sb / g.R, r = sb % g.R;
+    const int p = p0 + pb, w = p / g.K, jj = p % g.K;
+    const size_t idx = ((((size_t)r * g.W * 64) + (size_t)w * 64 + b) * g.K + jj) * nl;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int lag = lg + j * sh.ng;
+        if (lag < nl) {
+            const long long all = (long long)Lt * L2;
+            g.Cacc[idx + lag] += all - 2 * (long long)sn[j];
+            g.Qacc[idx + lag] += all * L2 - 4LL * L2 * sn[j] + 4LL * sq[j];
+        }
+    }
+}
+
+// Where the integer form is the faster one: its time grows as words x L_tau^2, that
+// of a short tensor unit hardly at all.  2,048 sample bits, us here / with tensor
+// tiles: L = 8, L_tau = 32 11 / 65, 128 20 / 71, 256 42 / 87; L = 10, L_tau = 128 29 / 73,
+// 256 79 / 91; L = 12, L_tau = 128 40 / 77, 192 58 / 94, 256 111 / 97; L = 16, L_tau = 128
+// 51 / 77, 192 112 / 95.  From two whole row blocks (L_tau = 256) on the tensor units
+// have steps to overlap and keep the work.
+static bool use_short(const Group &g) {
+    return g.nwx <= kShortWords && g.Ltau < 2 * 128 && g.nwx * g.Ltau <= 576;
+}
+
+static cudaError_t launch_gram_short(const Group &g, int p0, int npairs, const uint64_t *P, cudaStream_t st) {
+    const ShortShape sh = short_shape(g);
+    const int nsamples = npairs * g.R * 64, blocks = (nsamples + sh.samples - 1) / sh.samples;
+    count_launches(1);
+    switch (g.nwx) {
+        case 1: k_gram_short<1><<<blocks, kShortThreads, sh.bytes, st>>>(g, p0, P, nsamples, sh); break;
+        case 2: k_gram_short<2><<<blocks, kShortThreads, sh.bytes, st>>>(g, p0, P, nsamples, sh); break;
+        case 3: k_gram_short<3><<<blocks, kShortThreads, sh.bytes, st>>>(g, p0, P, nsamples, sh); break;
+        default: k_gram_short<4><<<blocks, kShortThreads, sh.bytes, st>>>(g, p0, P, nsamples, sh); break;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_words, int tensor, int triples,
                            int *status, unsigned wait_limit, cudaStream_t st) {
     const size_t per_pair = measure_scratch_words_per_pair(g);
@@ -149,7 +286,9 @@ cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_wor
                       st>>>(g, p0, np, scratch);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        if (tensor) {
+        if (tensor && use_short(g)) {
+            e = launch_gram_short(g, p0, np, scratch, st);
+        } else if (tensor) {
             e = launch_gram_tc(g, p0, np, scratch, status, wait_limit, st);
         } else {
             count_launches(1);
