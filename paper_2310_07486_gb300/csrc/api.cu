@@ -338,6 +338,7 @@ qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, 
     c->ws = (char *)d_workspace;
     c->ws_bytes = workspace_bytes;
     carve(c->groups, c->ws, &c->d_err, &c->scratch, &c->scratch_words, &c->pb);
+    for (Group &g : c->groups) g.err = c->d_err;
     c->stream = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream);
     for (const Group &g : c->groups)
@@ -452,7 +453,6 @@ qsg_status qsg_set_couplings(qsg_ctx *ctx, int32_t group, const int8_t *J_host) 
     return QSG_OK;
 }
 
-// Launch one sweep of every group; the sweep index is *sb + idx (sb may be null).
 // How the groups of one sweep are launched.
 enum SweepMode { MODE_SEQUENTIAL = 0, MODE_PERSISTENT = 1, MODE_CONCURRENT = 2 };
 
@@ -463,19 +463,36 @@ static SweepMode sweep_mode(const qsg_ctx *ctx) {
     return MODE_CONCURRENT;  // 3, or automatic with several groups
 }
 
-static qsg_status launch_one_sweep(qsg_ctx *ctx, bool persistent, const uint32_t *sb, uint32_t idx, cudaStream_t st);
+// `count` sweeps of one group on one stream, indices first .. first + count - 1
+// (added to *sb when sb is given).
+static qsg_status group_sweeps(qsg_ctx *ctx, const Group &g, const uint32_t *sb, uint32_t first, int count,
+                               cudaStream_t st) {
+    const bool fused = ctx->sweep_kernel != 1 && sweep_fused_supported(g, ctx->chunk);
+    if (!fused && sb) return QSG_ERR_ARG;  // the reference kernel takes its index by value only
+    for (int i = 0; i < count; ++i) {
+        const uint32_t idx = first + (uint32_t)i;
+        if (fused)
+            QSG_CUDA(ctx, launch_sweep_wavefront(g, sb, idx, ctx->seed, g.arrivals, ctx->chunk, ctx->tail, st));
+        else
+            QSG_CUDA(ctx, launch_sweep_reference(g, idx, ctx->seed, st));
+    }
+    return QSG_OK;
+}
 
 // `count` sweeps of every group with indices first .. first + count - 1 (added
-// to *sb when sb is given).  Concurrent mode: each group's chain of sweeps on
-// its own stream, forked from st and joined back into it (groups share no
+// to *sb when sb is given; it may be null).  Concurrent mode: each group's chain of
+// sweeps on its own stream, forked from st and joined back into it (groups share no
 // data, so only each group's own sweeps are ordered).
 static qsg_status launch_sweeps(qsg_ctx *ctx, SweepMode mode, const uint32_t *sb, uint32_t first, int count,
                                 cudaStream_t st) {
-    if (mode != MODE_CONCURRENT) {
-        for (int i = 0; i < count; ++i) {
-            qsg_status s = launch_one_sweep(ctx, mode == MODE_PERSISTENT, sb, first + (uint32_t)i, st);
-            if (s != QSG_OK) return s;
-        }
+    if (mode == MODE_PERSISTENT) {
+        for (int i = 0; i < count; ++i)
+            QSG_CUDA(ctx, launch_sweep_persistent(ctx->plan, sb, first + (uint32_t)i, ctx->seed, st));
+        return QSG_OK;
+    }
+    if (mode == MODE_SEQUENTIAL) {
+        for (const Group &g : ctx->groups)
+            if (qsg_status s = group_sweeps(ctx, g, sb, first, count, st)) return s;
         return QSG_OK;
     }
     const size_t ng = ctx->groups.size();
@@ -490,37 +507,11 @@ static qsg_status launch_sweeps(qsg_ctx *ctx, SweepMode mode, const uint32_t *sb
     }
     QSG_CUDA(ctx, cudaEventRecord(ctx->fork, st));
     for (size_t gi = 0; gi < ng; ++gi) {
-        const Group &g = ctx->groups[gi];
         cudaStream_t t = ctx->side[gi];
         QSG_CUDA(ctx, cudaStreamWaitEvent(t, ctx->fork, 0));
-        const int C = wavefront_chunk(g, ctx->chunk);
-        for (int i = 0; i < count; ++i) {
-            if (C > 0)
-                QSG_CUDA(ctx, launch_sweep_wavefront(g, sb, first + (uint32_t)i, ctx->seed, g.arrivals, C, ctx->tail, t));
-            else if (sb)
-                return QSG_ERR_ARG;
-            else
-                QSG_CUDA(ctx, launch_sweep_reference(g, first + (uint32_t)i, ctx->seed, t));
-        }
+        if (qsg_status s = group_sweeps(ctx, ctx->groups[gi], sb, first, count, t)) return s;
         QSG_CUDA(ctx, cudaEventRecord(ctx->joins[gi], t));
         QSG_CUDA(ctx, cudaStreamWaitEvent(st, ctx->joins[gi], 0));
-    }
-    return QSG_OK;
-}
-
-static qsg_status launch_one_sweep(qsg_ctx *ctx, bool persistent, const uint32_t *sb, uint32_t idx, cudaStream_t st) {
-    if (persistent) {
-        QSG_CUDA(ctx, launch_sweep_persistent(ctx->plan, sb, idx, ctx->seed, st));
-        return QSG_OK;
-    }
-    for (const Group &g : ctx->groups) {
-        const int C = ctx->sweep_kernel == 1 ? 0 : wavefront_chunk(g, ctx->chunk);
-        if (C > 0)
-            QSG_CUDA(ctx, launch_sweep_wavefront(g, sb, idx, ctx->seed, g.arrivals, C, ctx->tail, st));
-        else if (sb)
-            return QSG_ERR_ARG;  // the reference kernel takes its index by value only
-        else
-            QSG_CUDA(ctx, launch_sweep_reference(g, idx, ctx->seed, st));
     }
     return QSG_OK;
 }

@@ -474,17 +474,24 @@ static cudaError_t launch_wf_algo(const Group &g, int C, int tail, const uint32_
     return launch_wf_slot<ALGO, 1024>(g, C, tail, sb, sweep, seed, arrivals, st);
 }
 
+bool sweep_fused_supported(const Group &g, int requested) {
+    if (requested == 0 && g_wavefront_variant != 2 && sweep_unit_supported(g)) return true;
+    return wavefront_chunk(g, requested) > 0;
+}
+
 cudaError_t launch_sweep_wavefront(const Group &g, const uint32_t *sweep_base, uint32_t sweep, uint64_t seed,
-                                   unsigned *arrivals, int C, int tail, cudaStream_t st) {
-    // one unit per block with the lattice size compiled in (k_sweep_unit.cu)
-    // where that kernel exists, unless the generic kernel is asked for
-    if (g_wavefront_variant != 2 && sweep_unit_supported(g)) {
-        const int ts = tail_slots(g, C, tail);
-        // planes per barrier: four by default (the faster form for both
-        // algorithms), two as variant 1
-        const int pb = g_wavefront_variant == 1 ? 2 : 4;
-        return launch_sweep_unit(g, pb, C, ts > 0 ? C / 4 : C, g.nslots - ts, sweep_base, sweep, seed, arrivals, st);
+                                   unsigned *arrivals, int requested, int tail, cudaStream_t st) {
+    const bool unit = g_wavefront_variant != 2 && sweep_unit_supported(g);
+    const int C = wavefront_chunk(g, requested);
+    const int ts = C > 0 ? tail_slots(g, C, tail) : 0;
+    if (unit && requested == 0 && ts == 0) {
+        const int nch = sweep_unit_chunks(g);
+        return launch_sweep_unit(g, nch, nch, g.nslots, sweep_base, sweep, seed, arrivals, st);
     }
+    if (C == 0) return cudaErrorInvalidValue;
+    if (unit)
+        return launch_sweep_unit(g, g.Ltau / C, g.Ltau / (ts > 0 ? C / 4 : C), g.nslots - ts, sweep_base, sweep, seed,
+                                 arrivals, st);
     if (g.algo == 0) return launch_wf_algo<0>(g, C, tail, sweep_base, sweep, seed, arrivals, st);
     return launch_wf_algo<1>(g, C, tail, sweep_base, sweep, seed, arrivals, st);
 }

@@ -27,24 +27,26 @@ cudaError_t launch_init_spins(const Group &g, uint64_t seed, cudaStream_t st);
 // The "reference" variant runs one launch per colour with one thread per site.
 cudaError_t launch_sweep_reference(const Group &g, uint32_t sweep, uint64_t seed, cudaStream_t st);
 
-// The fused wavefront sweep: C = planes per work unit (0 if the group cannot
-// use this kernel), arrivals = nslots * (L_tau / 4) zeroed counters.
+// Planes per work unit of the generic wavefront kernel (0 if the group cannot use
+// it: L_tau no multiple of 16, or `requested` > 0 no multiple of 16 dividing it).
 int wavefront_chunk(const Group &g, int requested);
-// 0: one unit per block where k_sweep_unit exists (four planes per
-// barrier); 1: two planes per barrier; 3: four (as 0); 2: the generic kernel
+// 0, 1, 3: the fused kernel with the lattice size compiled in (k_sweep_unit.cuh)
+// where it exists; 2: the generic wavefront kernel
 extern int g_wavefront_variant;
-// The sweep index is *sweep_base + sweep (sweep_base may be null), so that a
-// captured CUDA graph of several sweeps can be replayed later.  The last
-// `tail` slots (0 = none) run chunks of C / 4 planes after every other unit.
+// One fused sweep, arrivals = nslots * (L_tau / 4) zeroed counters.  The sweep
+// index is *sweep_base + sweep (sweep_base may be null), so that a captured CUDA
+// graph of several sweeps can be replayed later.  requested: planes per work unit
+// (0 = automatic); the last `tail` slots (0 = none) run chunks of a quarter of
+// that after every other unit.
+bool sweep_fused_supported(const Group &g, int requested);
 cudaError_t launch_sweep_wavefront(const Group &g, const uint32_t *sweep_base, uint32_t sweep, uint64_t seed,
-                                   unsigned *arrivals, int C, int tail, cudaStream_t st);
-// The one-unit-per-block form (k_sweep_unit.cu) for L = 20, 24: slots
-// [0, S1) in chunks of C planes, the others in chunks of C2; 2 or 4 planes
-// per block barrier.
+                                   unsigned *arrivals, int requested, int tail, cudaStream_t st);
+// The form with the lattice size compiled in (L >= 6, any L_tau): slots [0, S1)
+// in nch chunks, the others in nch2.
 bool sweep_unit_supported(const Group &g);
-cudaError_t launch_sweep_unit(const Group &g, int planes_per_barrier, int C, int C2, int S1,
-                              const uint32_t *sweep_base, uint32_t sweep, uint64_t seed, unsigned *arrivals,
-                              cudaStream_t st);
+int sweep_unit_chunks(const Group &g);  // the automatic choice of nch
+cudaError_t launch_sweep_unit(const Group &g, int nch, int nch2, int S1, const uint32_t *sweep_base, uint32_t sweep,
+                              uint64_t seed, unsigned *arrivals, cudaStream_t st);
 cudaError_t launch_set_word(uint32_t *p, uint32_t value, cudaStream_t st);
 // dst[0..words) = src[0..words), device to device, by a kernel when both are
 // 16-byte aligned and words is even (else by cudaMemcpyAsync).
