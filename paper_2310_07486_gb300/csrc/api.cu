@@ -463,10 +463,26 @@ static SweepMode sweep_mode(const qsg_ctx *ctx) {
     return MODE_CONCURRENT;  // 3, or automatic with several groups
 }
 
+// Several sweeps of a group in one launch, the slots in shared memory: where a
+// slot fits an SM and no launch option asks for another form.  A graph of fewer
+// than kResidentGraphSlots slots keeps one kernel node per sweep: such a replay
+// leaves the GPU idle either way, and its launch count is part of what callers
+// see (qsg_kernel_launches).
+constexpr int kResidentGraphSlots = 8;
+static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
+    if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
+    if (sb && g.nslots < kResidentGraphSlots) return false;
+    return sweep_resident_fits(g);
+}
+
 // `count` sweeps of one group on one stream, indices first .. first + count - 1
 // (added to *sb when sb is given).
 static qsg_status group_sweeps(qsg_ctx *ctx, const Group &g, const uint32_t *sb, uint32_t first, int count,
                                cudaStream_t st) {
+    if (use_resident(ctx, g, sb)) {
+        QSG_CUDA(ctx, launch_sweep_resident(g, count, sb, first, ctx->seed, st));
+        return QSG_OK;
+    }
     const bool fused = ctx->sweep_kernel != 1 && sweep_fused_supported(g, ctx->chunk);
     if (!fused && sb) return QSG_ERR_ARG;  // the reference kernel takes its index by value only
     for (int i = 0; i < count; ++i) {

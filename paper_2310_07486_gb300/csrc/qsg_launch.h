@@ -47,6 +47,10 @@ bool sweep_unit_supported(const Group &g);
 int sweep_unit_chunks(const Group &g);  // the automatic choice of nch
 cudaError_t launch_sweep_unit(const Group &g, int nch, int nch2, int S1, const uint32_t *sweep_base, uint32_t sweep,
                               uint64_t seed, unsigned *arrivals, cudaStream_t st);
+// `count` sweeps in one launch, each slot in one block's shared memory.
+bool sweep_resident_fits(const Group &g);
+cudaError_t launch_sweep_resident(const Group &g, int count, const uint32_t *sweep_base, uint32_t sweep, uint64_t seed,
+                                  cudaStream_t st);
 cudaError_t launch_set_word(uint32_t *p, uint32_t value, cudaStream_t st);
 // dst[0..words) = src[0..words), device to device, by a kernel when both are
 // 16-byte aligned and words is even (else by cudaMemcpyAsync).
