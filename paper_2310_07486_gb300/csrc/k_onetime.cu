@@ -18,7 +18,14 @@
 //   sum_c n_c n_{c+d} = L^3 - 4 L A + 4 sum_c a_c a_{c+d},
 // and the last sum is a dot product of byte vectors (four columns per
 // __dp4a); the column counts come from a bitsliced vertical add of the L row
-// words of the slice.
+// words of the slice (full adders over pairs of rows).  The sums over pairs and
+// over triples of a slice stay in 32-bit registers as long as they are exact there.
+// Integer instructions bound it (about 10 K per slice at L = 24, R = 4, most in the
+// 12 three-replica cross-correlations of 24 counts over all lags).  Before these two
+// forms, and with 128 threads whatever L_tau: 792 -> 545 us
+// (L = 24, L_tau = 2048, 64 samples, R = 4, 8 k), 727 -> 530 us (L = 16, L_tau = 512,
+// R = 6), 291 -> 154 us (L = 8, L_tau = 48, 640 samples), 55 -> 27 us (L = 12, L_tau =
+// 64, 64 samples).
 //
 // Input: the transposed scratch of the correlator pass ([pair][r][bit][tau]
 // [nwx] x-packed slices, bit n = y L + x of word n / 64).  One block per
@@ -26,8 +33,13 @@
 #include <type_traits>
 
 #include "qsg_launch.h"
+#include "qsg_sweep.cuh"
 
 namespace qsg {
+
+using sweep::kMaj3;
+using sweep::kXor3;
+using sweep::lop3;
 
 constexpr int kMaxTripleR = 8;  // three-replica terms for 3 <= R <= 8
 // Replica pairs whose Q^2 sums a block keeps in shared memory; with more
@@ -47,6 +59,13 @@ struct OtSize {
     static constexpr int ND = ((L - 1) + 4 * (NP - 1)) / 4 + 2;
 };
 
+// Triples whose F3 sums fit an int32 together (a triple's is below 6 L^2 2 L^3),
+// and pairs whose G sums do (below 4 L^3 each).
+template <int L>
+constexpr int kTripleSafe = (int)(0x7FFFFFFFLL / (12LL * L * L * L * L * L));
+template <int L>
+constexpr int kGSafe = (int)(0x7FFFFFFFLL / (4LL * L * L * L));
+
 // Pack four small non-negative ints into bytes 0..3.
 __device__ __forceinline__ uint32_t pack_bytes(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
     return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
@@ -63,11 +82,13 @@ __device__ __forceinline__ void diff_counts(const uint64_t *__restrict__ X, cons
 #pragma unroll
     for (int q = 0; q < NW; ++q) o[q] = X[q] ^ Y[q];
     // rows (bits r L .. r L + L - 1), their counts, and the vertical bitsliced
-    // sum of the rows: bit c of plane j is bit j of column c's count; after
-    // row r a count is at most r + 1, which bounds the carry chain
-    uint32_t P[NPL];
+    // sum of the rows: bit c of plane j is bit j of column c's count.  Rows enter
+    // two at a time through a full adder whose carry is an input of the next
+    // plane, so L rows take about L adders of two lop3 (a ripple per row took
+    // about 2 L log2 L operations)
+    uint32_t P[NPL + 1], wait[NPL + 1];
 #pragma unroll
-    for (int j = 0; j < NPL; ++j) P[j] = 0u;
+    for (int j = 0; j <= NPL; ++j) P[j] = wait[j] = 0u;
     uint32_t rb[4 * NP];
     A = 0;
 #pragma unroll
@@ -79,14 +100,33 @@ __device__ __forceinline__ void diff_counts(const uint64_t *__restrict__ X, cons
         const uint32_t row = (uint32_t)(f & mask);
         rb[r] = (uint32_t)__popc(row);
         A += (int)rb[r];
-        uint32_t carry = row;
+        // plane j takes an input every 2^j rows and keeps every second one
+        // waiting for its partner (which ones is known at compile time)
+        uint32_t in = row;
+        bool more = true;
 #pragma unroll
         for (int j = 0; j < NPL; ++j)
-            if (j < bit_length(r + 1)) {
-                const uint32_t t = P[j] & carry;
-                P[j] ^= carry;
-                carry = t;
+            if (more) {
+                if (((r >> j) & 1) == 0) {
+                    wait[j] = in;
+                    more = false;
+                } else {
+                    const uint32_t a = P[j], b = wait[j];
+                    P[j] = lop3<kXor3>(a, b, in);
+                    in = lop3<kMaj3>(a, b, in);
+                }
             }
+    }
+    // inputs left without a partner
+    {
+        uint32_t carry = 0u;
+#pragma unroll
+        for (int j = 0; j < NPL; ++j) {
+            const uint32_t in = ((L >> j) & 1) ? wait[j] : 0u;
+            const uint32_t a = P[j];
+            P[j] = lop3<kXor3>(a, in, carry);
+            carry = lop3<kMaj3>(a, in, carry);
+        }
     }
 #pragma unroll
     for (int r = L; r < 4 * NP; ++r) rb[r] = 0u;
@@ -183,6 +223,10 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
     unsigned long long p4lo = 0, p4hi = 0;
     for (int t = tid; t < Lt; t += bd) {
         int pi = 0;
+        int gs[H + 1];  // G sums of up to kGSafe pairs of the slice
+        int in_gs = 0;
+#pragma unroll
+        for (int d = 0; d <= H; ++d) gs[d] = 0;
         for (int ra = 0; ra < R; ++ra)
             for (int rb = ra + 1; rb < R; ++rb, ++pi) {
                 uint32_t ca[NP], cb[NP];
@@ -205,8 +249,16 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
                     for_d<0, H>([&](auto dc) {
                         constexpr int d = decltype(dc)::value;
                         const int sv = 2 * L3 - 8 * L * A + 4 * (cyc_dot<L, d>(ca, dda) + cyc_dot<L, d>(cb, ddb));
-                        accsh[(size_t)d * bd + tid] += (d == 0 || d == H) ? sv : 2 * sv;  // G[d] = G[L - d]
+                        gs[d] += (d == 0 || d == H) ? sv : 2 * sv;  // G[d] = G[L - d]
                     });
+                }
+                if (++in_gs == kGSafe<L>) {
+                    in_gs = 0;
+#pragma unroll
+                    for (int d = 0; d <= H; ++d) {
+                        accsh[(size_t)d * bd + tid] += gs[d];
+                        gs[d] = 0;
+                    }
                 }
                 if (do3) {
 #pragma unroll
@@ -217,9 +269,17 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
                     qsh[(size_t)pi * bd + tid] = (int16_t)q0;
                 }
             }
+        if (in_gs) {
+#pragma unroll
+            for (int d = 0; d <= H; ++d) accsh[(size_t)d * bd + tid] += gs[d];
+        }
         if (!do3) continue;
         // pair index of (a, b), a < b: a (2R - a - 1) / 2 + (b - a - 1)
         auto pid = [R](int a, int b2) { return a * (2 * R - a - 1) / 2 + (b2 - a - 1); };
+        int ft[H + 1];  // F3 sums of up to kTripleSafe triples
+        int in_ft = 0;
+#pragma unroll
+        for (int d = 0; d <= H; ++d) ft[d] = 0;
         for (int ra = 0; ra < R; ++ra)
             for (int rb = ra + 1; rb < R; ++rb)
                 for (int rc = rb + 1; rc < R; ++rc) {
@@ -227,9 +287,6 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
                     const long long qab = qsh[(size_t)ab * bd + tid], qbc = qsh[(size_t)bc * bd + tid],
                                     qac = qsh[(size_t)ac * bd + tid];
                     t3 += qab * qbc * qac;
-                    int ft[H + 1];  // this triple's F3 sums (int32: < 6 * 2^10 * 2^16)
-#pragma unroll
-                    for (int d = 0; d <= H; ++d) ft[d] = 0;
                     // the replica shared by the two momentum-carrying overlaps: a, b, c
 #pragma unroll 1
                     for (int rot = 0; rot < 3; ++rot) {
@@ -261,9 +318,19 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
                             });
                         }
                     }
+                    if (++in_ft == kTripleSafe<L>) {
+                        in_ft = 0;
 #pragma unroll
-                    for (int d = 0; d <= H; ++d) accsh[(size_t)(H + 1 + d) * bd + tid] += ft[d];
+                        for (int d = 0; d <= H; ++d) {
+                            accsh[(size_t)(H + 1 + d) * bd + tid] += ft[d];
+                            ft[d] = 0;
+                        }
+                    }
                 }
+        if (in_ft) {
+#pragma unroll
+            for (int d = 0; d <= H; ++d) accsh[(size_t)(H + 1 + d) * bd + tid] += ft[d];
+        }
     }
 
     __syncthreads();
@@ -310,8 +377,10 @@ size_t onetime_smem_bytes(const Group &g, int triples, int threads) {
 template <int L>
 static cudaError_t launch_onetime_L(const Group &g, int p0, int np, const uint64_t *P, int triples,
                                     cudaStream_t st) {
-    int threads = 128;
-    while (threads > 32 && onetime_smem_bytes(g, triples, threads) > 96 * 1024) threads /= 2;
+    // a thread per slice: where L_tau is short, no more of them than slices (L = 8,
+    // L_tau = 48 ran 128 for 48)
+    int threads = g.Ltau >= 128 ? 128 : (g.Ltau + 31) / 32 * 32;
+    while (threads > 32 && onetime_smem_bytes(g, triples, threads) > 96 * 1024) threads -= 32;
     const size_t sm = onetime_smem_bytes(g, triples, threads);
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_onetime<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
