@@ -181,8 +181,7 @@ __global__ void __launch_bounds__(512, 2) k_energy(Group g) {
         if (cnt[b]) atomicAdd(&g.U[(size_t)s * 64 + b], cnt[b]);
 }
 
-// k_energy with L compiled in (the lattice sizes of the sweep's fixed-L
-// kernels and the smaller even sizes of the ragged workloads).  The same
+// k_energy with L compiled in (L = 6 .. 24).  The same
 // count, in a leaner loop: each step's four planes come in one cp.async group
 // and the four refill copies use constant offsets; a thread keeps its own two
 // words of the next plane (they are the +tau neighbours of this one) in
@@ -412,12 +411,18 @@ cudaError_t launch_energy(const Group &g, cudaStream_t st) {
     // runs of 256 planes halve the final warp sums per word where L_tau
     // leaves enough blocks (4.5 waves of 456 resident blocks at the 256-slot
     // L = 24, L_tau = 2048 state: 0.55 -> 0.52 ms)
-    const bool long_runs = g.Ltau >= 1024;
+    // and runs of 128 where they do not (64 slots of L = 18, L_tau = 1024: 256 blocks)
+    const bool long_runs = g.Ltau >= 1024 && (long long)g.nslots * (g.Ltau / 256) >= 152 * 3 * 2;
     switch (g.L) {
+        case 6: return long_runs ? launch_energy_l<6, 256>(g, st) : launch_energy_l<6, 128>(g, st);
         case 8: return long_runs ? launch_energy_l<8, 256>(g, st) : launch_energy_l<8, 128>(g, st);
+        case 10: return long_runs ? launch_energy_l<10, 256>(g, st) : launch_energy_l<10, 128>(g, st);
         case 12: return long_runs ? launch_energy_l<12, 256>(g, st) : launch_energy_l<12, 128>(g, st);
+        case 14: return long_runs ? launch_energy_l<14, 256>(g, st) : launch_energy_l<14, 128>(g, st);
         case 16: return long_runs ? launch_energy_l<16, 256>(g, st) : launch_energy_l<16, 128>(g, st);
+        case 18: return long_runs ? launch_energy_l<18, 256>(g, st) : launch_energy_l<18, 128>(g, st);
         case 20: return long_runs ? launch_energy_l<20, 256>(g, st) : launch_energy_l<20, 128>(g, st);
+        case 22: return long_runs ? launch_energy_l<22, 256>(g, st) : launch_energy_l<22, 128>(g, st);
         case 24: return long_runs ? launch_energy_l<24, 256>(g, st) : launch_energy_l<24, 128>(g, st);
         default: return launch_energy_generic(g, st);
     }
@@ -432,40 +437,88 @@ cudaError_t launch_energy(const Group &g, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 constexpr int kMaxK = 128;
 
-__global__ void __launch_bounds__(64) k_pt_decide(Group g, uint32_t m, uint32_t k0, uint32_t k1) {
-    const int wr = blockIdx.x, b = threadIdx.x;
+//
+// The chain over pairs is serial (the configuration that meets pair i is the one
+// pair i - 1 left), so everything that does not depend on it is brought to shared
+// memory first by the whole block: the counts of every position, the uniforms
+// (one Philox call for four samples of a pair), the 64-entry tables B and the first
+// kDecideA entries of the tables A (differences below 64 kDecideA; the few above
+// read global memory).  With all of them fetched inside the chain a step of 32
+// positions took 21-28 us; it takes 11.
+constexpr int kDecideThreads = 256;
+constexpr int kDecideA = 64;
+
+struct DecideShared {  // offsets into the dynamic shared memory, for K positions
+    size_t u, b, a, off, total;
+    __host__ __device__ explicit DecideShared(int K) {
+        u = sizeof(int32_t) * 64 * (size_t)K;                      // after the counts [K][64]
+        b = (u + sizeof(uint32_t) * 64 * (size_t)(K - 1) + 7) / 8 * 8;  // after the uniforms [K - 1][64]
+        a = b + sizeof(uint64_t) * 64 * (size_t)(K - 1);           // after the tables B [K - 1][64]
+        off = a + sizeof(uint64_t) * kDecideA * (size_t)(K - 1);   // after the heads of the tables A
+        total = off + 2 * sizeof(int32_t) * (size_t)(K - 1);       // offsets and lengths of the tables A
+    }
+};
+
+__global__ void __launch_bounds__(kDecideThreads) k_pt_decide(Group g, uint32_t m, uint32_t k0, uint32_t k1) {
+    extern __shared__ __align__(16) unsigned char dec_smem[];
+    const int wr = blockIdx.x, tid = threadIdx.x;
     const int w = wr / g.R;
     const int K = g.K;
-    const long long three_n = 3LL * g.N;
-    long long E[kMaxK];
-    for (int j = 0; j < K; ++j) E[j] = 2LL * g.U[((size_t)wr * K + j) * 64 + b] - three_n;
+    const DecideShared ds(K);
+    int32_t *sU = reinterpret_cast<int32_t *>(dec_smem);
+    uint32_t *su = reinterpret_cast<uint32_t *>(dec_smem + ds.u);
+    uint64_t *sB = reinterpret_cast<uint64_t *>(dec_smem + ds.b);
+    uint64_t *sA = reinterpret_cast<uint64_t *>(dec_smem + ds.a);
+    int32_t *sOff = reinterpret_cast<int32_t *>(dec_smem + ds.off), *sLen = sOff + (K - 1);
+    const int32_t *U = g.U + (size_t)wr * K * 64;
     const uint32_t tag = (STREAM_PT << 24) | ((uint32_t)g.gid << 8);
-    for (int i = 0; i + 1 < K; ++i) {
-        const uint4 r = philox4x32_10(make_uint4((uint32_t)(i * 16 + b / 4), m, (uint32_t)wr, tag), k0, k1);
-        const uint32_t u = pick(r, b & 3);
-        bool accept;
-        if (E[i + 1] >= E[i]) {
-            accept = true;
-        } else {
-            const long long n = E[i] - E[i + 1];
-            if ((n >> 6) >= g.ptA_len[i]) {
-                accept = false;
+    for (int i = tid; i < K * 64; i += kDecideThreads) sU[i] = U[i];
+    for (int i = tid; i < (K - 1) * 64; i += kDecideThreads) sB[i] = g.ptB[i];
+    for (int i = tid; i < (K - 1) * kDecideA; i += kDecideThreads) {
+        const int pair = i / kDecideA, e = i % kDecideA;
+        if (e < g.ptA_len[pair]) sA[i] = g.ptA[g.ptA_off[pair] + e];
+    }
+    for (int i = tid; i < K - 1; i += kDecideThreads) {
+        sOff[i] = g.ptA_off[i];
+        sLen[i] = g.ptA_len[i];
+    }
+    for (int i = tid; i < (K - 1) * 16; i += kDecideThreads) {  // pair i / 16, samples 4 (i % 16) ..
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)i, m, (uint32_t)wr, tag), k0, k1);
+        *reinterpret_cast<uint4 *>(su + 4 * i) = r;
+    }
+    __syncthreads();
+    if (tid < 64) {
+        const int b = tid;
+        int cur = sU[b];  // the count of the configuration at position i
+        for (int i = 0; i + 1 < K; ++i) {
+            const int nxt = sU[(i + 1) * 64 + b];
+            const uint32_t u = su[i * 64 + b];
+            // E = 2 U - 3 N: n = E_i - E_i+1
+            bool accept = nxt >= cur;
+            if (!accept) {
+                const int n = 2 * (cur - nxt);  // below 2^31: U <= 3 N < 2^29
+                if ((n >> 6) < sLen[i]) {
+                    const int e = n >> 6;
+                    const uint64_t A = e < kDecideA ? sA[i * kDecideA + e] : g.ptA[sOff[i] + e];
+                    const unsigned long long thr = (A * sB[i * 64 + (n & 63)]) >> 32;
+                    accept = (unsigned long long)u < thr;
+                }
+            }
+            const uint32_t ball = __ballot_sync(0xffffffffu, accept);
+            if ((b & 31) == 0) g.swapmask[((size_t)wr * (K - 1) + i) * 2 + (b >> 5)] = ball;
+            if (accept) {
+                sU[i * 64 + b] = nxt;  // cur moves on to position i + 1
+                atomicAdd(&g.acc[((size_t)w * 64 + b) * (K - 1) + i], 1ull);
             } else {
-                const unsigned long long thr =
-                    (g.ptA[g.ptA_off[i] + (n >> 6)] * g.ptB[i * 64 + (n & 63)]) >> 32;
-                accept = (unsigned long long)u < thr;
+                sU[i * 64 + b] = cur;
+                cur = nxt;
             }
         }
-        const uint32_t ball = __ballot_sync(0xffffffffu, accept);
-        if ((b & 31) == 0) g.swapmask[((size_t)wr * (K - 1) + i) * 2 + (b >> 5)] = ball;
-        if (accept) {
-            const long long tmp = E[i];
-            E[i] = E[i + 1];
-            E[i + 1] = tmp;
-            atomicAdd(&g.acc[((size_t)w * 64 + b) * (K - 1) + i], 1ull);
-        }
+        sU[(K - 1) * 64 + b] = cur;
     }
-    for (int j = 0; j < K; ++j) g.U[((size_t)wr * K + j) * 64 + b] = (int32_t)((E[j] + three_n) / 2);
+    __syncthreads();
+    int32_t *out = g.U + (size_t)wr * K * 64;
+    for (int i = tid; i < K * 64; i += kDecideThreads) out[i] = sU[i];
 }
 
 // Apply the swaps of one tempering step to the spin words.  A block serves
@@ -552,9 +605,13 @@ static cudaError_t launch_apply(const Group &g, cudaStream_t st);
 
 cudaError_t launch_tempering(const Group &g, uint32_t m, uint64_t seed, cudaStream_t st) {
     if (g.K < 2) return cudaSuccess;
+    const size_t sm = DecideShared(g.K).total;
+    cudaError_t e = cudaSuccess;
+    if (sm > 48 * 1024) e = cudaFuncSetAttribute(k_pt_decide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
     count_launches(1);
-    k_pt_decide<<<g.W * g.R, 64, 0, st>>>(g, m, (uint32_t)seed, (uint32_t)(seed >> 32));
-    const cudaError_t e = cudaGetLastError();
+    k_pt_decide<<<g.W * g.R, kDecideThreads, sm, st>>>(g, m, (uint32_t)seed, (uint32_t)(seed >> 32));
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_apply(g, st);
 }
