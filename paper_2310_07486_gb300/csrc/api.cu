@@ -29,6 +29,7 @@ struct Range {
 
 constexpr size_t kAlign = 256;
 constexpr int kMaxA = 16384;               // longest A_i table of the tempering test
+constexpr size_t kOwnScratch = 64u << 20;  // largest whole correlator scratch of a group that gets its own
 constexpr size_t kScratchCap = 1024u << 20;  // bytes of correlator scratch (transposed bits, E4M3 rows)
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -87,6 +88,7 @@ size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, 
     };
     *err = (int *)take(sizeof(int) * 4);
     size_t sw = 0;
+    const bool several = gs.size() > 1;
     for (auto &g : gs) {
         g.S = (uint64_t *)take(sizeof(uint64_t) * (size_t)g.nslots * g.N);
         g.Jx = (uint64_t *)take(sizeof(uint64_t) * (size_t)g.W * g.L * g.L);
@@ -123,6 +125,15 @@ size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, 
         if (want < per) want = per;
         const size_t all = per * (size_t)g.W * g.K;
         if (want > all) want = all;
+        // a small group among several has a scratch of its own, so that the
+        // measurements of small groups can overlap; the others share one
+        g.scratch = nullptr;
+        g.scratch_words = 0;
+        if (several && all * sizeof(uint64_t) <= kOwnScratch) {
+            g.scratch = (uint64_t *)take(sizeof(uint64_t) * all);
+            g.scratch_words = all;
+            want = 0;
+        }
         // the scratch also holds the coupling features, [W*64][64] float
         const size_t feat = (size_t)g.W * 64 * 64 / 2;
         if (want < feat) want = feat;
@@ -463,6 +474,40 @@ static SweepMode sweep_mode(const qsg_ctx *ctx) {
     return MODE_CONCURRENT;  // 3, or automatic with several groups
 }
 
+// Run work(g, stream) for every group: those with side(g) each on a stream of its
+// own, forked from st, the others one after another on st; st continues after all
+// of them.  Groups share no data (but for the correlator scratch, see
+// qsg_measure_correlators), so only each group's own work is ordered.
+extern "C++" {
+template <class Side, class Work>
+static qsg_status on_side_streams(qsg_ctx *ctx, cudaStream_t st, Side side, Work work) {
+    const size_t ng = ctx->groups.size();
+    if (!ctx->fork) QSG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming));
+    while (ctx->side.size() < ng) {
+        cudaStream_t t = nullptr;
+        cudaEvent_t e = nullptr;
+        QSG_CUDA(ctx, cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+        ctx->side.push_back(t);
+        QSG_CUDA(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        ctx->joins.push_back(e);
+    }
+    QSG_CUDA(ctx, cudaEventRecord(ctx->fork, st));
+    for (size_t gi = 0; gi < ng; ++gi) {
+        const Group &g = ctx->groups[gi];
+        if (!side(g)) continue;
+        QSG_CUDA(ctx, cudaStreamWaitEvent(ctx->side[gi], ctx->fork, 0));
+        if (qsg_status s = work(g, ctx->side[gi])) return s;
+        QSG_CUDA(ctx, cudaEventRecord(ctx->joins[gi], ctx->side[gi]));
+    }
+    for (const Group &g : ctx->groups)
+        if (!side(g))
+            if (qsg_status s = work(g, st)) return s;
+    for (size_t gi = 0; gi < ng; ++gi)
+        if (side(ctx->groups[gi])) QSG_CUDA(ctx, cudaStreamWaitEvent(st, ctx->joins[gi], 0));
+    return QSG_OK;
+}
+}  // extern "C++"
+
 // Several sweeps of a group in one launch, the slots in shared memory: where a
 // slot fits an SM and no launch option asks for another form.  A graph of fewer
 // than kResidentGraphSlots slots keeps one kernel node per sweep: such a replay
@@ -511,25 +556,9 @@ static qsg_status launch_sweeps(qsg_ctx *ctx, SweepMode mode, const uint32_t *sb
             if (qsg_status s = group_sweeps(ctx, g, sb, first, count, st)) return s;
         return QSG_OK;
     }
-    const size_t ng = ctx->groups.size();
-    if (!ctx->fork) QSG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming));
-    while (ctx->side.size() < ng) {
-        cudaStream_t t = nullptr;
-        cudaEvent_t e = nullptr;
-        QSG_CUDA(ctx, cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
-        ctx->side.push_back(t);
-        QSG_CUDA(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        ctx->joins.push_back(e);
-    }
-    QSG_CUDA(ctx, cudaEventRecord(ctx->fork, st));
-    for (size_t gi = 0; gi < ng; ++gi) {
-        cudaStream_t t = ctx->side[gi];
-        QSG_CUDA(ctx, cudaStreamWaitEvent(t, ctx->fork, 0));
-        if (qsg_status s = group_sweeps(ctx, ctx->groups[gi], sb, first, count, t)) return s;
-        QSG_CUDA(ctx, cudaEventRecord(ctx->joins[gi], t));
-        QSG_CUDA(ctx, cudaStreamWaitEvent(st, ctx->joins[gi], 0));
-    }
-    return QSG_OK;
+    return on_side_streams(
+        ctx, st, [](const Group &) { return true; },
+        [&](const Group &g, cudaStream_t t) { return group_sweeps(ctx, g, sb, first, count, t); });
 }
 
 // (Re)capture the graph of graph_batch sweeps when a launch option changed.
@@ -609,9 +638,18 @@ qsg_status qsg_tempering_swap(qsg_ctx *ctx) {
     Range range("qsg_tempering_swap");
     if (!ctx) return QSG_ERR_ARG;
     if (!ctx->initialised) return QSG_ERR_STATE;
-    qsg_status s = ensure_energy(ctx);
-    if (s != QSG_OK) return s;
-    for (const Group &g : ctx->groups) QSG_CUDA(ctx, launch_tempering(g, ctx->swaps, ctx->seed, ctx->stream));
+    auto work = [&](const Group &g, cudaStream_t st) -> qsg_status {
+        if (!ctx->energy_fresh) QSG_CUDA(ctx, launch_energy(g, st));
+        QSG_CUDA(ctx, launch_tempering(g, ctx->swaps, ctx->seed, st));
+        return QSG_OK;
+    };
+    if (sweep_mode(ctx) == MODE_CONCURRENT) {
+        if (qsg_status s = on_side_streams(ctx, ctx->stream, [](const Group &) { return true; }, work)) return s;
+    } else {
+        for (const Group &g : ctx->groups)
+            if (qsg_status s = work(g, ctx->stream)) return s;
+    }
+    ctx->energy_fresh = true;
     ctx->swaps++;
     return QSG_OK;
 }
@@ -621,9 +659,21 @@ qsg_status qsg_measure_correlators(qsg_ctx *ctx) {
     if (!ctx) return QSG_ERR_ARG;
     if (!ctx->initialised) return QSG_ERR_STATE;
     if (qsg_status o = order_after_copies(ctx)) return o;
-    for (const Group &g : ctx->groups)
-        QSG_CUDA(ctx, launch_measure(g, ctx->scratch, ctx->scratch_words, ctx->corr_tensor, ctx->triples, ctx->d_err,
-                                     ctx->wait_limit, ctx->stream));
+    auto work = [&](const Group &g, cudaStream_t st) -> qsg_status {
+        uint64_t *scratch = g.scratch ? g.scratch : ctx->scratch;
+        const size_t words = g.scratch ? g.scratch_words : ctx->scratch_words;
+        QSG_CUDA(ctx, launch_measure(g, scratch, words, ctx->corr_tensor, ctx->triples, ctx->d_err, ctx->wait_limit, st));
+        return QSG_OK;
+    };
+    if (sweep_mode(ctx) == MODE_CONCURRENT) {
+        // groups on the shared scratch follow one another on the context's stream
+        if (qsg_status s =
+                on_side_streams(ctx, ctx->stream, [](const Group &g) { return g.scratch != nullptr; }, work))
+            return s;
+    } else {
+        for (const Group &g : ctx->groups)
+            if (qsg_status s = work(g, ctx->stream)) return s;
+    }
     ctx->n_meas++;
     return QSG_OK;
 }

@@ -41,6 +41,8 @@ struct Group {
     double xi_norm;           // 2 sin(pi / L), host FP64
     unsigned *arrivals;  // [nslots][L_tau/4] boundary arrival counters of the wavefront sweep
     int upb;             // work units per block of the generic wavefront kernel (0 = automatic)
+    uint64_t *scratch;   // correlator scratch of its own (small groups among several), else null
+    size_t scratch_words;
     int *err;            // device status word for waits that gave up (may be null)
 };
 
