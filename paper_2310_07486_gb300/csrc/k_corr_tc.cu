@@ -298,29 +298,46 @@ __device__ __forceinline__ void tmem_ld_oct8(uint32_t taddr, uint32_t (&v)[32]) 
         : "memory");
 }
 
-// Shift the sums v[0 .. N) of a warp one level down a tree over its lanes: add to
-// every lane the sums `from` of lane `src`, whose elements lie at offsets 8 higher
-// where that lane's row wrapped (then its sum k belongs to k + 1).  v[N] is new.
-template <int N, class T>
-__device__ __forceinline__ void fold_level(T (&v)[22], const T (&from)[22], bool wraps, int src) {
+// Shift a warp's sums of both kinds, c[0 .. N) and q[0 .. N), one level down a tree
+// over its lanes: add to every lane the sums (fc, fq) of lane `src`, whose elements
+// lie at offsets 8 higher where that lane's row wrapped (then its sum k belongs to k +
+// 1).  c[N], q[N] are new.  Two sums of each kind at a time: four shuffles in flight
+// (one at a time, the fold took 11,000 cycles a unit, most of them their latency).
+template <int N>
+__device__ __forceinline__ void fold_level(float (&c)[22], int (&q)[22], const float (&fc)[22], const int (&fq)[22],
+                                           bool wraps, int src) {
+    auto sc = [&](int k) { return wraps ? (k > 0 ? fc[k > 0 ? k - 1 : 0] : 0.0f) : (k < N ? fc[k] : 0.0f); };
+    auto sq = [&](int k) { return wraps ? (k > 0 ? fq[k > 0 ? k - 1 : 0] : 0) : (k < N ? fq[k] : 0); };
 #pragma unroll
-    for (int k = N; k >= 0; --k) {
-        const T same = k < N ? from[k < N ? k : 0] : T(0), lower = k > 0 ? from[k > 0 ? k - 1 : 0] : T(0);
-        v[k] = (k < N ? v[k] : T(0)) + __shfl_sync(0xffffffffu, wraps ? lower : same, src);
+    for (int k = N; k >= 0; k -= 2) {
+        const float c0 = __shfl_sync(0xffffffffu, sc(k), src);
+        const int q0 = __shfl_sync(0xffffffffu, sq(k), src);
+        float c1 = 0.0f;
+        int q1 = 0;
+        if (k > 0) {
+            c1 = __shfl_sync(0xffffffffu, sc(k - 1), src);
+            q1 = __shfl_sync(0xffffffffu, sq(k - 1), src);
+        }
+        c[k] = (k < N ? c[k] : 0.0f) + c0;
+        q[k] = (k < N ? q[k] : 0) + q0;
+        if (k > 0) {
+            c[k - 1] += c1;
+            q[k - 1] += q1;
+        }
     }
 }
 
-// The warp's sums of one kind, v[kappa] of column 2 c and w[kappa] of column 2 c + 1
-// of every lane (row r = lane / 4, c = lane % 4), element offset 8 kappa + 2 c + q -
-// r, summed over lanes of equal offset: lane 4 r then holds in v[k] the sum of offset
-// 8 k - r.
-template <class T>
-__device__ __forceinline__ void fold_lanes(T (&v)[22], const T (&w)[22], int lane) {
+// The warp's sums, index kappa of column 2 c (c, q) and of column 2 c + 1 (c1, q1) of
+// every lane (row r = lane / 4, c = lane % 4), element offset 8 kappa + 2 c + q - r,
+// summed over lanes of equal offset: lane 4 r then holds in c[k], q[k] the sums of
+// offset 8 k - r.
+__device__ __forceinline__ void fold_lanes(float (&c)[22], int (&q)[22], const float (&c1)[22], const int (&q1)[22],
+                                           int lane) {
     static_assert(kOct == 19, "levels of 19, 20 and 21 sums");
-    const int r = lane >> 2, c = lane & 3;
-    fold_level<19>(v, w, r < 1, (((r + 1) & 7) << 2) | c);              // q = 1 into q = 0
-    fold_level<20>(v, v, r < 2, (((r + 2) & 7) << 2) | ((c + 1) & 3));  // c odd into c even
-    fold_level<21>(v, v, r < 4, (((r + 4) & 7) << 2) | ((c + 2) & 3));  // c = 2 into c = 0
+    const int r = lane >> 2, l = lane & 3;
+    fold_level<19>(c, q, c1, q1, r < 1, (((r + 1) & 7) << 2) | l);              // second column into first
+    fold_level<20>(c, q, c, q, r < 2, (((r + 2) & 7) << 2) | ((l + 1) & 3));  // odd lanes into even ones
+    fold_level<21>(c, q, c, q, r < 4, (((r + 4) & 7) << 2) | ((l + 2) & 3));
 }
 
 }  // namespace
@@ -491,46 +508,44 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // below 2^24), those of squares need integers
                     const int dbase = kTile * e - 32 * quad - 24 - r;
                     const bool owner = (lane & 3) == 0;
-                    {
-                        float v[22], w[22];
+                    // every offset of the tile is a lag: no tests per element
+                    const bool inside = !un.mirror && kTile * e >= kTile && kTile * e + kTile - 1 <= half;
+                    float vc[22], wc[22];
+                    int vq[22], wq[22];
 #pragma unroll
-                        for (int k = 0; k < 22; ++k) {
-                            v[k] = k < kOct ? accC[k < kOct ? k : 0][0] : 0.0f;
-                            w[k] = k < kOct ? accC[k < kOct ? k : 0][1] : 0.0f;
-                        }
-                        fold_lanes(v, w, lane);
+                    for (int k = 0; k < 22; ++k) {
+                        vc[k] = k < kOct ? accC[k < kOct ? k : 0][0] : 0.0f;
+                        wc[k] = k < kOct ? accC[k < kOct ? k : 0][1] : 0.0f;
+                        vq[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][0]) : 0;
+                        wq[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][1]) : 0;
+                    }
+                    fold_lanes(vc, vq, wc, wq, lane);
+                    if (inside) {
+                        // (sums past the tile's last offset, k > 18, are of nothing)
+#pragma unroll
+                        for (int k = 0; k < 22; ++k)
+                            if (owner && (k <= 18 || dbase + 8 * k <= kTile * e + kTile - 1)) {
+                                atomicAdd(binC + (dbase - lag0) + 8 * k, __float2int_rn(vc[k]));
+                                atomicAdd(binQ + (dbase - lag0) + 8 * k, (unsigned)vq[k]);
+                            }
+                    } else if (owner) {
 #pragma unroll
                         for (int k = 0; k < 22; ++k) {
                             const int d = dbase + 8 * k;
-                            int cv = __float2int_rn(v[k]), lag = d;
+                            int cv = __float2int_rn(vc[k]), lag = d;
+                            unsigned qv = (unsigned)vq[k];
                             if (un.mirror && d >= half) {
                                 // half the row blocks: an element past L_tau / 2 is
                                 // the wrapped pair of lag L_tau - d, and one at
                                 // L_tau / 2 stands for both directions
                                 lag = Lt - d;
+                                if (d == half) qv *= 2u;
                                 cv = d == half ? (g.boundary == 1 ? 0 : 2 * cv) : (g.boundary == 1 ? -cv : cv);
                             }
-                            if (owner && d >= 0 && lag >= lag0 && lag <= half) atomicAdd(&binC[lag - lag0], cv);
-                        }
-                    }
-                    {
-                        int v[22], w[22];
-#pragma unroll
-                        for (int k = 0; k < 22; ++k) {
-                            v[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][0]) : 0;
-                            w[k] = k < kOct ? __float2int_rn(accQ[k < kOct ? k : 0][1]) : 0;
-                        }
-                        fold_lanes(v, w, lane);
-#pragma unroll
-                        for (int k = 0; k < 22; ++k) {
-                            const int d = dbase + 8 * k;
-                            unsigned qv = (unsigned)v[k];
-                            int lag = d;
-                            if (un.mirror && d >= half) {
-                                lag = Lt - d;
-                                if (d == half) qv *= 2u;
+                            if (d >= 0 && lag >= lag0 && lag <= half) {
+                                atomicAdd(&binC[lag - lag0], cv);
+                                atomicAdd(&binQ[lag - lag0], qv);
                             }
-                            if (owner && d >= 0 && lag >= lag0 && lag <= half) atomicAdd(&binQ[lag - lag0], qv);
                         }
                     }
 #pragma unroll

@@ -1,0 +1,167 @@
+"""The forms that the dispatch chooses by size, each against the oracle or against
+the plain kernel, at the sizes where they can go wrong: edges of tiles, chunks and
+row blocks, remainders, the smallest and largest of their range.  Integers bit for
+bit."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import learned as OL
+from paper_2310_07486_gb300 import qsg as Q
+
+pytestmark = pytest.mark.gpu
+
+
+def _context(shape, seed, ladder=None, **options):
+    ctx = Q.Context([shape])
+    ctx.qsg_init_samples(seed, [np.linspace(0.25, 0.35, shape.n_k) if ladder is None else ladder])
+    for name, value in options.items():
+        ctx.qsg_set_option(getattr(Q, "OPT_" + name), value)
+    return ctx
+
+
+@pytest.fixture
+def chunked_sweep():
+    """The fused kernel instead of the resident one where both serve a shape (the
+    kernel form is process-wide: put back afterwards)."""
+    shape = Q.Shape(8, 16, 1, 1, 1)
+    Q.Context([shape]).qsg_set_option(Q.OPT_WAVEFRONT_VARIANT, 1)
+    yield
+    Q.Context([shape]).qsg_set_option(Q.OPT_WAVEFRONT_VARIANT, 0)
+
+
+SMALL = [(2, 2), (2, 6), (4, 34), (6, 32), (8, 48), (10, 200), (12, 100), (14, 146), (16, 110), (22, 58), (28, 18), (32, 26)]
+
+
+@pytest.mark.parametrize("L,Ltau", SMALL)
+@pytest.mark.parametrize("algo,boundary", [(Q.METROPOLIS, Q.APBC), (Q.HEATBATH, Q.PBC)])
+def test_resident_sweeps_match_the_plain_kernel(L, Ltau, algo, boundary):
+    shape = Q.Shape(L, Ltau, 70, 2, 2, algo, boundary)
+    plain, fused = _context(shape, 3, SWEEP_KERNEL=1), _context(shape, 3)
+    for n in (1, 4, 2):
+        plain.qsg_sweep(n)
+        fused.qsg_sweep(n)
+    assert np.array_equal(plain.qsg_get_spins(0), fused.qsg_get_spins(0))
+
+
+@pytest.mark.parametrize("L,Ltau", [(6, 2), (6, 4), (6, 18), (6, 820), (8, 30), (10, 310), (12, 6), (14, 34), (16, 130),
+                                    (18, 1022), (20, 50), (22, 14), (24, 66), (26, 20), (30, 36), (32, 10)])
+@pytest.mark.parametrize("algo,boundary", [(Q.METROPOLIS, Q.PBC), (Q.HEATBATH, Q.APBC)])
+def test_chunked_sweeps_of_any_ltau_match_the_plain_kernel(chunked_sweep, L, Ltau, algo, boundary):
+    shape = Q.Shape(L, Ltau, 70, 1, 2, algo, boundary)
+    plain, fused = _context(shape, 4, SWEEP_KERNEL=1), _context(shape, 4)
+    plain.qsg_sweep(3)
+    fused.qsg_sweep(3)
+    assert np.array_equal(plain.qsg_get_spins(0), fused.qsg_get_spins(0))
+
+
+# short extents (up to 4 words of sites), one and several row blocks, a last offset that
+# is mirrored (L_tau / 2 a whole number of blocks) or not, streamed column blocks (L > 24)
+CORR = [(2, 2), (4, 64), (8, 238), (8, 254), (8, 256), (10, 240), (12, 192), (14, 144), (16, 146), (16, 384), (6, 258),
+        (12, 512), (18, 128), (18, 126), (20, 640), (22, 300), (24, 256), (24, 1024), (26, 512), (32, 256), (30, 130)]
+
+
+@pytest.mark.parametrize("L,Ltau", CORR)
+@pytest.mark.parametrize("boundary", [Q.PBC, Q.APBC])
+def test_correlator_forms_match_the_integer_kernel(L, Ltau, boundary):
+    shape = Q.Shape(L, Ltau, 66, 2, 2, Q.HEATBATH, boundary)
+    got = []
+    for kernel in (Q.CORR_TENSOR, Q.CORR_INTEGER):
+        ctx = _context(shape, 5, CORR_KERNEL=kernel)
+        for _ in range(2):
+            ctx.qsg_sweep(2)
+            ctx.qsg_measure_correlators()
+        got.append(ctx.qsg_read_correlators(0, raw=True))
+    for key in ("C_raw", "Q2_raw", "q2_raw"):
+        assert np.array_equal(got[0][key], got[1][key]), key
+
+
+def test_frozen_spins_reach_the_largest_correlator_sums():
+    """All spins equal: every Gram element is L^2, the largest of every running sum."""
+    shape = Q.Shape(24, 2048, 1, 2, 1, Q.HEATBATH, Q.PBC)
+    ctx = _context(shape, 6)
+    ctx.qsg_set_spins(0, np.zeros((shape.slots, shape.Ltau, 24, 24), dtype=np.uint64))
+    ctx.qsg_measure_correlators()
+    got = ctx.qsg_read_correlators(0, raw=True)
+    assert np.all(got["C_raw"] == 2048 * 576) and np.all(got["Q2_raw"] == 2048 * 576 ** 2)
+
+
+@pytest.mark.parametrize("spacing", [2e-4, 3e-2])
+def test_tempering_tables_beyond_their_shared_heads_match_oracle(spacing):
+    """A fine ladder (table entries past those held in shared memory) and a coarse one."""
+    shape = Q.Shape(12, 64, 70, 2, 5, Q.METROPOLIS, Q.PBC)
+    ladder = 0.3 + spacing * np.arange(5)
+    ctx = _context(shape, 7, ladder)
+    orc = oracle.OracleGroup(12, 64, 70, 2, 5, algo="metropolis")
+    orc.init(7, ladder)
+    for _ in range(3):
+        ctx.qsg_sweep(1)
+        orc.sweep(1)
+        ctx.qsg_tempering_swap()
+        orc.swap()
+    assert np.array_equal(Q.unpack_spins(ctx.qsg_get_spins(0), shape), orc.spins())
+    assert np.array_equal(ctx.qsg_read_accepts(0), orc.accepts())
+
+
+def test_overlapped_groups_equal_groups_in_turn():
+    """Tempering and measurements of groups with and without a scratch of their own, on
+    side streams and one after another."""
+    shapes = [Q.Shape(8, 48, 70, 3, 4, Q.HEATBATH, Q.PBC), Q.Shape(24, 512, 64, 4, 12, Q.HEATBATH, Q.APBC),
+              Q.Shape(12, 64, 64, 4, 6, Q.HEATBATH, Q.PBC), Q.Shape(16, 256, 64, 2, 3, Q.HEATBATH, Q.PBC)]
+    ladders = [np.linspace(0.25, 0.3, s.n_k) for s in shapes]
+    got = []
+    for mode in (1, 3):
+        ctx = Q.Context(shapes)
+        ctx.qsg_init_samples(9, ladders)
+        ctx.qsg_set_option(Q.OPT_PERSISTENT, mode)
+        for _ in range(3):
+            ctx.qsg_sweep(2)
+            ctx.qsg_tempering_swap()
+            ctx.qsg_measure_correlators()
+        got.append([(ctx.qsg_get_spins(g), ctx.qsg_read_correlators(g, raw=True), ctx.qsg_read_onetime(g)["raw"],
+                     ctx.qsg_read_accepts(g), ctx.qsg_read_energies(g)) for g in range(len(shapes))])
+    for a, b in zip(*got):
+        assert np.array_equal(a[0], b[0])
+        assert all(np.array_equal(a[1][k], b[1][k]) for k in a[1])
+        assert all(np.array_equal(x, y) for x, y in zip(a[2:], b[2:]))
+
+
+@pytest.mark.parametrize("L,Ltau,R", [(2, 4, 3), (14, 34, 8), (24, 66, 6), (26, 40, 4), (32, 130, 8)])
+def test_onetime_sums_of_many_replicas_match_oracle(L, Ltau, R):
+    shape = Q.Shape(L, Ltau, 3, R, 1, Q.METROPOLIS, Q.PBC)
+    lad = np.array([0.3])
+    ctx = _context(shape, 8, lad)
+    orc = oracle.OracleGroup(L, Ltau, 3, R, 1, algo="metropolis")
+    orc.init(8, lad)
+    ctx.qsg_measure_correlators()
+    orc.measure()
+    assert np.array_equal(ctx.qsg_read_onetime()["raw"], orc.read_onetime()["raw"])
+
+
+@pytest.mark.parametrize("n", [1, 608, 609, 3000])
+def test_prediction_tiles_match_oracle(n):
+    X = np.random.default_rng(n).random((n, 64), dtype=np.float32)
+    theta = OL.init_params(3)
+    m = Q.MLP(n, 16)
+    m.set_params(theta)
+    ref, e, _ = OL.fp32_forward_bound(theta.astype(np.float64), X)
+    assert np.all(np.abs(m.predict(X, bf16=False).astype(np.float64) - ref) <= e)
+
+
+@pytest.mark.parametrize("batch", [15, 3000])
+def test_training_steps_of_one_call_equal_single_calls(batch):
+    """257 steps (two launches) for a small batch; more tiles than SMs for a large one."""
+    rng = np.random.default_rng(batch)
+    X = rng.random((3000, 64), dtype=np.float32)
+    T = np.full((3000, 33), 1.0 / 32, dtype=np.float32)
+    steps = 257 if batch < 100 else 3
+    idx = rng.integers(0, 3000, size=(steps, batch)).astype(np.int32)
+    params, losses = [], []
+    for cuts in ([0, steps], [0, 1, 2, steps]):
+        m = Q.MLP(3000, batch)
+        m.set_params(OL.init_params(4))
+        m.set_data(X, T)
+        losses.append(np.concatenate([m.train(idx[a:b], 1e-3) for a, b in zip(cuts, cuts[1:])]))
+        params.append(m.get_params())
+    assert np.array_equal(losses[0], losses[1]) and np.array_equal(params[0], params[1])
+    assert np.all(np.isfinite(params[0]))
