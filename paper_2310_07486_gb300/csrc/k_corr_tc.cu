@@ -22,7 +22,7 @@
 // kind cover its 128 elements of a tile.  (The form before this one ordered
 // the tiles by row block and folded every tile with two shared-memory atomics
 // per element: 3.92 ms for 2,048 sample bits at L = 24, L_tau = 2048, where
-// this one takes 2.57 ms.)  The wrap past L_tau is taken where the rows
+// this one takes 2.31 ms.)  The wrap past L_tau is taken where the rows
 // are loaded: the row of t2 >= L_tau is that of t2 - L_tau, with its sign
 // flipped under APBC, so C needs no sign in the epilogue.
 //
@@ -42,11 +42,13 @@
 //     step) reads the accumulators, double-buffered in tensor memory.
 // Per step of two tiles at L = 24 the MMAs read 216 KB and the producers write 144
 // KB of shared memory (2,880 cycles at 128 B per cycle) beside 2,304 cycles of
-// tensor work; measured, a step takes 5,200: the producers' expansion (470 cycles a
-// chunk, 740 with its fences and hand-over) and the MMA thread's waits alternate
-// more than they overlap in the three chunks that fit in flight.  Lattices of L > 22..24 whose two
-// resident column blocks do not fit (more than five chunks) take every offset
-// as a unit of its own, both operands streamed.
+// tensor work; measured, a step takes 4,700.  The MMAs alone, without waits, run at
+// 2,300 (1.16 ms for the batch above); with the hand-over but neither expansion nor
+// reads 2.02 ms, so most of what is left is the hand-over of chunks between the
+// roles.  A fourth chunk in flight (both slots' half-empty last chunks in one) did not
+// help, nor did one polling lane per warp (6.7 ms).  Lattices of more than five chunks
+// (L > 24), whose column blocks do not fit, take every offset as a unit of its own,
+// both operands streamed.
 #include "qsg_launch.h"
 
 namespace qsg {
@@ -80,16 +82,14 @@ constexpr unsigned kSpinLimit = 1u << 22;    // polls of the wait for issued MMA
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
+// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B
+// apart.  Its upper half is constant; the lower half is the address / 16 (below 2^14)
+// and a constant, so a step along K or to another chunk is one 32-bit addition.  (With
+// 64-bit descriptors built per MMA the issuing thread was late: 2,507 -> 2,313 us at L =
+// 24, L_tau = 2048, 665 -> 622 us at L = 20, L_tau = 1024, 576 -> 562 us at L = 16, L_tau =
+// 512.)
+constexpr uint32_t kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_low(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
 
 // Instruction descriptor: D = FP32, A = B = E4M3, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t idesc_e4m3(int n) {
@@ -191,10 +191,10 @@ __device__ __forceinline__ void expand_word(uint8_t *rowp, uint64_t wv, int vali
         expand_part(rowp, wv, valid, hh, row, one);
 }
 
-__device__ __forceinline__ void mma_f8(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-                 "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                 "l"(da), "l"(db), "r"(idesc), "r"(acc));
+__device__ __forceinline__ void mma_f8(uint32_t d, uint32_t da, uint32_t db, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n.reg .pred p;\n.reg .b64 a, b;\nmov.b64 a, {%1, %5};\nmov.b64 b, {%2, %5};\nsetp.ne.u32 p, %4, 0;\n"
+                 "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], a, b, %3, p;\n}\n" ::"r"(d),
+                 "r"(da), "r"(db), "r"(idesc), "r"(acc), "r"(kDescHigh));
 }
 
 // How the offsets of one sample are cut into units and steps.
@@ -581,7 +581,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             // hold a lattice site (the bit-interleaved order spreads a word's
             // sites over its whole 64-byte span)
             const int nk_last = min(kChunk / 32, 2 * ((L2 - (NC - 1) * kChunk + 63) / 64));
-            const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+            constexpr uint32_t kC = kChunkBytes / 16;  // a chunk in descriptor units
+            const uint32_t sA0 = desc_low(smem_u32(sA)), sB0 = desc_low(smem_u32(sB));
             uint32_t par = 0u, n_t = 0;
             int st = 0, slot = 0, older = NS - 1;  // slots of the step's new column block and of the one before
             bool issued = false;
@@ -599,27 +600,33 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // N = 128 MMA per column block, the older block's first
                     const uint32_t idesc = un.pair && NS == 2 ? id256 : id128;
                     const uint32_t b0 =
-                        un.pair ? (NS == 2 ? 0u : (uint32_t)(older * kChunkBytes)) : (uint32_t)(slot * kChunkBytes);
-                    const uint32_t b1 = (uint32_t)(slot * kChunkBytes);
+                        un.pair ? (NS == 2 ? 0u : (uint32_t)older * kC) : (uint32_t)slot * kC;
+                    const uint32_t b1 = (uint32_t)slot * kC;
                     const bool second = un.pair && NS > 2;
 #pragma unroll 1  // rolled: the three roles' code shares the instruction cache
                     for (int kc = 0; kc < NC; ++kc) {
                         ok = mbar_wait(&ctl.full[st], par, &ctl.abort, wait_limit) && ok;
                         asm volatile("tcgen05.fence::after_thread_sync;\n");
                         if (ok && i >= 0) {
-                            const uint32_t ab = sA0 + st * kChunkBytes;
-                            const uint32_t bb = RESIDENT ? sB0 + NS * kc * kChunkBytes : sB0 + st * kChunkBytes;
+                            const uint32_t ab = sA0 + (uint32_t)st * kC;
+                            const uint32_t bb = RESIDENT ? sB0 + (uint32_t)(NS * kc) * kC : sB0 + (uint32_t)st * kC;
                             const uint32_t bb0 = RESIDENT ? bb + b0 : bb;
                             const int nk = kc == NC - 1 ? nk_last : kChunk / 32;
-#pragma unroll
-                            for (int kk = 0; kk < kChunk / 32; ++kk)
-                                if (kk < nk) {
-                                    mma_f8(d, sdesc_sw128(ab + kk * 32), sdesc_sw128(bb0 + kk * 32), idesc,
-                                           (kc > 0 || kk > 0) ? 1u : 0u);
-                                    if (NS > 2 && second)
-                                        mma_f8(d + kTile, sdesc_sw128(ab + kk * 32), sdesc_sw128(bb + b1 + kk * 32),
-                                               id128, (kc > 0 || kk > 0) ? 1u : 0u);
+                            const uint32_t acc0 = kc > 0 ? 1u : 0u;
+                            mma_f8(d, ab, bb0, idesc, acc0);
+                            mma_f8(d, ab + 2u, bb0 + 2u, idesc, 1u);
+                            if (nk > 2) {
+                                mma_f8(d, ab + 4u, bb0 + 4u, idesc, 1u);
+                                mma_f8(d, ab + 6u, bb0 + 6u, idesc, 1u);
+                            }
+                            if (NS > 2 && second) {
+                                mma_f8(d + kTile, ab, bb + b1, id128, acc0);
+                                mma_f8(d + kTile, ab + 2u, bb + b1 + 2u, id128, 1u);
+                                if (nk > 2) {
+                                    mma_f8(d + kTile, ab + 4u, bb + b1 + 4u, id128, 1u);
+                                    mma_f8(d + kTile, ab + 6u, bb + b1 + 6u, id128, 1u);
                                 }
+                            }
                             issued = true;
                         }
                         mma_commit(&ctl.empty[st]);
