@@ -327,23 +327,25 @@ qsg_status qsg_get_counters(qsg_ctx *ctx, uint32_t *sweeps, uint32_t *swaps, int
 qsg_status qsg_set_counters(qsg_ctx *ctx, uint32_t sweeps, uint32_t swaps, int64_t n_meas);
 
 /* Tuning options (apply to every group of the context):
- *   QSG_OPT_SWEEP_KERNEL  0 = automatic, 1 = one thread per site and colour
- *                         (two launches per sweep), 2 = fused tau-wavefront
- *                         (one launch per sweep; needs L_tau % 16 == 0)
+ *   QSG_OPT_SWEEP_KERNEL  0 = automatic (several sweeps per launch with the
+ *                         slot in shared memory where it fits, else the
+ *                         fused wavefront for any L_tau), 1 = one thread per
+ *                         site and colour (two launches per sweep), 2 = fused
+ *                         tau-wavefront (one launch per sweep; needs
+ *                         L_tau % 16 == 0)
  *   QSG_OPT_CHUNK         tau planes per wavefront work unit (0 = automatic;
  *                         otherwise a multiple of 16 that divides every L_tau)
- *   QSG_OPT_WAVEFRONT_VARIANT  form of the wavefront kernel, process-wide:
- *                         0 = one work unit per block with L compiled in
- *                         (L = 8, 12, 16, 20, 24; 72 registers, three blocks of 288
- *                         threads per SM at L = 24), four tau planes per
- *                         block barrier; other L use the
- *                         generic kernel;
- *                         1 = the same with two planes per barrier; 3 = with
- *                         four; 2 = the generic kernel (several units per
- *                         block, L at run time, two blocks per SM)
- *   QSG_OPT_CORR_KERNEL   0 = tensor cores (Gram tiles by tcgen05.mma in FP8,
- *                         exact for +-1 spins), 1 = XOR/popcount on the
- *                         integer pipes
+ *   QSG_OPT_WAVEFRONT_VARIANT  form of the fused sweep, process-wide:
+ *                         0 = automatic; 1, 3 = the wavefront with L compiled
+ *                         in (L = 6 .. 32; 72 registers, three blocks of 288
+ *                         threads per SM at L = 24) also where a slot fits
+ *                         shared memory; 2 = the generic wavefront (several
+ *                         units per block, L at run time, two blocks per SM)
+ *   QSG_OPT_CORR_KERNEL   0 = automatic: tensor cores (Gram tiles by
+ *                         tcgen05.mma in FP8, exact for +-1 spins), short
+ *                         extents of tau (below 256) of small lattices on
+ *                         the integer pipes; 1 = the plain XOR/popcount
+ *                         kernel
  *   QSG_OPT_PERSISTENT    how the groups of a context are swept:
  *                         0 = automatic (mode 3 when the context has several
  *                         groups), 1 = one launch per group and sweep, in
@@ -355,14 +357,15 @@ qsg_status qsg_set_counters(qsg_ctx *ctx, uint32_t sweeps, uint32_t swaps, int64
  *                         and joined back into the context's stream (inside
  *                         the CUDA graph when QSG_OPT_GRAPH is on), so that
  *                         the groups' launches overlap and small groups fill
- *                         the last waves of large ones
+ *                         the last waves of large ones; tempering steps and
+ *                         the measurements of small groups overlap likewise
  *   QSG_OPT_GRAPH         0 = off; G in 1..4096 = qsg_sweep replays a CUDA
  *                         graph of G sweeps (captured on first use and again
  *                         after an option change) for each whole batch of G,
  *                         and launches the remainder directly.  The graph
  *                         reads the sweep index from a device counter, so
  *                         its Philox draws equal those of direct launches.
- *                         Needs the wavefront kernel for every group.
+ *                         Needs L_tau % 16 == 0 in every group.
  *   QSG_OPT_ONETIME       0 = accumulate every one-time sum (default),
  *                         1 = skip the three-replica sums (chi3, F3 become
  *                         NaN); only before the first measurement
@@ -383,8 +386,7 @@ qsg_status qsg_set_counters(qsg_ctx *ctx, uint32_t sweeps, uint32_t swaps, int64
  *                         small value is a way to exercise that path; the
  *                         default never gives up on a working GPU.
  *   QSG_OPT_UNITS_PER_BLOCK  work units (slot, tau chunk) per thread block of
- *                         the generic wavefront kernel, which serves the
- *                         lattice sizes without a compiled kernel: 0 =
+ *                         the generic wavefront kernel (variant 2): 0 =
  *                         automatic (as many as fit 256 threads, at most 16),
  *                         or 1, 2, 4, 8, 16 (rounded down to at most 512
  *                         threads).  A unit's thread owns two site words of
