@@ -25,6 +25,7 @@ using namespace sweep;
 using namespace unit;
 
 constexpr size_t kSlotLimit = 226 * 1024;  // bytes of a slot that fit beside the static barrier
+constexpr long long kLaunchWords = 1ll << 36;  // site-word updates of a launch at most (about 0.25 s)
 
 // A value the compiler knows nothing about: keeps it from carrying the addresses
 // of every plane pair from one half sweep to the next in registers (they spilled).
@@ -177,8 +178,16 @@ cudaError_t launch_sweep_resident(const Group &g, int count, const uint32_t *swe
     const ResidentShape r = resident_shape(g, nsm);
     const int threads = r.rows * (g.L * g.L / 2);
     if (threads > 1024) return cudaErrorInvalidValue;
-    return g.algo == 0 ? launch_ip<0>(r.ip, g, threads, sm, count, sweep_base, sweep, seed, st)
-                       : launch_ip<1>(r.ip, g, threads, sm, count, sweep_base, sweep, seed, st);
+    // launches of a bounded length, however many sweeps are asked for
+    const long long most = kLaunchWords / ((long long)g.nslots * (long long)g.N);
+    for (int done = 0; done < count && e == cudaSuccess;) {
+        const int n = most < 1 ? 1 : (int)(most < count - done ? most : count - done);
+        const uint32_t first = sweep + (uint32_t)done;
+        e = g.algo == 0 ? launch_ip<0>(r.ip, g, threads, sm, n, sweep_base, first, seed, st)
+                        : launch_ip<1>(r.ip, g, threads, sm, n, sweep_base, first, seed, st);
+        done += n;
+    }
+    return e;
 }
 
 }  // namespace qsg

@@ -44,6 +44,18 @@ def test_resident_sweeps_match_the_plain_kernel(L, Ltau, algo, boundary):
     assert np.array_equal(plain.qsg_get_spins(0), fused.qsg_get_spins(0))
 
 
+def test_long_calls_of_resident_sweeps_are_cut():
+    """2^36 site-word updates per launch: 16,644 sweeps of 4.1 M words here."""
+    shape = Q.Shape(8, 48, 64, 42, 32, Q.HEATBATH, Q.PBC)
+    whole, halves = _context(shape, 5), _context(shape, 5)
+    before = Q.qsg_kernel_launches()
+    whole.qsg_sweep(17000)
+    assert Q.qsg_kernel_launches() == before + 2
+    for n in (16000, 1000):
+        halves.qsg_sweep(n)
+    assert np.array_equal(whole.qsg_get_spins(0), halves.qsg_get_spins(0))
+
+
 @pytest.mark.parametrize("L,Ltau", [(6, 2), (6, 4), (6, 18), (6, 820), (8, 30), (10, 310), (12, 6), (14, 34), (16, 130),
                                     (18, 1022), (20, 50), (22, 14), (24, 66), (26, 20), (30, 36), (32, 10)])
 @pytest.mark.parametrize("algo,boundary", [(Q.METROPOLIS, Q.PBC), (Q.HEATBATH, Q.APBC)])
