@@ -30,7 +30,7 @@ struct Range {
 constexpr size_t kAlign = 256;
 constexpr int kMaxA = 16384;               // longest A_i table of the tempering test
 constexpr size_t kOwnScratch = 64u << 20;  // largest whole correlator scratch of a group that gets its own
-constexpr size_t kScratchCap = 1024u << 20;  // bytes of correlator scratch (transposed bits, E4M3 rows)
+constexpr size_t kScratchCap = 1024u << 20;  // bytes of correlator scratch (transposed bits); of the groups' own, too
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -87,7 +87,8 @@ size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, 
         return p;
     };
     *err = (int *)take(sizeof(int) * 4);
-    size_t sw = 0;
+    size_t sw = 0;   // words of the shared scratch
+    size_t own = 0;  // bytes of the groups' own
     const bool several = gs.size() > 1;
     for (auto &g : gs) {
         g.S = (uint64_t *)take(sizeof(uint64_t) * (size_t)g.nslots * g.N);
@@ -126,12 +127,14 @@ size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, 
         const size_t all = per * (size_t)g.W * g.K;
         if (want > all) want = all;
         // a small group among several has a scratch of its own, so that the
-        // measurements of small groups can overlap; the others share one
+        // measurements of small groups can overlap (up to the cap in all); the
+        // others share one
         g.scratch = nullptr;
         g.scratch_words = 0;
-        if (several && all * sizeof(uint64_t) <= kOwnScratch) {
+        if (several && all * sizeof(uint64_t) <= kOwnScratch && own + all * sizeof(uint64_t) <= kScratchCap) {
             g.scratch = (uint64_t *)take(sizeof(uint64_t) * all);
             g.scratch_words = all;
+            own += all * sizeof(uint64_t);
             want = 0;
         }
         // the scratch also holds the coupling features, [W*64][64] float
