@@ -19,7 +19,7 @@ constexpr int kMaxBatch = 4096;
 size_t up(size_t v) { return (v + kAlignM - 1) / kAlignM * kAlignM; }
 
 struct Layout {
-    float *P, *M, *V, *grad, *partial, *lossp, *losses, *corr, *X, *T, *Xp, *Yp;
+    float *P, *M, *V, *grad, *act, *losses, *corr, *X, *T, *Xp, *Yp;
     int *idx;
     unsigned *sync;  // grid-barrier count and status of the training launch
 };
@@ -32,14 +32,12 @@ size_t carve_mlp(char *base, long long n_data, int max_batch, Layout *l) {
         return p;
     };
     const size_t np = (size_t)mlp_param_count();
-    const size_t tiles = (size_t)(max_batch + 15) / 16;
     Layout t;
     t.P = (float *)take(np * 4);
     t.M = (float *)take(np * 4);
     t.V = (float *)take(np * 4);
     t.grad = (float *)take(np * 4);
-    t.partial = (float *)take(tiles * np * 4);
-    t.lossp = (float *)take(tiles * 4);
+    t.act = (float *)take(mlp_act_words(max_batch) * 4);
     t.losses = (float *)take((size_t)kChunk * 4);
     t.corr = (float *)take((size_t)kChunk * 2 * 4);
     t.sync = (unsigned *)take(2 * sizeof(unsigned));
@@ -144,8 +142,8 @@ qsg_status qsg_mlp_grad(qsg_mlp *m, const int32_t *idx, int32_t batch, float *lo
     if (!m->has_params || m->n_loaded == 0) return QSG_ERR_STATE;
     qsg_status s = upload_idx(m, idx, (size_t)batch);
     if (s != QSG_OK) return s;
-    MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, 1, batch, m->l.partial, m->l.lossp,
-                              m->l.grad, 0, 0.0f, m->l.corr, m->l.losses, m->l.sync, m->st));
+    MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, 1, batch, m->l.act, m->l.grad,
+                              0, 0.0f, m->l.corr, m->l.losses, m->l.sync, m->st));
     if (grad_host)
         MLP_CUDA(cudaMemcpyAsync(grad_host, m->l.grad, (size_t)mlp_param_count() * 4, cudaMemcpyDeviceToHost, m->st));
     float l = 0.0f;
@@ -170,8 +168,8 @@ qsg_status qsg_mlp_train(qsg_mlp *m, const int32_t *idx, int32_t steps, int32_t 
             corr[2 * i + 1] = (float)(1.0 - std::pow(0.999, (double)m->step));
         }
         MLP_CUDA(cudaMemcpyAsync(m->l.corr, corr, sizeof(float) * 2 * nc, cudaMemcpyHostToDevice, m->st));
-        MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, nc, batch, m->l.partial,
-                                  m->l.lossp, nullptr, 1, lr, m->l.corr, m->l.losses, m->l.sync, m->st));
+        MLP_CUDA(launch_mlp_steps(m->l.P, m->l.M, m->l.V, m->l.X, m->l.T, m->l.idx, nc, batch, m->l.act,
+                                  nullptr, 1, lr, m->l.corr, m->l.losses, m->l.sync, m->st));
         if (losses) MLP_CUDA(cudaMemcpyAsync(losses + c0, m->l.losses, (size_t)nc * 4, cudaMemcpyDeviceToHost, m->st));
         // the index buffer is reused by the next chunk
         s = finish_steps(m);

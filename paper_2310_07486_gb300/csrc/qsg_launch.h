@@ -103,15 +103,16 @@ size_t measure_scratch_words_per_pair(const Group &g);
 cudaError_t launch_features(const Group &g, float *out, cudaStream_t st);
 
 // Learned-ladder MLP (k_mlp.cu).  P: FP32 parameters, M, V: Adam moments;
-// `steps` steps over the batches idx[steps][batch] (tiles of 16 samples into
-// `partial`), Adam's bias corrections in corr[steps][2]; adam = 0 only writes
+// `steps` steps over the batches idx[steps][batch] (activations and dL/dz in act,
+// mlp_act_words(batch) floats), Adam's bias corrections in corr[steps][2]; adam = 0 only writes
 // the gradient to grad_out (device, may be null).  loss_out: [steps] (device);
 // sync: two device words, the second a status (DEVERR_TIMEOUT after a bounded
-// grid wait gave up).  X, T and P are 16-byte aligned.
+// grid wait gave up).  X, T, P and act are 16-byte aligned.
 int mlp_param_count();
+size_t mlp_act_words(int batch);
 cudaError_t launch_mlp_steps(float *P, float *M, float *V, const float *X, const float *T, const int *idx, int steps,
-                             int batch, float *partial, float *loss_partial, float *grad_out, int adam, float lr,
-                             const float *corr, float *loss_out, unsigned *sync, cudaStream_t st);
+                             int batch, float *act, float *grad_out, int adam, float lr, const float *corr,
+                             float *loss_out, unsigned *sync, cudaStream_t st);
 cudaError_t launch_mlp_infer(const float *P, const float *X, float *Y, long long n, int bf16, cudaStream_t st);
 
 }  // namespace qsg
