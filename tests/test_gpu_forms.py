@@ -138,6 +138,18 @@ def test_overlapped_groups_equal_groups_in_turn():
         assert all(np.array_equal(x, y) for x, y in zip(a[2:], b[2:]))
 
 
+@pytest.mark.parametrize("L,Ltau,n_meas", [(2, 4, 1), (6, 34, 3), (14, 70, 7), (22, 258, 5), (32, 26, 49)])
+def test_finish_rounds_like_one_division(L, Ltau, n_meas):
+    ctx = _context(Q.Shape(L, Ltau, 70, 3, 2, Q.HEATBATH, Q.APBC), 15)
+    for _ in range(n_meas):
+        ctx.qsg_sweep(1)
+        ctx.qsg_measure_correlators()
+    got = ctx.qsg_read_correlators(0, raw=True)
+    n, L2 = float(n_meas), float(L * L)
+    assert np.array_equal(got["C"], got["C_raw"].astype(float) / (n * L2 * Ltau))
+    assert np.array_equal(got["Q2"], got["Q2_raw"].astype(float) / (n * L2 * L2 * Ltau))
+
+
 @pytest.mark.parametrize("L,Ltau,R", [(2, 4, 3), (14, 34, 8), (24, 66, 6), (26, 40, 4), (32, 130, 8)])
 def test_onetime_sums_of_many_replicas_match_oracle(L, Ltau, R):
     shape = Q.Shape(L, Ltau, 3, R, 1, Q.METROPOLIS, Q.PBC)
