@@ -511,8 +511,30 @@ static qsg_status on_side_streams(qsg_ctx *ctx, cudaStream_t st, Side side, Work
 }
 }  // extern "C++"
 
+// A resident slot is the work of one SM, so few large slots leave the others idle,
+// where chunks spread over all of them.  Measured, us per sweep: resident 0.55 per
+// 1,000 words of a slot and round of one slot per SM, chunked 5 + 6.2 per million
+// words, at least 9.3.  Resident / chunked: L = 12, L_tau = 128, 8 slots 10.8 / 9.4; L =
+// 8, L_tau = 448, 16 slots 14.7 / 9.5; L = 12, L_tau = 192, 30 slots 14.5 / 12.4; but L =
+// 8, L_tau = 256, 80 slots 8.8 / 12.2; L = 14, L_tau = 144, 64 slots 15.2 / 17.0; L = 12,
+// L_tau = 128, 160 slots 21.3 / 23.2.
+static bool few_large_slots(const Group &g) {
+    static std::atomic<int> sms{0};
+    int n = sms.load(std::memory_order_relaxed);
+    if (n == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+            return false;
+        sms.store(n, std::memory_order_relaxed);
+    }
+    const double resident = 0.55e-3 * (double)g.N * (double)((g.nslots + n - 1) / n);
+    const double chunked = 5.0 + 6.2e-6 * (double)g.N * (double)g.nslots;
+    return resident > (chunked > 9.3 ? chunked : 9.3);
+}
+
 // Several sweeps of a group in one launch, the slots in shared memory: where a
-// slot fits an SM and no launch option asks for another form.  A graph of fewer
+// slot fits an SM, the slots keep the SMs busy and no launch option asks for another form.  A graph of fewer
 // than kResidentGraphSlots slots keeps one kernel node per sweep: such a replay
 // leaves the GPU idle either way, and its launch count is part of what callers
 // see (qsg_kernel_launches).
@@ -520,7 +542,7 @@ constexpr int kResidentGraphSlots = 8;
 static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
     if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
     if (sb && g.nslots < kResidentGraphSlots) return false;
-    return sweep_resident_fits(g);
+    return sweep_resident_fits(g) && !(sweep_unit_supported(g) && few_large_slots(g));
 }
 
 // `count` sweeps of one group on one stream, indices first .. first + count - 1

@@ -35,8 +35,10 @@ SMALL = [(2, 2), (2, 6), (4, 34), (6, 32), (8, 48), (10, 200), (12, 100), (14, 1
 
 @pytest.mark.parametrize("L,Ltau", SMALL)
 @pytest.mark.parametrize("algo,boundary", [(Q.METROPOLIS, Q.APBC), (Q.HEATBATH, Q.PBC)])
-def test_resident_sweeps_match_the_plain_kernel(L, Ltau, algo, boundary):
-    shape = Q.Shape(L, Ltau, 70, 2, 2, algo, boundary)
+@pytest.mark.parametrize("K", [2, 20])
+def test_resident_sweeps_match_the_plain_kernel(L, Ltau, algo, boundary, K):
+    """20 ladder values make 80 slots, which stay resident; few large slots are chunked."""
+    shape = Q.Shape(L, Ltau, 70, 2, K, algo, boundary)
     plain, fused = _context(shape, 3, SWEEP_KERNEL=1), _context(shape, 3)
     for n in (1, 4, 2):
         plain.qsg_sweep(n)
