@@ -330,9 +330,9 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     for (int m0 = 0; m0 < M; m0 += 4) {
         if (m0 == 0 || 4 * (m0 + 3) + 5 > Cmin) {
             step(m0, std::integral_constant<int, 0>{}, std::true_type{});
-            step(m0 + 1, std::integral_constant<int, 1>{}, std::true_type{});
-            step(m0 + 2, std::integral_constant<int, 2>{}, std::true_type{});
-            step(m0 + 3, std::integral_constant<int, 3>{}, std::true_type{});
+            if (P > 1 || m0 + 1 < M) step(m0 + 1, std::integral_constant<int, 1>{}, std::true_type{});
+            if (P > 1 || m0 + 2 < M) step(m0 + 2, std::integral_constant<int, 2>{}, std::true_type{});
+            if (P > 1 || m0 + 3 < M) step(m0 + 3, std::integral_constant<int, 3>{}, std::true_type{});
         } else {
             step(m0, std::integral_constant<int, 0>{}, std::false_type{});
             step(m0 + 1, std::integral_constant<int, 1>{}, std::false_type{});
@@ -340,7 +340,10 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
             step(m0 + 3, std::integral_constant<int, 3>{}, std::false_type{});
         }
     }
-    const int Mr = (M + 3) / 4 * 4;  // steps run
+    // steps run: no more than the planes need (up to three idle ones cost 3 % at L = 24,
+    // L_tau = 2048, 1,005 -> 970 us, 10 % at L = 16, L_tau = 512, 96 slots, 55 -> 50 us; with
+    // several chunks per block the checks cost more than they save)
+    const int Mr = P > 1 ? (M + 3) / 4 * 4 : M;
     fence_async_smem();
     __syncthreads();
     const int chn = ch + 1 == nu ? 0 : ch + 1;  // the chunk after the last is the first
