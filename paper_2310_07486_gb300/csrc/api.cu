@@ -545,6 +545,16 @@ static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb)
     return sweep_resident_fits(g) && !(sweep_unit_supported(g) && few_large_slots(g));
 }
 
+// Very few words without a graph: the plain kernel's two short launches take less
+// than a chunk's chain of steps.  us per sweep, plain / chunked: L = 12, L_tau = 330, 2
+// slots 8.3 / 12.4; L = 24, L_tau = 100, 6 slots 12.4 / 14.7; L = 8, L_tau = 700, 8 slots 12.4
+// / 12.4; L = 6 (16 chunks per block in lockstep), L_tau = 820, 16 slots 16.5 / 22.6, 120
+// slots 62 / 38.  For L_tau a multiple of 16, which the graphs take, chunks as ever.
+static bool plain_pays(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
+    if (sb || ctx->sweep_kernel != 0 || g_wavefront_variant != 0 || g.Ltau % 16 == 0) return false;
+    return (double)g.N * (double)g.nslots < (g.L == 6 ? 1.5e6 : 4e5);
+}
+
 // `count` sweeps of one group on one stream, indices first .. first + count - 1
 // (added to *sb when sb is given).
 static qsg_status group_sweeps(qsg_ctx *ctx, const Group &g, const uint32_t *sb, uint32_t first, int count,
@@ -553,7 +563,7 @@ static qsg_status group_sweeps(qsg_ctx *ctx, const Group &g, const uint32_t *sb,
         QSG_CUDA(ctx, launch_sweep_resident(g, count, sb, first, ctx->seed, st));
         return QSG_OK;
     }
-    const bool fused = ctx->sweep_kernel != 1 && sweep_fused_supported(g, ctx->chunk);
+    const bool fused = ctx->sweep_kernel != 1 && sweep_fused_supported(g, ctx->chunk) && !plain_pays(ctx, g, sb);
     if (!fused && sb) return QSG_ERR_ARG;  // the reference kernel takes its index by value only
     for (int i = 0; i < count; ++i) {
         const uint32_t idx = first + (uint32_t)i;
