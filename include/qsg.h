@@ -375,16 +375,20 @@ qsg_status qsg_set_counters(qsg_ctx *ctx, uint32_t sweeps, uint32_t swaps, int64
  *                         quarter of the chunk length (when that is a multiple
  *                         of 16), scheduled after all other units, so that
  *                         short units fill the last wave of blocks
- *   QSG_OPT_WAIT_LIMIT    polls of each bounded device wait of the tensor-core
- *                         correlator pipeline before it gives up (default
- *                         2^22, 0..2^30).  A wait that gives up makes every
- *                         role of the kernel run out its loops without
- *                         further work and sets the context's device flag:
- *                         that measurement is not accumulated, and
- *                         qsg_read_correlators returns QSG_ERR_TIMEOUT from
- *                         then on (the flag stays set for the context).  A
- *                         small value is a way to exercise that path; the
- *                         default never gives up on a working GPU.
+ *   QSG_OPT_WAIT_LIMIT    polls of each bounded device wait before it gives up
+ *                         (default 2^22, 0..2^30): the waits of the
+ *                         tensor-core correlator pipeline and those of the
+ *                         sweeps for their bulk copies.  A wait that gives up
+ *                         sets the context's device flag.  In the correlator
+ *                         kernel every role then runs out its loops without
+ *                         further work and that measurement is not
+ *                         accumulated; in a sweep the block starts no further
+ *                         copy, so planes it had not yet written stay as they
+ *                         were.  qsg_read_correlators returns
+ *                         QSG_ERR_TIMEOUT from then on (the flag stays set
+ *                         for the context).  A small value is a way to
+ *                         exercise that path; the default never gives up on a
+ *                         working GPU.
  *   QSG_OPT_UNITS_PER_BLOCK  work units (slot, tau chunk) per thread block of
  *                         the generic wavefront kernel (variant 2): 0 =
  *                         automatic (as many as fit 256 threads, at most 16),

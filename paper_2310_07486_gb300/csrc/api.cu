@@ -62,6 +62,7 @@ Group describe(const qsg_shape &s, int gid) {
     g.n_samples = s.n_samples;
     g.nwx = (s.L * s.L + 63) / 64;
     g.xi_norm = 2.0 * std::sin(3.14159265358979323846 / s.L);
+    g.wait_limit = kDefaultWaitLimit;
     return g;
 }
 
@@ -999,6 +1000,8 @@ qsg_status qsg_set_option(qsg_ctx *ctx, int32_t option, int64_t value) {
     if (option == QSG_OPT_WAIT_LIMIT) {
         if (value < 0 || value > (1LL << 30)) return QSG_ERR_ARG;
         ctx->wait_limit = (unsigned)value;
+        for (Group &g : ctx->groups) g.wait_limit = ctx->wait_limit;
+        ctx->graph_key = -1;  // captured sweeps carry the limit
         return QSG_OK;
     }
     if (option == QSG_OPT_CHUNK) {

@@ -50,7 +50,7 @@ namespace unit {
 using namespace sweep;
 
 constexpr int kRing = 16;                  // planes in the ring
-constexpr unsigned kWaitPolls = 1u << 20;  // polls of a bounded wait for a bulk copy
+constexpr unsigned kDrainPolls = 1u << 24; // polls of the wait for copies in flight after a wait gave up
 
 // Chunks per block.
 __host__ __device__ constexpr int units_per_block(int L) {
@@ -64,18 +64,41 @@ __device__ __forceinline__ void bar_init(uint64_t *b) {
 __device__ __forceinline__ void bar_expect(uint64_t *b, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
 }
-// Wait for the phase of the given parity; false after `limit` polls.
-__device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, unsigned limit) {
+// A flag in shared memory that any thread may set (32-bit addresses: a generic
+// pointer would take a register pair of the sweep's 72).
+__device__ __forceinline__ bool flag_set(const int *f) {
+    int v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(smem_addr(f)) : "memory");
+    return v != 0;
+}
+__device__ __forceinline__ void set_flag(int *f, int v) {
+    asm volatile("st.volatile.shared.u32 [%0], %1;\n" ::"r"(smem_addr(f)), "r"(v) : "memory");
+}
+// Wait for the phase of the given parity; false after `limit` polls (*gave_up is
+// set then) or when another thread of the block has given up.
+__device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, unsigned limit, int *gave_up) {
     const uint32_t a = smem_addr(b);
-    for (unsigned it = 0; it < limit; ++it) {
+    for (; limit != 0; --limit) {
         uint32_t done;
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done)
                      : "r"(a), "r"(parity)
                      : "memory");
         if (done) return true;
+        if (flag_set(gave_up)) return false;
     }
+    set_flag(gave_up, 1);
     return false;
+}
+// Wait for a copy in flight before the block that it writes to ends.
+__device__ __forceinline__ void bar_drain(uint64_t *b, uint32_t parity) {
+    const uint32_t a = smem_addr(b);
+    uint32_t done = 0;
+    for (unsigned it = 0; it < kDrainPolls && !done; ++it)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done)
+                     : "r"(a), "r"(parity)
+                     : "memory");
 }
 // Bulk copies: 16-byte aligned on both sides, sizes multiples of 16 (a plane is
 // 8 L^2 bytes, L even).
@@ -172,8 +195,10 @@ __device__ __forceinline__ void boundary_sites(const Group &g, const Cols &k, co
 
 // Slots [0, S1) run nch chunks, slots [S1, nslots) nch2, every slot's chunks of
 // nearly equal length, P consecutive ones per block; the boundary counter at the start of chunk ch of slot s is
-// arrivals[s * astride + ch].  err (may be null) receives DEVERR_TIMEOUT when a
-// wait for a copy gave up.
+// arrivals[s * astride + ch].  When a wait for a copy gives up, the block starts no
+// further copy, neither way, and updates no boundary site; it runs out its loop on
+// what the ring holds, waits for the copies in flight, leaves the counters as a
+// finished block would and sets *err (may be null) to DEVERR_TIMEOUT.
 template <int ALGO, int L, int P, int NREG>
 __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     k_sweep_unit(const Group g, const int nch, const int S1, const int nch2, const uint32_t *sweep_base,
@@ -184,6 +209,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     extern __shared__ __align__(128) uint64_t smem[];
     __shared__ uint64_t full_all[P][4];
     __shared__ int do_boundary[P];
+    __shared__ int gave_up, loaded[P];  // a wait gave up; groups of planes loaded by each unit
     const uint32_t sweep = (sweep_base ? *sweep_base : 0u) + sweep_off;
     const int un = P == 1 ? 0 : (int)threadIdx.x / NT, c = (int)threadIdx.x - un * NT;
     const int bps1 = (nch + P - 1) / P, bps2 = (nch2 + P - 1) / P;  // blocks per slot
@@ -204,7 +230,6 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     uint64_t *ring = smem + (size_t)un * kRing * SLOT;
     uint64_t *full = full_all[un];
     const bool leader = c == 0 && active;
-    bool failed = false;
 
     // group gi: planes a - 1 + 4 gi .. a + 2 + 4 gi (those up to b) into ring slots 4 (gi & 3) ..
     auto load_group = [&](int gi) {
@@ -241,6 +266,8 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         load_group(2);
         load_group(3);
     }
+    if (threadIdx.x == 0) gave_up = 0;
+    if (leader) loaded[un] = (b - a + 1) / 4 + 1;
     const Cols k(L, c);
     const Couplings J(g, w, k);
     Thresh T;
@@ -255,7 +282,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     uint4 ra = draw(a), rb = draw(a + 2);
     uint32_t carry = 0;
     __syncthreads();  // the barriers are initialised
-    if (active && !bar_wait(&full[0], 0u, kWaitPolls)) failed = true;
+    if (active) bar_wait(&full[0], 0u, g.wait_limit, &gave_up);
     uint64_t W0[8], W1[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) W0[i] = W1[i] = 0;
@@ -271,9 +298,8 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         const int q = a + 4 * m;
         auto slot = [&](auto ic) -> uint64_t * { return ring + ((decltype(ic)::value + 1) & 15) * SLOT; };
 #define IC(N) std::integral_constant<int, Q + (N)>{}
-        if (active && !failed && (!EDGE || q + 3 <= b) &&
-            !bar_wait(&full[(m + 1) & 3], (uint32_t)((m + 1) >> 2) & 1u, kWaitPolls))
-            failed = true;
+        if (active && (!EDGE || q + 3 <= b))
+            bar_wait(&full[(m + 1) & 3], (uint32_t)((m + 1) >> 2) & 1u, g.wait_limit, &gave_up);
         auto own = [&](auto ic) {
             W0[decltype(ic)::value & 7] = slot(ic)[k.o0];
             W1[decltype(ic)::value & 7] = slot(ic)[k.o1];
@@ -306,7 +332,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         }
         fence_async_smem();
         __syncthreads();
-        if (leader && (!EDGE || m > 0)) {
+        if (leader && (!EDGE || m > 0) && !flag_set(&gave_up)) {
             store_group(m - 1);
             bulk_commit();
         }
@@ -320,8 +346,12 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         rb = draw(q + 6);
         carry = r1.z;
         if (leader && (!EDGE || m > 0)) {
-            bulk_wait_read();
-            load_group(m + 3);
+            if (!flag_set(&gave_up)) {
+                bulk_wait_read();
+                load_group(m + 3);
+            } else {
+                loaded[un] = min(loaded[un], m + 3);
+            }
         }
 #undef IC
     };
@@ -349,10 +379,17 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     const int chn = ch + 1 == nu ? 0 : ch + 1;  // the chunk after the last is the first
     if (c == 0) {
         int flags = 0;
+        const bool ok = !flag_set(&gave_up);
         if (active) {
-            store_group(Mr - 1);
-            store_group(Mr);
-            bulk_commit();
+            if (ok) {
+                store_group(Mr - 1);
+                store_group(Mr);
+                bulk_commit();
+            } else {
+                const int n = loaded[un];
+                for (int gi = max(n - 4, 0); gi < n; ++gi) bar_drain(&full[gi & 3], (uint32_t)(gi >> 2) & 1u);
+                if (err) atomicExch(err, (int)DEVERR_TIMEOUT);
+            }
             bulk_wait_all();
             fence_async();
             __threadfence();
@@ -360,15 +397,14 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
             if (atomicAdd(&arrivals[s * astride + chn], 1u) == 1u) flags |= 2;
             __threadfence();
         }
-        do_boundary[un] = flags;
+        do_boundary[un] = ok ? flags : flags | 4;
     }
     __syncthreads();
-    if (failed && err) atomicExch(err, (int)DEVERR_TIMEOUT);
     const int flags = do_boundary[un];
     if (flags) {
-        if (flags & 1)
+        if ((flags & 5) == 1)
             boundary_sites<ALGO, L>(g, k, J, Sg, a, T, sweep, (uint32_t)s, k0, k1);
-        if (flags & 2)
+        if ((flags & 6) == 2)
             boundary_sites<ALGO, L>(g, k, J, Sg, b == Lt ? 0 : b, T, sweep, (uint32_t)s, k0, k1);
         if (c == 0) {
             if (flags & 1) arrivals[s * astride + ch] = 0u;

@@ -623,6 +623,7 @@ extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t
     g.nlag = sh.Ltau / 2 + 1;
     g.n_samples = sh.n_samples;
     g.nwx = (sh.L * sh.L + 63) / 64;
+    g.wait_limit = kDefaultWaitLimit;
     if ((long long)g.W * g.R * g.K > (1LL << 30)) return QSG_ERR_SHAPE;
     const int C = wavefront_chunk(g, 0);
     if (C == 0) return QSG_ERR_SHAPE;  // L_tau must be a multiple of 16

@@ -44,6 +44,7 @@ struct Group {
     uint64_t *scratch;   // correlator scratch of its own (small groups among several), else null
     size_t scratch_words;
     int *err;            // device status word for waits that gave up (may be null)
+    unsigned wait_limit; // polls of each bounded wait of the sweeps
 };
 
 // ---------------------------------------------------------------------------

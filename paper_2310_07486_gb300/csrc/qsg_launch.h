@@ -19,6 +19,8 @@ bool build_accept_tables(const double *k, int K, uint32_t *table);
 
 // Device-side status word: non-zero after a bounded wait gave up.
 enum : int { DEVERR_NONE = 0, DEVERR_TIMEOUT = 1 };
+// Polls of each bounded device wait (QSG_OPT_WAIT_LIMIT replaces it).
+constexpr unsigned kDefaultWaitLimit = 1u << 22;
 
 cudaError_t launch_init_couplings(const Group &g, uint64_t seed, cudaStream_t st);
 cudaError_t launch_init_spins(const Group &g, uint64_t seed, cudaStream_t st);
@@ -81,7 +83,6 @@ cudaError_t launch_tempering(const Group &g, uint32_t m, uint64_t seed, cudaStre
 // XOR/popcount on the integer pipes.  status receives DEVERR_TIMEOUT if a
 // bounded wait of the tensor path gave up (after wait_limit polls).
 // triples = 1 also accumulates the three-replica one-time sums (3 <= R <= 8).
-constexpr unsigned kDefaultWaitLimit = 1u << 22;
 cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_words, int tensor, int triples,
                            int *status, unsigned wait_limit, cudaStream_t st);
 // One-time observable sums of a batch of (w, j) pairs from the transposed scratch.

@@ -84,3 +84,44 @@ def test_asynchronous_read_reports_the_flag_when_waited_for():
     ref = good.qsg_read_correlators()
     for key in ("C", "Q2", "q2"):
         assert np.array_equal(out[key], ref[key]), key
+
+
+def _spins_on_device(ctx, shape):
+    out = torch.empty(shape.slots * shape.Ltau * shape.L ** 2, dtype=torch.int64, device=ctx.device)
+    ctx.qsg_get_spins_device(0, out)
+    return out
+
+
+@pytest.mark.parametrize("L,Ltau,R,variant", [(8, 48, 9, 0), (6, 32, 9, 1), (6, 820, 2, 1), (10, 6, 3, 1), (16, 512, 3, 1),
+                                              (24, 256, 2, 1)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_sweep_whose_waits_give_up_leaves_the_spins_and_the_counters(L, Ltau, R, variant, graph):
+    """The resident form and chunks of one and of several planes per step: no spin
+    changes, every block ends, the device flag is set, and sweeps with the limit put
+    back are those of a context that never gave up."""
+    if graph and Ltau % 16:
+        pytest.skip("graphs need L_tau to be a multiple of 16")
+    shape = Q.Shape(L, Ltau, 70, R, 2, Q.HEATBATH, Q.APBC)
+    lad = np.array([0.25, 0.3])
+    ctx, plain = Q.Context([shape]), Q.Context([shape])
+    for c in (ctx, plain):
+        c.qsg_init_samples(7, [lad])
+    try:
+        ctx.qsg_set_option(Q.OPT_WAVEFRONT_VARIANT, variant)
+        if graph:
+            ctx.qsg_set_option(Q.OPT_GRAPH, 2)
+        ctx.qsg_set_option(Q.OPT_WAIT_LIMIT, 0)
+        before = _spins_on_device(ctx, shape)
+        ctx.qsg_sweep(2)
+        assert torch.equal(_spins_on_device(ctx, shape), before)
+        with pytest.raises(Q.QSGError) as e:
+            ctx.qsg_read_correlators()
+        assert e.value.status == -4
+        ctx.qsg_set_option(Q.OPT_WAIT_LIMIT, 1 << 22)
+        ctx.qsg_set_counters(0, 0)
+        ctx.qsg_sweep(4)
+        plain.qsg_set_option(Q.OPT_SWEEP_KERNEL, Q.SWEEP_REFERENCE)
+        plain.qsg_sweep(4)
+        assert torch.equal(_spins_on_device(ctx, shape), _spins_on_device(plain, shape))
+    finally:
+        ctx.qsg_set_option(Q.OPT_WAVEFRONT_VARIANT, 0)
