@@ -384,7 +384,8 @@ qsg_status qsg_set_counters(qsg_ctx *ctx, uint32_t sweeps, uint32_t swaps, int64
  *                         further work and that measurement is not
  *                         accumulated; in a sweep the block starts no further
  *                         copy, so planes it had not yet written stay as they
- *                         were.  qsg_read_correlators returns
+ *                         were.  Every read_* call of sweep or measurement
+ *                         results (and qsg_get_spins) returns
  *                         QSG_ERR_TIMEOUT from then on (the flag stays set
  *                         for the context).  A small value is a way to
  *                         exercise that path; the default never gives up on a

@@ -248,7 +248,12 @@ struct qsg_ctx {
     // writer of the correlator buffers waits for
     cudaEvent_t fin_ev = nullptr, copy_ev = nullptr;
     bool copy_pending = false;
-    int *h_flag = nullptr;  // page-locked copy of the device flag, taken with the copies
+    // page-locked copies of the device flag: [0] taken with the copies of an
+    // asynchronous read, [1] as last read by fetch_flag
+    int *h_flag = nullptr;
+    // kernels that may set the device flag were queued since it was last read, or
+    // were captured by the caller, who may replay them at any time
+    bool flag_unread = false, flag_captured = false;
     bool flag_pending = false;
     ~qsg_ctx() {
         // the copies read the workspace, which the caller frees after this
@@ -286,11 +291,28 @@ static qsg_status order_after_copies(qsg_ctx *c) {
     return QSG_OK;
 }
 
+// Kernels with bounded waits are about to be queued.
+static void expect_flag(qsg_ctx *c) {
+    c->flag_unread = true;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) c->flag_captured = true;
+}
+
+// Queues the read of the device flag where it can have changed.  A read of a few bytes
+// is all latency, so it goes ahead of the results' copies: behind a copy to pageable
+// memory, which waits for the stream, it took 8 us of a monitoring pass of 555.
+static qsg_status fetch_flag(qsg_ctx *c) {
+    if (c->flag_unread || c->flag_captured)
+        QSG_CUDA(c, cudaMemcpyAsync(&c->h_flag[1], c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    c->flag_unread = false;
+    return QSG_OK;
+}
+
+// Waits for the context's stream and reports the flag that fetch_flag read.
 static qsg_status check_device_flag(qsg_ctx *c) {
-    int h = 0;
-    QSG_CUDA(c, cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     QSG_CUDA(c, cudaStreamSynchronize(c->stream));
-    return h == DEVERR_NONE ? QSG_OK : QSG_ERR_TIMEOUT;
+    return c->h_flag[1] == DEVERR_NONE ? QSG_OK : QSG_ERR_TIMEOUT;
 }
 
 // Build the persistent-launch plan (all groups with the same algorithm, L <= 24,
@@ -355,7 +377,11 @@ qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, 
     carve(c->groups, c->ws, &c->d_err, &c->scratch, &c->scratch_words, &c->pb);
     for (Group &g : c->groups) g.err = c->d_err;
     c->stream = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream);
+    cudaError_t e = cudaHostAlloc((void **)&c->h_flag, 2 * sizeof(int), cudaHostAllocDefault);
+    if (e == cudaSuccess) {
+        c->h_flag[0] = c->h_flag[1] = DEVERR_NONE;
+        e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream);
+    }
     for (const Group &g : c->groups)
         if (e == cudaSuccess)
             e = cudaMemsetAsync(g.arrivals, 0, sizeof(unsigned) * (size_t)g.nslots * (g.Ltau / 4 > 0 ? g.Ltau / 4 : 1),
@@ -638,6 +664,7 @@ qsg_status qsg_sweep(qsg_ctx *ctx, int32_t n_sweeps) {
     if (!ctx->initialised) return QSG_ERR_STATE;
     if ((uint64_t)ctx->sweeps + (uint64_t)n_sweeps > 0xFFFFFFFFull) return QSG_ERR_ARG;
     const SweepMode mode = sweep_mode(ctx);
+    expect_flag(ctx);
     int done = 0;
     const int G = ctx->graph_batch;
     if (G > 0 && n_sweeps >= G) {
@@ -695,6 +722,7 @@ qsg_status qsg_measure_correlators(qsg_ctx *ctx) {
     if (!ctx) return QSG_ERR_ARG;
     if (!ctx->initialised) return QSG_ERR_STATE;
     if (qsg_status o = order_after_copies(ctx)) return o;
+    expect_flag(ctx);
     auto work = [&](const Group &g, cudaStream_t st) -> qsg_status {
         uint64_t *scratch = g.scratch ? g.scratch : ctx->scratch;
         const size_t words = g.scratch ? g.scratch_words : ctx->scratch_words;
@@ -749,6 +777,7 @@ qsg_status qsg_read_correlators(qsg_ctx *ctx, int32_t group, double *C, double *
     if (qsg_status o = order_after_copies(ctx)) return o;
     const Group &g = ctx->groups[group];
     QSG_CUDA(ctx, launch_finish(g, ctx->n_meas, ctx->stream));
+    if (qsg_status o = fetch_flag(ctx)) return o;
     if (qsg_status o = copy_correlators(ctx, g, C, Q2, q2, raw, ctx->stream)) return o;
     return check_device_flag(ctx);
 }
@@ -763,7 +792,6 @@ qsg_status qsg_read_correlators_async(qsg_ctx *ctx, int32_t group, double *C, do
     if (qsg_status o = order_after_copies(ctx)) return o;
     if (!ctx->fin_ev) QSG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fin_ev, cudaEventDisableTiming));
     if (!ctx->copy_ev) QSG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->copy_ev, cudaEventDisableTiming));
-    if (!ctx->h_flag) QSG_CUDA(ctx, cudaHostAlloc((void **)&ctx->h_flag, sizeof(int), cudaHostAllocDefault));
     const Group &g = ctx->groups[group];
     // the finish runs on the copy stream too, once the context's stream has
     // done the measurements: it writes only what the copies read, and the
@@ -796,6 +824,7 @@ qsg_status qsg_read_onetime(qsg_ctx *ctx, int32_t group, double *per_sample, dou
     std::vector<double> ho(nsk * 7), hk((size_t)g.K * 8);
     std::vector<long long> rp, rt, rg, rf;
     std::vector<unsigned long long> r4;
+    if (qsg_status f = fetch_flag(ctx)) return f;
     QSG_CUDA(ctx, cudaMemcpyAsync(ho.data(), g.outO, sizeof(double) * ho.size(), cudaMemcpyDeviceToHost, ctx->stream));
     QSG_CUDA(ctx, cudaMemcpyAsync(hk.data(), g.outK, sizeof(double) * hk.size(), cudaMemcpyDeviceToHost, ctx->stream));
     if (raw) {
@@ -813,7 +842,7 @@ qsg_status qsg_read_onetime(qsg_ctx *ctx, int32_t group, double *per_sample, dou
         QSG_CUDA(ctx, cudaMemcpyAsync(rf.data(), g.F3acc, sizeof(long long) * nsk * nd, cudaMemcpyDeviceToHost,
                                       ctx->stream));
     }
-    QSG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (qsg_status s = check_device_flag(ctx)) return s;
     const size_t ns = (size_t)g.n_samples * g.K;
     if (per_sample) std::memcpy(per_sample, ho.data(), sizeof(double) * ns * 7);
     if (per_k) std::memcpy(per_k, hk.data(), sizeof(double) * hk.size());
@@ -842,10 +871,10 @@ qsg_status qsg_read_pair_overlaps(qsg_ctx *ctx, int32_t group, int64_t *out) {
     const Group &g = ctx->groups[group];
     const size_t np = (size_t)(g.R * (g.R - 1) / 2);
     if (np == 0) return QSG_OK;
+    if (qsg_status f = fetch_flag(ctx)) return f;
     QSG_CUDA(ctx, cudaMemcpyAsync(out, g.PPacc, sizeof(long long) * (size_t)g.n_samples * g.K * np,
                                   cudaMemcpyDeviceToHost, ctx->stream));
-    QSG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return QSG_OK;
+    return check_device_flag(ctx);
 }
 
 qsg_status qsg_sample_features(qsg_ctx *ctx, int32_t group, float *out) {
@@ -869,8 +898,9 @@ qsg_status qsg_read_energies(qsg_ctx *ctx, int32_t group, int64_t *E_host) {
     if (s != QSG_OK) return s;
     const Group &g = ctx->groups[group];
     std::vector<int32_t> U((size_t)g.nslots * 64);
+    if (qsg_status f = fetch_flag(ctx)) return f;
     QSG_CUDA(ctx, cudaMemcpyAsync(U.data(), g.U, sizeof(int32_t) * U.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    QSG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (qsg_status f = check_device_flag(ctx)) return f;
     for (int b = 0; b < g.n_samples; ++b)
         for (int r = 0; r < g.R; ++r)
             for (int j = 0; j < g.K; ++j) {
@@ -886,8 +916,9 @@ qsg_status qsg_read_accepts(qsg_ctx *ctx, int32_t group, int64_t *acc_host) {
     const Group &g = ctx->groups[group];
     const int np = g.K > 1 ? g.K - 1 : 1;
     std::vector<unsigned long long> a((size_t)g.W * 64 * np);
+    if (qsg_status f = fetch_flag(ctx)) return f;
     QSG_CUDA(ctx, cudaMemcpyAsync(a.data(), g.acc, sizeof(unsigned long long) * a.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    QSG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (qsg_status f = check_device_flag(ctx)) return f;
     for (size_t i = 0; i < (size_t)g.n_samples * np; ++i) acc_host[i] = (int64_t)a[i];
     return QSG_OK;
 }
@@ -895,9 +926,9 @@ qsg_status qsg_read_accepts(qsg_ctx *ctx, int32_t group, int64_t *acc_host) {
 qsg_status qsg_get_spins(qsg_ctx *ctx, int32_t group, uint64_t *host) {
     if (!ctx || !host || group < 0 || group >= (int)ctx->groups.size()) return QSG_ERR_ARG;
     const Group &g = ctx->groups[group];
+    if (qsg_status f = fetch_flag(ctx)) return f;
     QSG_CUDA(ctx, cudaMemcpyAsync(host, g.S, sizeof(uint64_t) * (size_t)g.nslots * g.N, cudaMemcpyDeviceToHost, ctx->stream));
-    QSG_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return QSG_OK;
+    return check_device_flag(ctx);
 }
 
 qsg_status qsg_set_spins(qsg_ctx *ctx, int32_t group, const uint64_t *host) {

@@ -125,3 +125,29 @@ def test_sweep_whose_waits_give_up_leaves_the_spins_and_the_counters(L, Ltau, R,
         assert torch.equal(_spins_on_device(ctx, shape), _spins_on_device(plain, shape))
     finally:
         ctx.qsg_set_option(Q.OPT_WAVEFRONT_VARIANT, 0)
+
+
+@pytest.mark.parametrize("what", ["sweep", "measurement"])
+def test_every_read_of_results_reports_the_flag(what):
+    """Energies, accepted swaps, one-time sums, overlaps and spins as the correlators,
+    more than once; a context whose waits never gave up reads all of them."""
+    shape = Q.Shape(8, 256, 64, 3, 2, Q.HEATBATH, Q.PBC)
+    reads = ("qsg_get_spins", "qsg_read_energies", "qsg_read_accepts", "qsg_read_onetime", "qsg_read_pair_overlaps",
+             "qsg_read_correlators", "qsg_get_spins", "qsg_read_energies")
+    for limit in (0, 1 << 22):
+        ctx = Q.Context([shape])
+        ctx.qsg_init_samples(7, [np.array([0.25, 0.3])])
+        ctx.qsg_read_energies()  # the flag read before the wait that gives up
+        if what == "sweep":
+            ctx.qsg_set_option(Q.OPT_WAIT_LIMIT, limit)
+            ctx.qsg_sweep(1)
+        ctx.qsg_tempering_swap()
+        ctx.qsg_set_option(Q.OPT_WAIT_LIMIT, limit)
+        ctx.qsg_measure_correlators()
+        for name in reads:
+            if limit:
+                getattr(ctx, name)()
+                continue
+            with pytest.raises(Q.QSGError) as e:
+                getattr(ctx, name)()
+            assert e.value.status == -4, name
