@@ -433,7 +433,10 @@ qsg_status qsg_set_option(qsg_ctx *ctx, int32_t option, int64_t value);
  * call's contents: calls that overlap on the GPU (other streams, other host
  * threads) race and must be serialised by the caller.  The call copies the
  * table to the device and waits for that copy on cuda_stream; the sweeps are
- * enqueued on cuda_stream without waiting.  Nothing is allocated. */
+ * enqueued on cuda_stream without waiting.  Nothing is allocated.
+ * A bounded wait of these sweeps that gave up is reported, once, by the next call
+ * on the device: it returns QSG_ERR_TIMEOUT and sweeps nothing (n_sweeps = 0 asks
+ * without sweeping). */
 qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t *d_Jx, const uint64_t *d_Jy,
                                     const qsg_shape *shape, int32_t group_id, const double *k_ladder, uint64_t seed,
                                     uint32_t first_sweep, int32_t n_sweeps, void *cuda_stream);

@@ -564,40 +564,48 @@ constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) unsigned g_static_arrivals[kStaticArrivals];
 __device__ __align__(256) uint32_t g_static_thr[kStaticMaxK * 16];
+__device__ int g_static_status;  // DEVERR_TIMEOUT after a wait of these sweeps gave up
 
 std::mutex g_static_mutex;
 void *g_static_arrivals_ptr[kMaxDevices];
 void *g_static_thr_ptr[kMaxDevices];
+void *g_static_status_ptr[kMaxDevices];
 
-// Device addresses of the two arrays on device `dev`, which must be current
-// (looked up, and the counters cleared, on the first call on that device).
-// The addresses are cached per device; they do not survive cudaDeviceReset.
-cudaError_t static_scratch(int dev, void **arrivals, void **thr) {
+// Device addresses of the two arrays and the status word on device `dev`, which
+// must be current (looked up, and the counters cleared, on the first call on that
+// device).  The addresses are cached per device; they do not survive cudaDeviceReset.
+cudaError_t static_scratch(int dev, void **arrivals, void **thr, void **status) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_static_mutex);
     if (!g_static_arrivals_ptr[dev]) {
-        void *a = nullptr, *t = nullptr;
+        void *a = nullptr, *t = nullptr, *s = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&a, g_static_arrivals);
         if (e != cudaSuccess) return e;
         e = cudaGetSymbolAddress(&t, g_static_thr);
+        if (e != cudaSuccess) return e;
+        e = cudaGetSymbolAddress(&s, g_static_status);
         if (e != cudaSuccess) return e;
         e = cudaMemset(a, 0, sizeof(unsigned) * kStaticArrivals);
         if (e != cudaSuccess) return e;
         g_static_arrivals_ptr[dev] = a;
         g_static_thr_ptr[dev] = t;
+        g_static_status_ptr[dev] = s;
     }
     *arrivals = g_static_arrivals_ptr[dev];
     *thr = g_static_thr_ptr[dev];
+    *status = g_static_status_ptr[dev];
     return cudaSuccess;
 }
 
 }  // namespace
 }  // namespace qsg
 
-extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t *d_Jx, const uint64_t *d_Jy,
-                                               const qsg_shape *shape, int32_t group_id, const double *k_ladder,
-                                               uint64_t seed, uint32_t first_sweep, int32_t n_sweeps,
-                                               void *cuda_stream) {
+// qsg_sweep_static_scratch with the polls of each bounded wait given (not part of the
+// ABI: with none, the report of a wait that gave up can be tested).
+extern "C" qsg_status qsg_internal_static_sweeps(uint64_t *d_spins, const uint64_t *d_Jx, const uint64_t *d_Jy,
+                                                 const qsg_shape *shape, int32_t group_id, const double *k_ladder,
+                                                 uint64_t seed, uint32_t first_sweep, int32_t n_sweeps,
+                                                 void *cuda_stream, uint32_t wait_limit) {
     using namespace qsg;
     // shape and limits first, so that an oversized shape is reported as such
     // whatever the buffers are
@@ -623,7 +631,7 @@ extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t
     g.nlag = sh.Ltau / 2 + 1;
     g.n_samples = sh.n_samples;
     g.nwx = (sh.L * sh.L + 63) / 64;
-    g.wait_limit = kDefaultWaitLimit;
+    g.wait_limit = wait_limit;
     if ((long long)g.W * g.R * g.K > (1LL << 30)) return QSG_ERR_SHAPE;
     const int C = wavefront_chunk(g, 0);
     if (C == 0) return QSG_ERR_SHAPE;  // L_tau must be a multiple of 16
@@ -641,12 +649,17 @@ extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t
     if (cudaGetDevice(&dev) != cudaSuccess) return QSG_ERR_CUDA;
     if (cudaStreamGetDevice(st, &sdev) != cudaSuccess) return QSG_ERR_ARG;
     if (sdev != dev) return QSG_ERR_ARG;
-    void *arr = nullptr, *thr = nullptr;
-    if (static_scratch(dev, &arr, &thr) != cudaSuccess) return QSG_ERR_CUDA;
-    // the table lives on this function's stack: copy it and wait for the copy
+    void *arr = nullptr, *thr = nullptr, *status = nullptr;
+    if (static_scratch(dev, &arr, &thr, &status) != cudaSuccess) return QSG_ERR_CUDA;
+    // the table lives on this function's stack: copy it and wait for the copy; the
+    // status that earlier calls left comes back by the same wait
+    int earlier = DEVERR_NONE;
+    if (cudaMemcpyAsync(&earlier, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return QSG_ERR_CUDA;
     if (cudaMemcpyAsync(thr, table, sizeof(uint32_t) * 16 * (size_t)g.K, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return QSG_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return QSG_ERR_CUDA;
+    if (earlier != DEVERR_NONE)  // reported once
+        return cudaMemsetAsync(status, 0, sizeof(int), st) == cudaSuccess ? QSG_ERR_TIMEOUT : QSG_ERR_CUDA;
     // counters start at zero (each sweep leaves them at zero; cleared anyway)
     if (cudaMemsetAsync(arr, 0, sizeof(unsigned) * (size_t)g.nslots * (g.Ltau / C), st) != cudaSuccess)
         return QSG_ERR_CUDA;
@@ -654,8 +667,17 @@ extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t
     g.Jx = const_cast<uint64_t *>(d_Jx);
     g.Jy = const_cast<uint64_t *>(d_Jy);
     g.thr = (uint32_t *)thr;
+    g.err = (int *)status;
     for (int it = 0; it < n_sweeps; ++it)
         if (launch_sweep_wavefront(g, nullptr, first_sweep + (uint32_t)it, seed, (unsigned *)arr, C, 0, st) != cudaSuccess)
             return QSG_ERR_CUDA;
     return QSG_OK;
+}
+
+extern "C" qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t *d_Jx, const uint64_t *d_Jy,
+                                               const qsg_shape *shape, int32_t group_id, const double *k_ladder,
+                                               uint64_t seed, uint32_t first_sweep, int32_t n_sweeps,
+                                               void *cuda_stream) {
+    return qsg_internal_static_sweeps(d_spins, d_Jx, d_Jy, shape, group_id, k_ladder, seed, first_sweep, n_sweeps,
+                                      cuda_stream, qsg::kDefaultWaitLimit);
 }

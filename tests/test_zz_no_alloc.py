@@ -72,3 +72,32 @@ def test_static_scratch_wrapper_rejects_buffers_that_do_not_fit_the_shape():
     with pytest.raises(Q.QSGError) as e:  # ladder length differs from n_k
         Q.qsg_sweep_static_scratch(spins, J, J, shape, 0, [0.3, 0.4], 1, 0, 1)
     assert e.value.status == -1
+
+
+def test_static_scratch_reports_a_wait_that_gave_up_once():
+    """The entry point with no polls at all: no spin changes, the next call returns the
+    timeout, the one after it sweeps as ever."""
+    import ctypes
+    shape = Q.Shape(8, 256, 64, 2, 1, Q.HEATBATH, Q.PBC)
+    ladder = np.array([0.3])
+    dev = torch.device("cuda")
+    spins = torch.randint(-2 ** 62, 2 ** 62, (shape.slots * shape.Ltau * 64,), dtype=torch.int64, device=dev)
+    J = torch.zeros(64, dtype=torch.int64, device=dev)
+    before, ref = spins.clone(), spins.clone()
+    f = Q.load_library().qsg_internal_static_sweeps
+    vp = ctypes.c_void_p
+    f.restype = ctypes.c_int32
+    f.argtypes = [vp, vp, vp, vp, ctypes.c_int32, vp, ctypes.c_uint64, ctypes.c_uint32, ctypes.c_int32, vp, ctypes.c_uint32]
+    sh = shape.c()
+    st = torch.cuda.current_stream().cuda_stream
+    assert f(spins.data_ptr(), J.data_ptr(), J.data_ptr(), ctypes.byref(sh), 0, ladder.ctypes.data, 5, 0, 2, st, 0) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(spins, before)
+    with pytest.raises(Q.QSGError) as e:
+        Q.qsg_sweep_static_scratch(spins, J, J, shape, 0, ladder, 5, 0, 2)
+    assert e.value.status == -4
+    Q.qsg_sweep_static_scratch(spins, J, J, shape, 0, ladder, 5, 0, 2)
+    Q.qsg_sweep_static_scratch(ref, J, J, shape, 0, ladder, 5, 0, 1)
+    Q.qsg_sweep_static_scratch(ref, J, J, shape, 0, ladder, 5, 1, 1)
+    torch.cuda.synchronize()
+    assert torch.equal(spins, ref) and not torch.equal(spins, before)
