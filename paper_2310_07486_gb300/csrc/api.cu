@@ -203,6 +203,17 @@ uint64_t pt_factor(double delta, long long n) {
 
 }  // namespace
 
+// Everything that a captured graph of sweeps holds by value.
+struct GraphKey {
+    int batch = 0, kernel = 0, mode = 0, variant = 0, chunk = 0, tail = 0, upb = 0;
+    unsigned wait_limit = 0;
+    uint64_t seed = 0;
+    bool operator==(const GraphKey &o) const {
+        return batch == o.batch && kernel == o.kernel && mode == o.mode && variant == o.variant && chunk == o.chunk &&
+               tail == o.tail && upb == o.upb && wait_limit == o.wait_limit && seed == o.seed;
+    }
+};
+
 struct qsg_ctx {
     std::vector<qsg_shape> shapes;
     std::vector<Group> groups;
@@ -232,7 +243,7 @@ struct qsg_ctx {
     // stream and replayed on `stream`; the kernels read the sweep index from
     // pb.sweep_base, which base_valid says equals `sweeps`.
     int graph_batch = 0;
-    long long graph_key = -1;
+    GraphKey graph_key;
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
     unsigned long long graph_launches = 0;  // kernels per replay
@@ -623,10 +634,18 @@ static qsg_status launch_sweeps(qsg_ctx *ctx, SweepMode mode, const uint32_t *sb
         [&](const Group &g, cudaStream_t t) { return group_sweeps(ctx, g, sb, first, count, t); });
 }
 
-// (Re)capture the graph of graph_batch sweeps when a launch option changed.
+// (Re)capture the graph of graph_batch sweeps when a launch option or the seed changed.
 static qsg_status ensure_graph(qsg_ctx *ctx, SweepMode mode) {
-    const long long key = ((((((long long)ctx->graph_batch * 4 + ctx->sweep_kernel) * 4 + (int)mode) * 4 +
-                             g_wavefront_variant) * 65537LL + ctx->chunk) * 65537LL + ctx->tail) * 32 + ctx->upb;
+    GraphKey key;
+    key.batch = ctx->graph_batch;
+    key.kernel = ctx->sweep_kernel;
+    key.mode = (int)mode;
+    key.variant = g_wavefront_variant;
+    key.chunk = ctx->chunk;
+    key.tail = ctx->tail;
+    key.upb = ctx->upb;
+    key.wait_limit = ctx->wait_limit;
+    key.seed = ctx->seed;
     if (ctx->graph_exec && ctx->graph_key == key) return QSG_OK;
     if (ctx->graph_exec) {
         cudaGraphExecDestroy(ctx->graph_exec);
@@ -1032,7 +1051,6 @@ qsg_status qsg_set_option(qsg_ctx *ctx, int32_t option, int64_t value) {
         if (value < 0 || value > (1LL << 30)) return QSG_ERR_ARG;
         ctx->wait_limit = (unsigned)value;
         for (Group &g : ctx->groups) g.wait_limit = ctx->wait_limit;
-        ctx->graph_key = -1;  // captured sweeps carry the limit
         return QSG_OK;
     }
     if (option == QSG_OPT_CHUNK) {

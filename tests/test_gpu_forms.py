@@ -191,3 +191,20 @@ def test_training_steps_of_one_call_equal_single_calls(batch):
         params.append(m.get_params())
     assert np.array_equal(losses[0], losses[1]) and np.array_equal(params[0], params[1])
     assert np.all(np.isfinite(params[0]))
+
+
+@pytest.mark.parametrize("shapes", [[Q.Shape(8, 48, 64, 4, 4, Q.HEATBATH)], [Q.Shape(16, 256, 64, 2, 8)],
+                                    [Q.Shape(12, 64, 64, 2, 8), Q.Shape(8, 32, 64, 1, 2)]])
+def test_graph_follows_a_second_initialisation_with_another_seed(shapes):
+    """Captured sweeps hold the seed: resident, chunked and few-slot forms, one and two
+    groups, against direct launches; another seed, then the first one again."""
+    lads = [np.linspace(0.25, 0.35, s.n_k) for s in shapes]
+    graphed, direct = Q.Context(shapes), Q.Context(shapes)
+    graphed.qsg_set_option(Q.OPT_GRAPH, 3)
+    for seed in (3, 2 ** 40 + 3, 3):
+        for ctx in (graphed, direct):
+            ctx.qsg_init_samples(seed, lads)
+            ctx.qsg_sweep(7)
+            ctx.qsg_tempering_swap()
+        for g in range(len(shapes)):
+            assert np.array_equal(graphed.qsg_get_spins(g), direct.qsg_get_spins(g)), (seed, g)
