@@ -25,7 +25,11 @@ using namespace sweep;
 using namespace unit;
 
 constexpr size_t kSlotLimit = 226 * 1024;  // bytes of a slot that fit beside the static barrier
-constexpr long long kLaunchWords = 1ll << 36;  // site-word updates of a launch at most (about 0.25 s)
+// Time of a launch at most, us, and that of a sweep of a slot of N words alone on an
+// SM (measured: 0.64 for N = 576, 1.4 for 2,304, 3.5 for 6,400; slots that share an SM
+// take less than the sum of theirs).
+constexpr double kLaunchTime = 250e3;
+constexpr double sweep_time(int N) { return 0.3 + 0.55e-3 * N; }
 
 // A value the compiler knows nothing about: keeps it from carrying the addresses
 // of every plane pair from one half sweep to the next in registers (they spilled).
@@ -187,8 +191,9 @@ cudaError_t launch_sweep_resident(const Group &g, int count, const uint32_t *swe
     const ResidentShape r = resident_shape(g, nsm);
     const int threads = r.rows * (g.L * g.L / 2);
     if (threads > 1024) return cudaErrorInvalidValue;
-    // launches of a bounded length, however many sweeps are asked for
-    const long long most = kLaunchWords / ((long long)g.nslots * (long long)g.N);
+    // launches of a bounded length, however many sweeps are asked for: an SM serves its
+    // share of the slots, so few slots take as long as one per SM
+    const long long most = (long long)(kLaunchTime / ((g.nslots + nsm - 1) / nsm * sweep_time(g.N)));
     for (int done = 0; done < count && e == cudaSuccess;) {
         const int n = most < 1 ? 1 : (int)(most < count - done ? most : count - done);
         const uint32_t first = sweep + (uint32_t)done;

@@ -208,3 +208,16 @@ def test_graph_follows_a_second_initialisation_with_another_seed(shapes):
             ctx.qsg_tempering_swap()
         for g in range(len(shapes)):
             assert np.array_equal(graphed.qsg_get_spins(g), direct.qsg_get_spins(g)), (seed, g)
+
+
+def test_long_calls_on_few_slots_are_cut_by_time():
+    """Two small slots: 600,000 sweeps are half a second on two SMs, whatever the words
+    add up to; a launch takes a quarter of one at most."""
+    shape = Q.Shape(6, 32, 1, 2, 1, Q.METROPOLIS, Q.PBC)
+    whole, parts = _context(shape, 5), _context(shape, 5)
+    before = Q.qsg_kernel_launches()
+    whole.qsg_sweep(600000)
+    assert 2 <= Q.qsg_kernel_launches() - before <= 4
+    for _ in range(6):
+        parts.qsg_sweep(100000)
+    assert np.array_equal(whole.qsg_get_spins(0), parts.qsg_get_spins(0))
