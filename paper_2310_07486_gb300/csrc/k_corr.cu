@@ -260,6 +260,8 @@ static cudaError_t launch_gram_short(const Group &g, int p0, int npairs, const u
     return cudaGetLastError();
 }
 
+constexpr size_t kGramSmem = 200 * 1024;  // rows of a sample that k_gram keeps in shared memory at most
+
 cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_words, int tensor, int triples,
                            int *status, unsigned wait_limit, cudaStream_t st) {
     const size_t per_pair = measure_scratch_words_per_pair(g);
@@ -267,9 +269,9 @@ cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_wor
     if (batch < 1) return cudaErrorInvalidValue;
     const int npairs_total = g.W * g.K;
     const size_t sh_bytes = (size_t)g.Ltau * g.nwx * sizeof(uint64_t);
-    const int use_smem = sh_bytes <= 200 * 1024 ? 1 : 0;
+    const int use_smem = sh_bytes <= kGramSmem ? 1 : 0;
     if (use_smem && !tensor) {
-        cudaError_t e = cudaFuncSetAttribute(k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh_bytes);
+        cudaError_t e = cudaFuncSetAttribute(k_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem);
         if (e != cudaSuccess) return e;
     }
     for (int p0 = 0; p0 < npairs_total; p0 += batch) {
@@ -277,7 +279,7 @@ cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_wor
         const size_t tr_smem = (size_t)64 * (kTrRun * g.nwx + 1) * sizeof(uint64_t);
         if (tr_smem > 48 * 1024) {
             const cudaError_t ea = cudaFuncSetAttribute(k_transpose, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        (int)tr_smem);
+                                                        64 * (kTrRun * 16 + 1) * (int)sizeof(uint64_t));
             if (ea != cudaSuccess) return ea;
         }
         count_launches(1);

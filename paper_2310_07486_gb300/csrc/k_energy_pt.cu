@@ -396,7 +396,8 @@ static cudaError_t launch_energy_generic(const Group &g, cudaStream_t st) {
     const int threads = (L2 / 2 + 31) / 32 * 32;
     const size_t sm = (size_t)kEnergyBuf * L2 * sizeof(uint64_t);
     if (sm > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        const cudaError_t e = cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kEnergyBuf * 32 * 32 * (int)sizeof(uint64_t));
         if (e != cudaSuccess) return e;
     }
     dim3 grid(g.nslots, (g.Ltau + kEnergyRun - 1) / kEnergyRun);
@@ -607,7 +608,9 @@ cudaError_t launch_tempering(const Group &g, uint32_t m, uint64_t seed, cudaStre
     if (g.K < 2) return cudaSuccess;
     const size_t sm = DecideShared(g.K).total;
     cudaError_t e = cudaSuccess;
-    if (sm > 48 * 1024) e = cudaFuncSetAttribute(k_pt_decide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (sm > 48 * 1024)
+        e = cudaFuncSetAttribute(k_pt_decide, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)DecideShared(kMaxK).total);
     if (e != cudaSuccess) return e;
     count_launches(1);
     k_pt_decide<<<g.W * g.R, kDecideThreads, sm, st>>>(g, m, (uint32_t)seed, (uint32_t)(seed >> 32));

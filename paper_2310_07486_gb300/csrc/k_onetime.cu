@@ -366,6 +366,9 @@ __global__ void __launch_bounds__(128, 3) k_onetime(Group g, int p0, const uint6
     }
 }
 
+// Shared memory of a block at most (a block of 32 threads needs less whatever R and L).
+constexpr int kOnetimeSmem = 96 * 1024;
+
 size_t onetime_smem_bytes(const Group &g, int triples, int threads) {
     const int npair = g.R * (g.R - 1) / 2;
     const size_t pp = (size_t)(npair <= kMaxSharedPairs ? npair : 0) * 8 + (size_t)2 * (g.L / 2 + 1) * threads * 8;
@@ -380,10 +383,10 @@ static cudaError_t launch_onetime_L(const Group &g, int p0, int np, const uint64
     // a thread per slice: where L_tau is short, no more of them than slices (L = 8,
     // L_tau = 48 ran 128 for 48)
     int threads = g.Ltau >= 128 ? 128 : (g.Ltau + 31) / 32 * 32;
-    while (threads > 32 && onetime_smem_bytes(g, triples, threads) > 96 * 1024) threads -= 32;
+    while (threads > 32 && onetime_smem_bytes(g, triples, threads) > kOnetimeSmem) threads -= 32;
     const size_t sm = onetime_smem_bytes(g, triples, threads);
     if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_onetime<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = cudaFuncSetAttribute(k_onetime<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnetimeSmem);
         if (e != cudaSuccess) return e;
     }
     count_launches(1);

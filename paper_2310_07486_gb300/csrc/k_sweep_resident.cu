@@ -123,7 +123,7 @@ template <int ALGO, int IP>
 cudaError_t launch(const Group &g, int threads, size_t sm, int count, const uint32_t *sb, uint32_t sweep, uint64_t seed,
                    cudaStream_t st) {
     auto kern = k_sweep_resident<ALGO, IP>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlotLimit);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     count_launches(1);

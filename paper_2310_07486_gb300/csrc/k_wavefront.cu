@@ -436,8 +436,12 @@ static cudaError_t launch_wf(const Group &g, int C, int tail, const uint32_t *sw
     const int blocks = (units + P - 1) / P;
     const size_t sm = (size_t)P * (kRing * SLOT + 2 * g.L * g.L) * sizeof(uint64_t);
     const int threads = P * (g.L * g.L / 2);
+    // the largest over the sizes and groupings that share an instance: 162,944 bytes (L = 22,
+    // two units of 242 threads)
+    constexpr int kMaxSmem = 160 * 1024;
+    if (sm > (size_t)kMaxSmem) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k_sweep_wavefront<ALGO, SLOT, NREG, JREG>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_sweep_wavefront<ALGO, SLOT, NREG, JREG>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  100);

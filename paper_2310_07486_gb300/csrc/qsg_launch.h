@@ -10,6 +10,11 @@ namespace qsg {
 // Process-wide count of kernel launches (qsg_kernel_launches()).
 void count_launches(int n);
 
+// Shared-memory limits of kernels (cudaFuncAttributeMaxDynamicSharedMemorySize) are set
+// to the largest size that any launch of the kernel takes, never to that of one
+// launch: contexts of other shapes on other host threads, or later nodes of the same
+// graph, would otherwise lower the limit before the launch that needs it.
+
 // Acceptance tables of a ladder k[0..K) (host FP64, integer results), 16 words
 // per ladder position: [0..2] Metropolis thresholds for S h = 2, 4, 6, [8..14]
 // heat-bath thresholds for h = 6 - 2 n, the rest zero.  False if the ladder is

@@ -2,6 +2,8 @@
 the plain kernel, at the sizes where they can go wrong: edges of tiles, chunks and
 row blocks, remainders, the smallest and largest of their range.  Integers bit for
 bit."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -221,3 +223,48 @@ def test_long_calls_on_few_slots_are_cut_by_time():
     for _ in range(6):
         parts.qsg_sweep(100000)
     assert np.array_equal(whole.qsg_get_spins(0), parts.qsg_get_spins(0))
+
+
+# pairs of shapes whose launches share a kernel instance and need different amounts of
+# shared memory above 48 KB: resident slots, ladder decisions, one-time sums
+SHARED = [("qsg_sweep", Q.Shape(16, 50, 1, 1, 1), Q.Shape(16, 64, 1, 1, 1)),
+          ("qsg_tempering_swap", Q.Shape(2, 2, 1, 1, 40), Q.Shape(2, 2, 1, 1, 128)),
+          ("qsg_measure_correlators", Q.Shape(24, 128, 1, 6, 1), Q.Shape(24, 128, 1, 7, 1))]
+
+
+@pytest.mark.parametrize("call,small,large", SHARED)
+def test_threads_with_contexts_of_different_sizes(call, small, large):
+    """Two host threads, each with its own context and stream: a launch of one must not
+    lower the shared-memory limit that the other has just set."""
+    torch = pytest.importorskip("torch")
+    errors, start = [], threading.Barrier(2)
+
+    def work(shape):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                ctx = _context(shape, 3, np.linspace(0.25, 0.35, shape.n_k))
+                start.wait()
+                for _ in range(4000):
+                    getattr(ctx, call)()
+                ctx.qsg_get_spins(0)
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in (small, large)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+
+
+def test_graph_of_resident_groups_of_different_sizes():
+    shapes = [Q.Shape(12, 160, 64, 2, 30, Q.HEATBATH), Q.Shape(12, 144, 64, 2, 30, Q.HEATBATH)]
+    lads = [np.linspace(0.25, 0.35, 30)] * 2
+    graphed, direct = Q.Context(shapes), Q.Context(shapes)
+    graphed.qsg_set_option(Q.OPT_GRAPH, 4)
+    for ctx in (graphed, direct):
+        ctx.qsg_init_samples(5, lads)
+        ctx.qsg_sweep(9)
+    for g in range(2):
+        assert np.array_equal(graphed.qsg_get_spins(g), direct.qsg_get_spins(g))
