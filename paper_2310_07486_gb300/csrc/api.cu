@@ -12,6 +12,7 @@
 
 #include "qsg.h"
 #include "qsg_launch.h"
+#include "side_streams.h"
 
 using namespace qsg;
 
@@ -249,11 +250,7 @@ struct qsg_ctx {
     unsigned long long graph_launches = 0;  // kernels per replay
     bool base_valid = false;
     std::string last_cuda;
-    // one stream per group for the concurrent multi-group mode, with the fork
-    // and join events that order them against the context's stream
-    std::vector<cudaStream_t> side;
-    std::vector<cudaEvent_t> joins;
-    cudaEvent_t fork = nullptr;
+    SideStreams side;  // of the concurrent multi-group mode
     // qsg_read_correlators_async: the point on `stream` the finish and copies
     // on the caller's stream wait for, and their completion, which every later
     // writer of the correlator buffers waits for
@@ -274,9 +271,6 @@ struct qsg_ctx {
         if (h_flag) cudaFreeHost(h_flag);
         if (graph_exec) cudaGraphExecDestroy(graph_exec);
         if (cap_stream) cudaStreamDestroy(cap_stream);
-        for (cudaStream_t t : side) cudaStreamDestroy(t);
-        for (cudaEvent_t e : joins) cudaEventDestroy(e);
-        if (fork) cudaEventDestroy(fork);
     }
 };
 
@@ -515,37 +509,16 @@ static SweepMode sweep_mode(const qsg_ctx *ctx) {
     return MODE_CONCURRENT;  // 3, or automatic with several groups
 }
 
-// Run work(g, stream) for every group: those with side(g) each on a stream of its
-// own, forked from st, the others one after another on st; st continues after all
-// of them.  Groups share no data (but for the correlator scratch, see
-// qsg_measure_correlators), so only each group's own work is ordered.
+// SideStreams::run over the context's groups.  Groups share no data (but for the
+// correlator scratch, see qsg_measure_correlators), so only each group's own work is
+// ordered.
 extern "C++" {
 template <class Side, class Work>
 static qsg_status on_side_streams(qsg_ctx *ctx, cudaStream_t st, Side side, Work work) {
-    const size_t ng = ctx->groups.size();
-    if (!ctx->fork) QSG_CUDA(ctx, cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming));
-    while (ctx->side.size() < ng) {
-        cudaStream_t t = nullptr;
-        cudaEvent_t e = nullptr;
-        QSG_CUDA(ctx, cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
-        ctx->side.push_back(t);
-        QSG_CUDA(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        ctx->joins.push_back(e);
-    }
-    QSG_CUDA(ctx, cudaEventRecord(ctx->fork, st));
-    for (size_t gi = 0; gi < ng; ++gi) {
-        const Group &g = ctx->groups[gi];
-        if (!side(g)) continue;
-        QSG_CUDA(ctx, cudaStreamWaitEvent(ctx->side[gi], ctx->fork, 0));
-        if (qsg_status s = work(g, ctx->side[gi])) return s;
-        QSG_CUDA(ctx, cudaEventRecord(ctx->joins[gi], ctx->side[gi]));
-    }
-    for (const Group &g : ctx->groups)
-        if (!side(g))
-            if (qsg_status s = work(g, st)) return s;
-    for (size_t gi = 0; gi < ng; ++gi)
-        if (side(ctx->groups[gi])) QSG_CUDA(ctx, cudaStreamWaitEvent(st, ctx->joins[gi], 0));
-    return QSG_OK;
+    const std::vector<Group> &gs = ctx->groups;
+    return ctx->side.run(
+        gs.size(), st, [&](size_t i) { return side(gs[i]); }, [&](size_t i, cudaStream_t t) { return work(gs[i], t); },
+        [&](cudaError_t e) { return cuda_fail(ctx, e); });
 }
 }  // extern "C++"
 
