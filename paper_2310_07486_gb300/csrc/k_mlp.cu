@@ -33,6 +33,7 @@
 
 #include <cuda_bf16.h>
 
+#include "coop_launch.h"
 #include "qsg_launch.h"
 
 namespace qsg {
@@ -439,15 +440,18 @@ cudaError_t launch_mlp_steps(float *P, float *M, float *V, const float *X, const
     if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 2 * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
     // a block per unit, and one for as many items of the parameter sums as it has
-    // teams; one block per SM at most (the blocks wait for one another)
+    // teams; one block per SM at most (the blocks wait for one another).  The sums do
+    // not depend on the number of blocks.
     const int units = (batch + kUnit - 1) / kUnit, share = (kItems + kTeams - 1) / kTeams;
     int blocks = units > share ? units : share;
     if (blocks > nsm) blocks = nsm;
     unsigned limit = kDefaultWaitLimit;
     void *args[] = {&P, &M, &V, &X, &T, &idx, &steps, &batch, &act, &grad_out, &adam, &lr, &corr, &loss_out, &sync, &limit};
     count_launches(1);
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_mlp_train), dim3((unsigned)blocks),
-                                       dim3(kMlpThreads), args, (size_t)sm, st);
+    return launch_resident_grid(blocks, [&](int n) {
+        return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_mlp_train), dim3((unsigned)n),
+                                           dim3(kMlpThreads), args, (size_t)sm, st);
+    });
 }
 
 // ---------------------------------------------------------------------------
