@@ -320,7 +320,9 @@ struct Divisor {
         y = __drcp_rn(by);
         yl = __dmul_rn(__fma_rn(-d, y, 1.0), y);
     }
+    // (by zero, with the count of measurements set to zero: the infinity or NaN of a division)
     __device__ __forceinline__ double into(double x) const {
+        if (d == 0.0) return __ddiv_rn(x, d);
         const double q = __fma_rn(x, y, __dmul_rn(x, yl));
         return __fma_rn(__fma_rn(-q, d, x), y, q);
     }

@@ -449,8 +449,12 @@ __global__ void __launch_bounds__(32 * kFinishWarps) k_onetime_finish(Group g, d
         for (int r = 0; r < R; ++r) {
             const long long *Cr = g.Cacc + (((size_t)r * g.W * 64 + s) * K + j) * nl;
             long long part = 0;
-            for (int lag = lane; lag < nl; lag += 32) part += (lag == 0 || lag == nl - 1) ? Cr[lag] : 2 * Cr[lag];
-            cl = __dadd_rn(cl, (double)part);
+            if (nm != 0.0) {
+                for (int lag = lane; lag < nl; lag += 32) part += (lag == 0 || lag == nl - 1) ? Cr[lag] : 2 * Cr[lag];
+                cl = __dadd_rn(cl, (double)part);
+            } else {  // a count set to zero: C itself is infinite or NaN, and so is its sum
+                for (int lag = lane; lag < nl; lag += 32) cl = __dadd_rn(cl, __ddiv_rn((double)Cr[lag], 0.0));
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) cl = __dadd_rn(cl, __shfl_xor_sync(0xffffffffu, cl, o));
@@ -474,7 +478,8 @@ __global__ void __launch_bounds__(32 * kFinishWarps) k_onetime_finish(Group g, d
         o[3] = __ddiv_rn(G, 2.0 * nm * npair * Lt * LD);
         o[4] = has3 ? __ddiv_rn((double)g.T3acc[c], nm * ntrip * Lt * LD) : __longlong_as_double(0x7ff8000000000000LL);
         o[5] = has3 ? __ddiv_rn(F3, 6.0 * nm * ntrip * Lt * LD) : __longlong_as_double(0x7ff8000000000000LL);
-        o[6] = __ddiv_rn(__ddiv_rn(cl, __dmul_rn(__dmul_rn(nm, LD), Lt)), (double)R);
+        const double norm = nm != 0.0 ? __dmul_rn(__dmul_rn(nm, LD), Lt) : 1.0;
+        o[6] = __ddiv_rn(__ddiv_rn(cl, norm), (double)R);
     }
 }
 

@@ -268,3 +268,20 @@ def test_graph_of_resident_groups_of_different_sizes():
         ctx.qsg_sweep(9)
     for g in range(2):
         assert np.array_equal(graphed.qsg_get_spins(g), direct.qsg_get_spins(g))
+
+
+def test_finish_of_sums_over_a_count_set_to_zero_is_that_of_a_division():
+    """Infinities with the sums' signs, NaN for 0 / 0; chi_lin adds up the C of every lag
+    and replica."""
+    shape = Q.Shape(8, 10, 70, 2, 2, Q.HEATBATH, Q.APBC)
+    ctx = _context(shape, 15)
+    ctx.qsg_sweep(3)
+    ctx.qsg_measure_correlators()
+    ctx.qsg_set_counters(3, 0, 0)
+    got = ctx.qsg_read_correlators(0, raw=True)
+    with np.errstate(divide="ignore", invalid="ignore"):
+        C = got["C_raw"] / 0.0
+        assert np.array_equal(got["C"], C, equal_nan=True) and np.isinf(C).any()
+        assert np.array_equal(got["Q2"], got["Q2_raw"] / 0.0, equal_nan=True)
+        chi = ctx.qsg_read_onetime()["chi_lin"]
+        assert np.array_equal(chi, C.sum(axis=(0, 3)), equal_nan=True) and np.isnan(chi).any()
