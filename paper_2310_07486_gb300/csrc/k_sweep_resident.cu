@@ -44,7 +44,6 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_resident(const Group g, const
                                                             const uint32_t k1) {
     extern __shared__ __align__(128) uint64_t smem[];
     __shared__ uint64_t full;
-    __shared__ int gave_up;
     const int L = g.L, L2 = L * L, ncol = L2 / 2, Lt = g.Ltau, M = Lt / 2;
     const int s = blockIdx.x;
     const int c = (int)threadIdx.x % ncol, m0 = (int)threadIdx.x / ncol, mt = (int)blockDim.x / ncol;
@@ -53,7 +52,6 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_resident(const Group g, const
     const uint32_t bytes = 8u * (uint32_t)g.N;
     const uint32_t sweep0 = (sweep_base ? *sweep_base : 0u) + sweep_off;
     if (threadIdx.x == 0) {
-        gave_up = 0;
         bar_init(&full);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         fence_async_smem();
@@ -69,9 +67,9 @@ __global__ void __launch_bounds__(1024, 1) k_sweep_resident(const Group g, const
     const uint64_t apbc = g.boundary == 1 ? ~0ull : 0ull;
     __syncthreads();
     // a wait that gives up leaves the slot as it is, once the copy is no longer in flight
-    if (!__syncthreads_and(bar_wait(&full, 0u, g.wait_limit, &gave_up))) {
+    if (!block_and(bar_wait(&full, 0u, g.wait_limit))) {
         if (threadIdx.x == 0) {
-            bar_drain(&full, 0u);
+            bar_wait(&full, 0u, kDrainPolls);
             if (g.err) atomicExch(g.err, (int)DEVERR_TIMEOUT);
         }
         return;

@@ -64,19 +64,8 @@ __device__ __forceinline__ void bar_init(uint64_t *b) {
 __device__ __forceinline__ void bar_expect(uint64_t *b, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
 }
-// A flag in shared memory that any thread may set (32-bit addresses: a generic
-// pointer would take a register pair of the sweep's 72).
-__device__ __forceinline__ bool flag_set(const int *f) {
-    int v;
-    asm volatile("ld.volatile.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(smem_addr(f)) : "memory");
-    return v != 0;
-}
-__device__ __forceinline__ void set_flag(int *f, int v) {
-    asm volatile("st.volatile.shared.u32 [%0], %1;\n" ::"r"(smem_addr(f)), "r"(v) : "memory");
-}
-// Wait for the phase of the given parity; false after `limit` polls (*gave_up is
-// set then) or when another thread of the block has given up.
-__device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, unsigned limit, int *gave_up) {
+// Wait for the phase of the given parity; false after `limit` polls.
+__device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, unsigned limit) {
     const uint32_t a = smem_addr(b);
     for (; limit != 0; --limit) {
         uint32_t done;
@@ -85,20 +74,19 @@ __device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, unsigned 
                      : "r"(a), "r"(parity)
                      : "memory");
         if (done) return true;
-        if (flag_set(gave_up)) return false;
     }
-    set_flag(gave_up, 1);
     return false;
 }
-// Wait for a copy in flight before the block that it writes to ends.
-__device__ __forceinline__ void bar_drain(uint64_t *b, uint32_t parity) {
-    const uint32_t a = smem_addr(b);
-    uint32_t done = 0;
-    for (unsigned it = 0; it < kDrainPolls && !done; ++it)
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(a), "r"(parity)
-                     : "memory");
+// Block barrier with the conjunction of v.  Not the .aligned form of
+// __syncthreads_and: threads of one warp wait for different units' copies and may
+// arrive apart (that form let L = 6 blocks through early).
+__device__ __forceinline__ bool block_and(bool v) {
+    uint32_t r;
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.and.pred q, 0, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(r)
+                 : "r"((uint32_t)v)
+                 : "memory");
+    return r != 0;
 }
 // Bulk copies: 16-byte aligned on both sides, sizes multiples of 16 (a plane is
 // 8 L^2 bytes, L even).
@@ -208,8 +196,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     constexpr uint32_t kPlaneBytes = 8u * L2;
     extern __shared__ __align__(128) uint64_t smem[];
     __shared__ uint64_t full_all[P][4];
-    __shared__ int do_boundary[P];
-    __shared__ int gave_up, loaded[P];  // a wait gave up; groups of planes loaded by each unit
+    __shared__ int do_boundary[P], loaded[P];  // loaded: groups of planes, of each unit
     const uint32_t sweep = (sweep_base ? *sweep_base : 0u) + sweep_off;
     const int un = P == 1 ? 0 : (int)threadIdx.x / NT, c = (int)threadIdx.x - un * NT;
     const int bps1 = (nch + P - 1) / P, bps2 = (nch2 + P - 1) / P;  // blocks per slot
@@ -266,7 +253,6 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         load_group(2);
         load_group(3);
     }
-    if (threadIdx.x == 0) gave_up = 0;
     if (leader) loaded[un] = (b - a + 1) / 4 + 1;
     const Cols k(L, c);
     const Couplings J(g, w, k);
@@ -282,7 +268,11 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     uint4 ra = draw(a), rb = draw(a + 2);
     uint32_t carry = 0;
     __syncthreads();  // the barriers are initialised
-    if (active) bar_wait(&full[0], 0u, g.wait_limit, &gave_up);
+    // no wait of this thread gave up; from the first step's barrier on, of the block.
+    // (Leaving the loop, or looking at a flag in shared memory while waiting, made the
+    // compiler spill, and a frame in local memory alone costs a launch of few slots 2 us:
+    // the host bounds the polls of all steps together instead, see step_polls.)
+    bool ok = !active || bar_wait(&full[0], 0u, g.wait_limit);
     uint64_t W0[8], W1[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) W0[i] = W1[i] = 0;
@@ -299,7 +289,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         auto slot = [&](auto ic) -> uint64_t * { return ring + ((decltype(ic)::value + 1) & 15) * SLOT; };
 #define IC(N) std::integral_constant<int, Q + (N)>{}
         if (active && (!EDGE || q + 3 <= b))
-            bar_wait(&full[(m + 1) & 3], (uint32_t)((m + 1) >> 2) & 1u, g.wait_limit, &gave_up);
+            ok = bar_wait(&full[(m + 1) & 3], (uint32_t)((m + 1) >> 2) & 1u, g.wait_limit) && ok;
         auto own = [&](auto ic) {
             W0[decltype(ic)::value & 7] = slot(ic)[k.o0];
             W1[decltype(ic)::value & 7] = slot(ic)[k.o1];
@@ -331,8 +321,8 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
             if (!EDGE || q + 3 < b) col1(IC(3), r1.w, EDGE && q + 4 == Lt ? apbc : 0ull);
         }
         fence_async_smem();
-        __syncthreads();
-        if (leader && (!EDGE || m > 0) && !flag_set(&gave_up)) {
+        ok = block_and(ok);
+        if (leader && ok && (!EDGE || m > 0)) {
             store_group(m - 1);
             bulk_commit();
         }
@@ -346,7 +336,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
         rb = draw(q + 6);
         carry = r1.z;
         if (leader && (!EDGE || m > 0)) {
-            if (!flag_set(&gave_up)) {
+            if (ok) {
                 bulk_wait_read();
                 load_group(m + 3);
             } else {
@@ -379,7 +369,6 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     const int chn = ch + 1 == nu ? 0 : ch + 1;  // the chunk after the last is the first
     if (c == 0) {
         int flags = 0;
-        const bool ok = !flag_set(&gave_up);
         if (active) {
             if (ok) {
                 store_group(Mr - 1);
@@ -387,7 +376,7 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
                 bulk_commit();
             } else {
                 const int n = loaded[un];
-                for (int gi = max(n - 4, 0); gi < n; ++gi) bar_drain(&full[gi & 3], (uint32_t)(gi >> 2) & 1u);
+                for (int gi = max(n - 4, 0); gi < n; ++gi) bar_wait(&full[gi & 3], (uint32_t)(gi >> 2) & 1u, kDrainPolls);
                 if (err) atomicExch(err, (int)DEVERR_TIMEOUT);
             }
             bulk_wait_all();
@@ -413,6 +402,15 @@ __global__ void __launch_bounds__(P *L *L / 2) __maxnreg__(NREG)
     }
 }
 
+// Polls of a step's wait: a block whose wait gave up runs out its steps, each of which
+// may wait in vain, so that they share eight limits; but no less than 1,024 polls a wait
+// (a poll suspends the thread for a while), unless the limit itself is smaller.
+inline unsigned step_polls(unsigned limit, int steps) {
+    const unsigned long long share = 8ull * limit / (unsigned)(steps < 8 ? 8 : steps);
+    const unsigned long long least = limit < 1024u ? limit : 1024u;
+    return (unsigned)(share > least ? share : least);
+}
+
 // The launch of one sweep: nch chunks per slot for the first S1 slots, nch2 for
 // the others; with arrivals == nullptr only *resident is set, to (SMs x 64 + the
 // blocks of this instance an SM holds) x 64 + the chunks of a block.
@@ -434,9 +432,12 @@ cudaError_t launch_unit(const Group &g, int nch, int nch2, int S1, const uint32_
         *resident = (nsm * 64 + per) * 64 + P;
         return e;
     }
+    Group gw = g;
+    const int shortest = nch < nch2 ? nch : nch2;  // chunks of a slot
+    gw.wait_limit = step_polls(g.wait_limit, (g.Ltau / 2 + shortest - 1) / shortest / 2 + 2);
     const int blocks = S1 * ((nch + P - 1) / P) + (g.nslots - S1) * ((nch2 + P - 1) / P);
     count_launches(1);
-    kern<<<blocks, threads, sm, st>>>(g, nch, S1, nch2, sweep_base, sweep, (uint32_t)seed, (uint32_t)(seed >> 32),
+    kern<<<blocks, threads, sm, st>>>(gw, nch, S1, nch2, sweep_base, sweep, (uint32_t)seed, (uint32_t)(seed >> 32),
                                       arrivals, nch > nch2 ? nch : nch2, err);
     return cudaGetLastError();
 }
