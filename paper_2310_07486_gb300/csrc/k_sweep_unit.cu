@@ -51,7 +51,8 @@ int sweep_unit_chunks(const Group &g) {
     int best = 1;
     double best_cost = 1e300;
     const int most = g.Ltau / 16 < 1 ? 1 : g.Ltau / 16;
-    for (int n = most < P ? most : P; n <= most; n += P) {  // whole blocks of chunks
+    // whole blocks of chunks, and the most chunks there can be
+    for (int n = most < P ? most : P; n <= most; n = n < most && n + P > most ? most : n + P) {
         const long long blocks = (long long)g.nslots * ((n + P - 1) / P), rest = blocks % R;
         double waves = (double)(blocks / R);
         if (rest > 0) {

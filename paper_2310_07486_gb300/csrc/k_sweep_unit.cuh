@@ -32,8 +32,11 @@
 // A block serves chunks of one slot, so everything that depends on the slot is
 // uniform (the thresholds stay in uniform registers) and 72 registers suffice,
 // three blocks of 288 threads per SM at L = 24 (the ring of 74 KB allows three too).
-// L = 6 has 18 threads per chunk and runs 16 neighbouring chunks per block, in
-// lockstep, so that its warps are full (93 slots of L_tau = 1024: 50 -> 30 us).  From
+// Where 80 registers cost no resident block they are given, see unit_regs.
+// L = 6 has 18 threads per chunk and runs 14 neighbouring chunks per block, in
+// lockstep, so that its eight warps are full (92 slots of L_tau = 1024, us per sweep:
+// a chunk per block 50, 16 chunks in nine warps of 72 registers, which spill more, 34.0
+// Metropolis and 30.1 heat bath, 14 in eight warps of 80 27.1 and 25.5).  From
 // L = 10 on that is no gain: five chunks per block at L = 10 (L_tau = 736, 348 slots)
 // 100 against 96 us, four at L = 12 (L_tau = 256, 192 slots) 46 / 44, two at L = 14
 // (L_tau = 400, 64 slots) 37 / 31: what the idle lanes cost is less than the coarser
@@ -54,7 +57,18 @@ constexpr unsigned kDrainPolls = 1u << 24; // polls of the wait for copies in fl
 
 // Chunks per block.
 __host__ __device__ constexpr int units_per_block(int L) {
-    return L <= 6 ? 16 : 1;
+    return L <= 6 ? 14 : 1;
+}
+// Registers of a thread: 80, which nearly every size needs to be free of spills, where
+// as many blocks fit an SM as with 72 (by registers, 24 against 28 warps, or by the
+// ring), else 72.  72 / 80, us per sweep: L = 8, L_tau = 1024, 92 slots 33.0 / 31.6; L = 18,
+// L_tau = 1024, 64 slots 90.2 / 88.4; L = 22, L_tau = 512, 64 slots 62.7 / 61.0; L = 30, L_tau
+// = 512, 32 slots 68.6 / 66.2; L = 16, L_tau = 512, 96 slots 50.1 / 50.2.
+__host__ __device__ constexpr int unit_regs(int L) {
+    const int warps = (units_per_block(L) * L * L / 2 + 31) / 32;
+    const int ring = 227 * 1024 / (units_per_block(L) * kRing * L * L * 8 + 1280);
+    const int at72 = 28 / warps < ring ? 28 / warps : ring, at80 = 24 / warps < ring ? 24 / warps : ring;
+    return at80 >= at72 ? 80 : 72;
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -420,7 +434,7 @@ cudaError_t launch_unit(const Group &g, int nch, int nch2, int S1, const uint32_
     constexpr int P = units_per_block(L);
     constexpr int threads = P * L * L / 2;
     constexpr size_t sm = (size_t)P * kRing * L * L * sizeof(uint64_t);
-    auto kern = k_sweep_unit<ALGO, L, P, 72>;
+    auto kern = k_sweep_unit<ALGO, L, P, unit_regs(L)>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
