@@ -1,6 +1,7 @@
 // k_sweep_unit.cu -- host side of the fused sweep (k_sweep_unit.cuh): which groups
 // it serves and how their slots are cut into chunks of tau planes.
 #include <atomic>
+#include <cmath>
 
 #include "qsg_launch.h"
 
@@ -42,11 +43,20 @@ static void residency(const Group &g, int *nsm, int *per, int *chunks) {
 // L_tau = 2048, 256 slots; 1, 3, 4, 5, 7, 12, 16 chunks) the ratios agree within 4
 // %; seven chunks are the best of them, and the choice.  Chunks need not divide
 // L_tau: they differ by two planes at most.
+// Blocks of one warp (L = 8) are the load of one of an SM's four schedulers, so they are
+// counted per scheduler, and x of the `per` blocks there take (x / per)^0.9 of a full
+// wave.  Counted per SM, the choice for L_tau = 1024, 92 slots was 18 chunks in 31.4 us
+// per sweep, where 26 take 29.2 and the best count, 33, 28.7.
 int sweep_unit_chunks(const Group &g) {
     constexpr double kOverhead = 8.0, kThin = 0.45;
     int nsm = 0, per = 0, P = 1;
     residency(g, &nsm, &per, &P);
     if (nsm <= 0 || per <= 0) return 1;
+    const bool one_warp = P == 1 && g.L * g.L / 2 <= 32 && per >= 4;
+    if (one_warp) {
+        nsm *= 4;
+        per /= 4;
+    }
     const long long R = (long long)nsm * per;
     int best = 1;
     double best_cost = 1e300;
@@ -56,7 +66,8 @@ int sweep_unit_chunks(const Group &g) {
         const long long blocks = (long long)g.nslots * ((n + P - 1) / P), rest = blocks % R;
         double waves = (double)(blocks / R);
         if (rest > 0) {
-            const double part = (double)((rest + nsm - 1) / nsm) / per;
+            double part = (double)((rest + nsm - 1) / nsm) / per;
+            if (one_warp) part = std::pow(part, 0.9);
             waves += part > kThin ? part : kThin;
         }
         const double cost = waves * ((double)g.Ltau / n + kOverhead);
