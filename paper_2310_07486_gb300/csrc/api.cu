@@ -544,18 +544,6 @@ static bool few_large_slots(const Group &g) {
     return resident > (chunked > 9.3 ? chunked : 9.3);
 }
 
-// Several sweeps of a group in one launch, the slots in shared memory: where a
-// slot fits an SM, the slots keep the SMs busy and no launch option asks for another form.  A graph of fewer
-// than kResidentGraphSlots slots keeps one kernel node per sweep: such a replay
-// leaves the GPU idle either way, and its launch count is part of what callers
-// see (qsg_kernel_launches).
-constexpr int kResidentGraphSlots = 8;
-static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
-    if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
-    if (sb && g.nslots < kResidentGraphSlots) return false;
-    return sweep_resident_fits(g) && !(sweep_unit_supported(g) && few_large_slots(g));
-}
-
 // Very few words without a graph: the plain kernel's two short launches take less
 // than a chunk's chain of steps.  us per sweep, plain / chunked: L = 12, L_tau = 330, 2
 // slots 8.3 / 12.4; L = 24, L_tau = 100, 6 slots 12.4 / 14.7; L = 8, L_tau = 700, 8 slots 12.4
@@ -566,12 +554,38 @@ static bool plain_pays(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
     return (double)g.N * (double)g.nslots < (g.L == 6 ? 1.5e6 : 4e5);
 }
 
+// Several sweeps of a group in one launch, the slots in shared memory: where a
+// slot fits an SM, the slots keep the SMs busy and no launch option asks for another
+// form.  A graph of fewer than kResidentGraphSlots slots keeps one kernel node per
+// sweep: its launch count is part of what callers see (qsg_kernel_launches).
+constexpr int kResidentGraphSlots = 8;
+static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
+    if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
+    if (sb && g.nslots < kResidentGraphSlots) return false;
+    return sweep_resident_fits(g) && !(sweep_unit_supported(g) && few_large_slots(g));
+}
+
+// Such a graph of small slots still has them resident, for a sweep at a time: a chunk's
+// chain of steps takes 8.3 us at least, a launch of this form 2.1 and 0.74 per 1,000 words
+// of a slot (L_tau = 16, us per sweep: L = 6 10.3 / 3.9, L = 8 8.4 / 4.1, L = 12 9.2 / 5.2, L =
+// 16 8.3 / 6.4, L = 20 10.1 / 8.6).
+constexpr int kResidentSweepWords = 8192;
+static bool resident_by_sweep(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
+    if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
+    return sb && g.nslots < kResidentGraphSlots && g.N <= kResidentSweepWords && sweep_resident_fits(g);
+}
+
 // `count` sweeps of one group on one stream, indices first .. first + count - 1
 // (added to *sb when sb is given).
 static qsg_status group_sweeps(qsg_ctx *ctx, const Group &g, const uint32_t *sb, uint32_t first, int count,
                                cudaStream_t st) {
     if (use_resident(ctx, g, sb)) {
         QSG_CUDA(ctx, launch_sweep_resident(g, count, sb, first, ctx->seed, st));
+        return QSG_OK;
+    }
+    if (resident_by_sweep(ctx, g, sb)) {
+        for (int i = 0; i < count; ++i)
+            QSG_CUDA(ctx, launch_sweep_resident(g, 1, sb, first + (uint32_t)i, ctx->seed, st));
         return QSG_OK;
     }
     const bool fused = ctx->sweep_kernel != 1 && sweep_fused_supported(g, ctx->chunk) && !plain_pays(ctx, g, sb);

@@ -285,3 +285,19 @@ def test_finish_of_sums_over_a_count_set_to_zero_is_that_of_a_division():
         assert np.array_equal(got["Q2"], got["Q2_raw"] / 0.0, equal_nan=True)
         chi = ctx.qsg_read_onetime()["chi_lin"]
         assert np.array_equal(chi, C.sum(axis=(0, 3)), equal_nan=True) and np.isnan(chi).any()
+
+
+@pytest.mark.parametrize("L,Ltau,slots", [(6, 16, 1), (8, 16, 3), (16, 32, 7), (20, 16, 2), (24, 16, 7), (4, 32, 2)])
+@pytest.mark.parametrize("algo,boundary", [(Q.METROPOLIS, Q.APBC), (Q.HEATBATH, Q.PBC)])
+def test_graphs_of_few_small_slots_match_the_plain_kernel(L, Ltau, slots, algo, boundary):
+    """One kernel per sweep as the larger slots have; the largest resident one (8,192 words)
+    and one beyond it."""
+    shape = Q.Shape(L, Ltau, 64, 1, slots, algo, boundary)
+    plain, graph = _context(shape, 3, SWEEP_KERNEL=1), _context(shape, 3, GRAPH=4)
+    for n in (4, 9, 1):
+        plain.qsg_sweep(n)
+        graph.qsg_sweep(n)
+    assert np.array_equal(plain.qsg_get_spins(0), graph.qsg_get_spins(0))
+    before = Q.qsg_kernel_launches()
+    graph.qsg_sweep(4)
+    assert Q.qsg_kernel_launches() - before == 4 + 2  # the counter set after direct sweeps, and advanced
