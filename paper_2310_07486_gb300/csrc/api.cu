@@ -558,10 +558,14 @@ static bool plain_pays(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
 // slot fits an SM, the slots keep the SMs busy and no launch option asks for another
 // form.  A graph of fewer than kResidentGraphSlots slots keeps one kernel node per
 // sweep: its launch count is part of what callers see (qsg_kernel_launches).
+// Where the plain kernel is the other choice (plain_pays), its two launches take 8.3 us up
+// to 140,000 words, a resident sweep 0.6 per 1,000 words of a slot (plain / resident: L =
+// 20, L_tau = 34 8.3 / 7.9, L = 12, L_tau = 100 8.3 / 8.7, L = 18, L_tau = 50 8.3 / 10.0).
 constexpr int kResidentGraphSlots = 8;
 static bool use_resident(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
     if (ctx->sweep_kernel != 0 || ctx->chunk != 0 || ctx->tail != 0 || g_wavefront_variant != 0) return false;
     if (sb && g.nslots < kResidentGraphSlots) return false;
+    if (plain_pays(ctx, g, sb) && (double)g.N * g.nslots < 1.4e5 && g.N > 13900) return false;
     return sweep_resident_fits(g) && !(sweep_unit_supported(g) && few_large_slots(g));
 }
 

@@ -301,3 +301,13 @@ def test_graphs_of_few_small_slots_match_the_plain_kernel(L, Ltau, slots, algo, 
     before = Q.qsg_kernel_launches()
     graph.qsg_sweep(4)
     assert Q.qsg_kernel_launches() - before == 4 + 2  # the counter set after direct sweeps, and advanced
+
+
+@pytest.mark.parametrize("L,Ltau,K,launches", [(18, 50, 1, 6), (12, 100, 8, 6), (20, 34, 8, 1), (18, 50, 16, 1)])
+def test_direct_sweeps_of_few_words_take_the_cheaper_form(L, Ltau, K, launches):
+    """Extents that are no multiple of 16: two plain launches per sweep for few words in
+    large slots, else one resident launch for the call."""
+    ctx = _context(Q.Shape(L, Ltau, 64, 1, K, Q.HEATBATH, Q.PBC), 3)
+    before = Q.qsg_kernel_launches()
+    ctx.qsg_sweep(3)
+    assert Q.qsg_kernel_launches() - before == launches
