@@ -242,9 +242,15 @@ __global__ void __launch_bounds__(kShortThreads) k_gram_short(Group g, int p0, c
 // tiles: L = 8, L_tau = 32 11 / 65, 128 20 / 71, 256 42 / 87; L = 10, L_tau = 128 29 / 73,
 // 256 79 / 91; L = 12, L_tau = 128 40 / 77, 192 58 / 94, 256 111 / 97; L = 16, L_tau = 128
 // 51 / 77, 192 112 / 95.  From two whole row blocks (L_tau = 256) on the tensor units
-// have steps to overlap and keep the work.
-static bool use_short(const Group &g) {
-    return g.nwx <= kShortWords && g.Ltau < 2 * 128 && g.nwx * g.Ltau <= 576;
+// have steps to overlap and keep the work.  So they do where the samples are few: the
+// rows of one sample are a serial walk here, and a tile takes no longer for 152 samples
+// than for one.  The line lies at L_tau (2 + 1.9 words) sample bits, 256 at least: whole
+// measurements, us here / with tensor tiles, L = 4, L_tau = 32 22 / 18 for 128 bits; L = 8, L_tau = 64 24 / 19 for 128 bits, 26 / 42 for 1,024; L = 8,
+// L_tau = 240 45 / 37 for 512, 46 / 54 for 1,024; L = 16, L_tau = 128 48 / 36 for 512, 62 / 54
+// for 1,024, 91 / 104 for 2,048.
+static bool use_short(const Group &g, int nsamples) {
+    if (g.nwx > kShortWords || g.Ltau >= 2 * 128 || g.nwx * g.Ltau > 576) return false;
+    return nsamples >= 256 && 10LL * nsamples >= (long long)g.Ltau * (20 + 19 * g.nwx);
 }
 
 static cudaError_t launch_gram_short(const Group &g, int p0, int npairs, const uint64_t *P, cudaStream_t st) {
@@ -288,7 +294,7 @@ cudaError_t launch_measure(const Group &g, uint64_t *scratch, size_t scratch_wor
                       st>>>(g, p0, np, scratch);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        if (tensor && use_short(g)) {
+        if (tensor && use_short(g, np * g.R * 64)) {
             e = launch_gram_short(g, p0, np, scratch, st);
         } else if (tensor) {
             e = launch_gram_tc(g, p0, np, scratch, status, wait_limit, st);

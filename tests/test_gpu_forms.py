@@ -311,3 +311,18 @@ def test_direct_sweeps_of_few_words_take_the_cheaper_form(L, Ltau, K, launches):
     before = Q.qsg_kernel_launches()
     ctx.qsg_sweep(3)
     assert Q.qsg_kernel_launches() - before == launches
+
+
+@pytest.mark.parametrize("L,Ltau,R,K", [(8, 64, 2, 1), (8, 64, 2, 2), (16, 128, 2, 9), (16, 128, 2, 10), (4, 240, 2, 7),
+                                        (12, 16, 2, 1), (12, 18, 2, 1)])
+def test_short_extents_on_both_sides_of_the_sample_line(L, Ltau, R, K):
+    """Tensor tiles for few sample bits, the integer form for many: the same sums."""
+    shape = Q.Shape(L, Ltau, 64, R, K, Q.HEATBATH, Q.APBC)
+    got = []
+    for kernel in (Q.CORR_TENSOR, Q.CORR_INTEGER):
+        ctx = _context(shape, 5, CORR_KERNEL=kernel)
+        ctx.qsg_sweep(2)
+        ctx.qsg_measure_correlators()
+        got.append(ctx.qsg_read_correlators(0, raw=True))
+    for key in ("C_raw", "Q2_raw", "q2_raw"):
+        assert np.array_equal(got[0][key], got[1][key]), key
