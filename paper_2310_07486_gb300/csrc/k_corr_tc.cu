@@ -205,6 +205,7 @@ struct GramPlan {
     int nsingle;  // units of one offset per sample, the first of them e = e_single
     int e_single;
     int e_mirror;  // offset whose steps stop at nb / 2 (each tile is the transpose of another), or -1
+    int triangle;  // one row block: only the tile of t2 >= t1, without the wrap past L_tau
     int nstages;
     int flush;     // steps after which the FP32 sums must be folded
     uint32_t unit;  // 1 (see spread_e4m3)
@@ -229,9 +230,9 @@ __device__ __forceinline__ Unit unit_of(const GramPlan &pl, int u) {
     } else {
         r.sample = (u - np) / pl.nsingle;
         r.e = pl.e_single + (u - np) - r.sample * pl.nsingle;
-        r.mirror = r.e == pl.e_mirror;
+        r.mirror = pl.triangle || r.e == pl.e_mirror;
     }
-    r.steps = r.mirror ? pl.nb / 2 : pl.nb;
+    r.steps = r.mirror && !pl.triangle ? pl.nb / 2 : pl.nb;
     return r;
 }
 __device__ __forceinline__ int unit_count(const GramPlan &pl) { return pl.nsamples * (pl.npair + pl.nsingle); }
@@ -399,7 +400,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint64_t w[2 * NC];
 #pragma unroll
         for (int k = 0; k < 2 * NC; ++k) w[k] = k < nwx ? __ldg(now.src + k) : 0ull;
-        const uint32_t one = isB ? 0x30303030u : 0x38383838u, unit = pl.unit;
+        // (a triangle leaves out the rows that wrap: +-0)
+        const uint32_t one = isB ? (pl.triangle && row >= Lt ? 0u : 0x30303030u) : 0x38383838u, unit = pl.unit;
         // the first use of a stage waits for the phase before the first
         // (complete at initialisation)
         uint32_t par = 1u;
@@ -535,9 +537,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                             int cv = __float2int_rn(vc[k]), lag = d;
                             unsigned qv = (unsigned)vq[k];
                             if (un.mirror && d >= half) {
-                                // half the row blocks: an element past L_tau / 2 is
-                                // the wrapped pair of lag L_tau - d, and one at
-                                // L_tau / 2 stands for both directions
+                                // half the row blocks, or the tile of t2 >= t1: an
+                                // element past L_tau / 2 is the wrapped pair of lag
+                                // L_tau - d, and one at L_tau / 2 stands for both
+                                // directions
                                 lag = Lt - d;
                                 if (d == half) qv *= 2u;
                                 cv = d == half ? (g.boundary == 1 ? 0 : 2 * cv) : (g.boundary == 1 ? -cv : cv);
@@ -682,6 +685,19 @@ GramPlan gram_plan(const Group &g, int nsamples) {
     // where L_tau / 2 is a whole number of blocks, the tiles (i, e) and
     // (i + nb / 2, e) of the last offset are each other's transpose
     pl.e_mirror = half % kTile == 0 && pl.nb > 1 ? half / kTile : -1;
+    // One row block of a lattice whose units have one offset and stream both operands (L >
+    // 24): the triangle of t2 >= t1 holds every pair of rows once, the offsets past L_tau
+    // / 2 standing for the wrapped ones, in one tile where the offsets up to L_tau / 2 take
+    // two (L_tau = 86 .. 128).  2,048 sample bits, us of a measurement with the offsets / the
+    // triangle: L = 26, L_tau = 112 214 / 159, L = 32, L_tau = 112 312 / 234.  With two row
+    // blocks (three tiles for four) the shorter units cost more than the tile saves (L = 26,
+    // L_tau = 160 302 / 371), and so they do with resident column blocks (L = 24, L_tau = 86
+    // 129 / 144).
+    pl.triangle = pl.nb == 1 && ne == 2 && nc > kPairNc;
+    if (pl.triangle) {
+        pl.e_single = 0;
+        pl.nsingle = 1;
+    }
     // resident: the slots' chunks, and no more stages than a stage's release
     // can stand for (it must imply that of the slot to be overwritten, block_slots
     // - 1 steps back); streamed: A and B chunks

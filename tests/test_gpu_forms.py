@@ -326,3 +326,22 @@ def test_short_extents_on_both_sides_of_the_sample_line(L, Ltau, R, K):
         got.append(ctx.qsg_read_correlators(0, raw=True))
     for key in ("C_raw", "Q2_raw", "q2_raw"):
         assert np.array_equal(got[0][key], got[1][key]), key
+
+
+@pytest.mark.parametrize("L,Ltau", [(4, 86), (8, 100), (12, 128), (16, 88), (18, 84), (20, 90), (24, 128), (26, 86), (28, 126),
+                                    (26, 128), (26, 130), (32, 160), (30, 254), (32, 256), (26, 84), (28, 258)])
+@pytest.mark.parametrize("boundary", [Q.PBC, Q.APBC])
+def test_tiles_of_one_and_two_row_blocks(L, Ltau, boundary):
+    """The triangle of row pairs at the ends of its range and the offsets beyond them, in the
+    lags, in the largest sums (all spins equal) and for few sample bits."""
+    shape = Q.Shape(L, Ltau, 64, 2, 1, Q.HEATBATH, boundary)
+    got = []
+    for kernel in (Q.CORR_TENSOR, Q.CORR_INTEGER):
+        ctx = _context(shape, 5, CORR_KERNEL=kernel)
+        ctx.qsg_sweep(2)
+        ctx.qsg_measure_correlators()
+        ctx.qsg_set_spins(0, np.zeros((shape.slots, Ltau, L, L), dtype=np.uint64))
+        ctx.qsg_measure_correlators()
+        got.append(ctx.qsg_read_correlators(0, raw=True))
+    for key in ("C_raw", "Q2_raw", "q2_raw"):
+        assert np.array_equal(got[0][key], got[1][key]), key
