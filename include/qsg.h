@@ -91,12 +91,15 @@ typedef struct {
     int32_t reserved;   /* must be 0 */
 } qsg_shape;
 
-/* Bytes of device workspace needed for these groups (0 on invalid shapes). */
+/* Bytes of device workspace for these groups (0 on invalid shapes).  With several
+ * groups this has room for a correlator scratch of its own for each small group (up to
+ * 64 MB, 1 GB in all), which lets their measurements overlap. */
 size_t qsg_workspace_bytes(const qsg_shape *shapes, int32_t n_groups);
 
 /* Create a context over a caller-owned device workspace (256-byte aligned,
- * at least qsg_workspace_bytes() bytes) on CUDA stream `cuda_stream`
- * (a cudaStream_t, may be NULL for the legacy default stream). */
+ * qsg_workspace_bytes() bytes; less by the small groups' own scratch serves too, then
+ * all groups share one and are measured in turn, with the same results) on CUDA stream
+ * `cuda_stream` (a cudaStream_t, may be NULL for the legacy default stream). */
 qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, void *d_workspace,
                       size_t workspace_bytes, void *cuda_stream);
 void qsg_destroy(qsg_ctx *ctx);

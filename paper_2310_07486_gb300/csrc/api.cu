@@ -79,9 +79,10 @@ struct PlanBuffers {
     uint32_t *sweep_base = nullptr;
 };
 
-// Walk the workspace: when base is null only the size is computed.
-size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, size_t *scratch_words,
-             PlanBuffers *pb = nullptr) {
+// Walk the workspace: when base is null only the size is computed.  own_scratch: small
+// groups of several have a correlator scratch of their own, else all share one.
+size_t carve(std::vector<Group> &gs, bool own_scratch, char *base, int **err, uint64_t **scratch,
+             size_t *scratch_words, PlanBuffers *pb = nullptr) {
     size_t off = 0;
     auto take = [&](size_t bytes) -> char * {
         char *p = base ? base + off : nullptr;
@@ -91,7 +92,7 @@ size_t carve(std::vector<Group> &gs, char *base, int **err, uint64_t **scratch, 
     *err = (int *)take(sizeof(int) * 4);
     size_t sw = 0;   // words of the shared scratch
     size_t own = 0;  // bytes of the groups' own
-    const bool several = gs.size() > 1;
+    const bool several = own_scratch && gs.size() > 1;
     for (auto &g : gs) {
         g.S = (uint64_t *)take(sizeof(uint64_t) * (size_t)g.nslots * g.N);
         g.Jx = (uint64_t *)take(sizeof(uint64_t) * (size_t)g.W * g.L * g.L);
@@ -350,6 +351,13 @@ static qsg_status upload_plan(qsg_ctx *c) {
     return QSG_OK;
 }
 
+static size_t workspace_size(std::vector<Group> gs, bool own_scratch) {
+    int *e;
+    uint64_t *s;
+    size_t sw;
+    return carve(gs, own_scratch, nullptr, &e, &s, &sw);
+}
+
 extern "C" {
 
 size_t qsg_workspace_bytes(const qsg_shape *shapes, int32_t n_groups) {
@@ -359,10 +367,7 @@ size_t qsg_workspace_bytes(const qsg_shape *shapes, int32_t n_groups) {
         if (!valid_shape(shapes[i])) return 0;
         gs.push_back(describe(shapes[i], i));
     }
-    int *e;
-    uint64_t *s;
-    size_t sw;
-    return carve(gs, nullptr, &e, &s, &sw);
+    return workspace_size(gs, true);
 }
 
 qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, void *d_workspace,
@@ -372,14 +377,19 @@ qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, 
     if (n_groups < 1 || n_groups > 255) return QSG_ERR_ARG;
     for (int i = 0; i < n_groups; ++i)
         if (!valid_shape(shapes[i])) return QSG_ERR_SHAPE;
-    const size_t need = qsg_workspace_bytes(shapes, n_groups);
-    if (!d_workspace || workspace_bytes < need || ((uintptr_t)d_workspace % kAlign) != 0) return QSG_ERR_WORKSPACE;
+    std::vector<Group> gs;
+    for (int i = 0; i < n_groups; ++i) gs.push_back(describe(shapes[i], i));
+    // a workspace without room for the groups' own scratch serves, too
+    const bool own_scratch = workspace_bytes >= workspace_size(gs, true);
+    if (!d_workspace || (!own_scratch && workspace_bytes < workspace_size(gs, false)) ||
+        ((uintptr_t)d_workspace % kAlign) != 0)
+        return QSG_ERR_WORKSPACE;
     qsg_ctx *c = new qsg_ctx();
     c->shapes.assign(shapes, shapes + n_groups);
-    for (int i = 0; i < n_groups; ++i) c->groups.push_back(describe(shapes[i], i));
+    c->groups = gs;
     c->ws = (char *)d_workspace;
     c->ws_bytes = workspace_bytes;
-    carve(c->groups, c->ws, &c->d_err, &c->scratch, &c->scratch_words, &c->pb);
+    carve(c->groups, own_scratch, c->ws, &c->d_err, &c->scratch, &c->scratch_words, &c->pb);
     for (Group &g : c->groups) g.err = c->d_err;
     c->stream = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaHostAlloc((void **)&c->h_flag, 2 * sizeof(int), cudaHostAllocDefault);

@@ -230,7 +230,7 @@ class Context:
     Methods map one-to-one onto the C entry points of the same name.
     """
 
-    def __init__(self, shapes, device=None, stream=None):
+    def __init__(self, shapes, device=None, stream=None, workspace_bytes=None):
         import torch
         self.lib = load_library()
         self.shapes = list(shapes)
@@ -238,6 +238,7 @@ class Context:
         nbytes = qsg_workspace_bytes(self.shapes)
         if nbytes == 0:
             raise QSGError(-2, "qsg_workspace_bytes")
+        nbytes = nbytes if workspace_bytes is None else int(workspace_bytes)  # less may serve, see qsg_create
         self.device = torch.device(device) if device is not None else torch.device("cuda", torch.cuda.current_device())
         # torch's caching allocator returns blocks aligned to at least 512 bytes
         self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.device)

@@ -345,3 +345,31 @@ def test_tiles_of_one_and_two_row_blocks(L, Ltau, boundary):
         got.append(ctx.qsg_read_correlators(0, raw=True))
     for key in ("C_raw", "Q2_raw", "q2_raw"):
         assert np.array_equal(got[0][key], got[1][key]), key
+
+
+def test_workspace_without_the_groups_own_scratch():
+    """Two small groups in a workspace that holds one correlator scratch: the same results;
+    a byte less is refused."""
+    shapes = [Q.Shape(8, 48, 70, 3, 4, Q.HEATBATH), Q.Shape(12, 64, 64, 4, 6, Q.HEATBATH, Q.APBC)]
+    lads = [np.linspace(0.25, 0.3, s.n_k) for s in shapes]
+    own = [s.n_replicas * 64 * s.Ltau * ((s.L ** 2 + 63) // 64) * s.words * s.n_k * 8 for s in shapes]
+    features = max(s.words for s in shapes) * 64 * 64 * 4
+    full = Q.qsg_workspace_bytes(shapes)
+    lean = full - sum(own) - features + max(own)
+    assert all(v % 256 == 0 for v in own) and max(own) > features
+    with pytest.raises(Q.QSGError) as e:
+        Q.Context(shapes, workspace_bytes=lean - 1)
+    assert e.value.status == -6
+    got = []
+    for size in (full, full - 1, lean):
+        ctx = Q.Context(shapes, workspace_bytes=size)
+        ctx.qsg_init_samples(9, lads)
+        for _ in range(2):
+            ctx.qsg_sweep(2)
+            ctx.qsg_measure_correlators()
+        got.append([(ctx.qsg_read_correlators(g, raw=True), ctx.qsg_read_onetime(g)["raw"], ctx.qsg_sample_features(g))
+                    for g in range(2)])
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert all(np.array_equal(a[0][k], b[0][k]) for k in a[0])
+            assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
