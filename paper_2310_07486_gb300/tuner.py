@@ -32,9 +32,9 @@ _NAMES = {Q.OPT_CHUNK: "chunk", Q.OPT_WAVEFRONT_VARIANT: "variant", Q.OPT_PERSIS
           Q.OPT_GRAPH: "graph", Q.OPT_TAIL: "tail", Q.OPT_UNITS_PER_BLOCK: "upb"}
 DEFAULTS = {"chunk": 0, "variant": 0, "persistent": 0, "graph": 0, "tail": 0, "upb": 0}
 UPB = [1, 2, 4, 8, 16]  # units per block of the generic kernel, tried after the first stage
-COMPILED_L = (8, 12, 16, 20, 24)  # sizes whose units per block are tried only for the generic form
+COMPILED_L = (8, 12, 16, 20, 24)  # the sizes of the simulation table
 TAILS = [0, 16, 24, 28, 32, 40, 48, 64]  # slots swept in quarter-length chunks, tried after the rest
-VARIANTS = [0, 1, 2, 3]  # forms of the wavefront kernel (QSG_OPT_WAVEFRONT_VARIANT)
+VARIANTS = [0, 2, 3]  # forms of the wavefront kernel (QSG_OPT_WAVEFRONT_VARIANT; 1 is the same kernel as 3)
 
 
 def _library_id() -> str:
@@ -78,9 +78,16 @@ def candidates(shapes, sweeps_per_call, space=None):
 
 
 def uses_generic_kernel(shapes, variant):
-    """True if the units per block of the generic wavefront kernel are worth
-    trying: the generic form is asked for, or some size is not in COMPILED_L."""
+    """True if the generic form is asked for or some size is outside the simulation
+    table (for those with L >= 6 there is a compiled kernel all the same, see
+    reads_units_per_block)."""
     return variant == 2 or any(s.L not in COMPILED_L for s in shapes)
+
+
+def reads_units_per_block(shapes, variant):
+    """True if some group is swept by the generic wavefront kernel, the only one that
+    reads the units per block: it is asked for, or L < 6, which has no compiled one."""
+    return uses_generic_kernel(shapes, variant) and (variant == 2 or any(s.L < 6 for s in shapes))
 
 
 def apply(ctx, choice: dict) -> None:
@@ -150,7 +157,7 @@ def tune(ctx, sweeps_per_call=10, reps=3, cache_path=DEFAULT_CACHE, use_cache=Tr
         # units per block of the generic kernel, with the best launch so far
         if table:
             t0, first = min(table, key=lambda tc: tc[0])
-            if uses_generic_kernel(ctx.shapes, first["variant"]):
+            if reads_units_per_block(ctx.shapes, first["variant"]):
                 for upb in [u for u in UPB if u in (space or {}).get("upb", UPB)]:
                     cand = dict(first, upb=upb)
                     try:

@@ -47,6 +47,36 @@ def test_candidates_restricted_to_a_space():
     assert len(got) == 3 * 2 * 3
 
 
+@pytest.mark.parametrize("L,generic_wins", [(10, False), (10, True), (24, False), (4, False)])
+def test_tuner_times_no_launch_twice(monkeypatch, L, generic_wins):
+    """Variant 1 is the kernel of variant 3, and only the generic kernel (variant 2, or L < 6)
+    reads the units per block: each form is timed once."""
+    torch = pytest.importorskip("torch")
+    monkeypatch.setattr(torch.cuda, "get_device_name", lambda d: "fake")
+    monkeypatch.setattr(tuner, "cache_key", lambda s, d: "key")
+    timed = []
+
+    class Context:
+        shapes, device = [Q.Shape(L, 64, 64, 1, 1)], "cuda"
+        now = {}
+
+        def qsg_set_option(self, option, value):
+            self.now[option] = value
+
+        def __getattr__(self, name):  # spins and counters, saved and put back
+            return lambda *a: (0, 0, 0)
+
+    def time_call(ctx, n, reps):
+        timed.append(dict(ctx.now))
+        return 1.0 if generic_wins == (ctx.now[Q.OPT_WAVEFRONT_VARIANT] == 2) else 2.0
+
+    monkeypatch.setattr(tuner, "_time_call", time_call)
+    tuner.tune(Context(), sweeps_per_call=4, cache_path=None, use_cache=False)
+    assert timed and not any(c[Q.OPT_WAVEFRONT_VARIANT] == 1 for c in timed)
+    tried = {c[Q.OPT_UNITS_PER_BLOCK] for c in timed}
+    assert tried == ({0, 1, 2, 4, 8, 16} if generic_wins or L < 6 else {0})
+
+
 @pytest.mark.gpu
 def test_tuned_context_samples_the_same_bits(tmp_path):
     torch = pytest.importorskip("torch")
