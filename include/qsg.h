@@ -445,7 +445,9 @@ qsg_status qsg_sweep_static_scratch(uint64_t *d_spins, const uint64_t *d_Jx, con
                                     uint32_t first_sweep, int32_t n_sweeps, void *cuda_stream);
 
 /* Number of kernels this library has launched in this process (all contexts);
- * a diagnostic for benchmarks and for checking that the GPU path ran. */
+ * a diagnostic for benchmarks and for checking that the GPU path ran.  How many a
+ * call of qsg_sweep takes depends on the form that the sizes and options choose:
+ * one for several sweeps, one or two per sweep. */
 uint64_t qsg_kernel_launches(void);
 
 const char *qsg_strerror(qsg_status status);

@@ -556,12 +556,12 @@ static bool few_large_slots(const Group &g) {
 
 // Very few words without a graph: the plain kernel's two short launches take less
 // than a chunk's chain of steps.  us per sweep, plain / chunked: L = 12, L_tau = 330, 2
-// slots 8.3 / 12.4; L = 24, L_tau = 100, 6 slots 12.4 / 14.7; L = 8, L_tau = 700, 8 slots 12.4
-// / 12.4; L = 6 (16 chunks per block in lockstep), L_tau = 820, 16 slots 16.5 / 22.6, 120
-// slots 62 / 38.  For L_tau a multiple of 16, which the graphs take, chunks as ever.
+// slots 8.3 / 12.4; L = 24, L_tau = 100, 6 slots 12.4 / 15.1; L = 8, L_tau = 700, 8 slots 12.3
+// / 12.4; L = 6 (14 chunks per block in lockstep), L_tau = 820, 16 slots 16.5 / 18.5, 32
+// slots 22.6 / 18.5.  For L_tau a multiple of 16, which the graphs take, chunks as ever.
 static bool plain_pays(const qsg_ctx *ctx, const Group &g, const uint32_t *sb) {
     if (sb || ctx->sweep_kernel != 0 || g_wavefront_variant != 0 || g.Ltau % 16 == 0) return false;
-    return (double)g.N * (double)g.nslots < (g.L == 6 ? 1.5e6 : 4e5);
+    return (double)g.N * (double)g.nslots < (g.L == 6 ? 6e5 : 4e5);
 }
 
 // Several sweeps of a group in one launch, the slots in shared memory: where a

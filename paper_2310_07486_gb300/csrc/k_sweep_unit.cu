@@ -40,9 +40,9 @@ static void residency(const Group &g, int *nsm, int *per, int *chunks) {
 // (filling the ring, the deferred boundary sites); a last wave that puts x of an
 // SM's `per` blocks on the fullest SM takes x / per of a full one, but not below
 // kThin (one block alone does not fill an SM).  Against measured times (L = 24,
-// L_tau = 2048, 256 slots; 1, 3, 4, 5, 7, 12, 16 chunks) the ratios agree within 4
-// %; seven chunks are the best of them, and the choice.  Chunks need not divide
-// L_tau: they differ by two planes at most.
+// L_tau = 2048, 256 slots; 3, 4, 5, 7, 12, 16 chunks) the ratios agree within 4 %, for a
+// single chunk within 8 %; seven chunks are the best of them, and the choice.  Chunks
+// need not divide L_tau: they differ by two planes at most.
 // Blocks of one warp (L = 8) are the load of one of an SM's four schedulers, so they are
 // counted per scheduler, and x of the `per` blocks there take (x / per)^0.9 of a full
 // wave.  Counted per SM, the choice for L_tau = 1024, 92 slots was 18 chunks in 31.4 us

@@ -61,9 +61,8 @@ __host__ __device__ constexpr int units_per_block(int L) {
 }
 // Registers of a thread: 80, which nearly every size needs to be free of spills, where
 // as many blocks fit an SM as with 72 (by registers, 24 against 28 warps, or by the
-// ring), else 72.  72 / 80, us per sweep: L = 8, L_tau = 1024, 92 slots 33.0 / 31.6; L = 18,
-// L_tau = 1024, 64 slots 90.2 / 88.4; L = 22, L_tau = 512, 64 slots 62.7 / 61.0; L = 30, L_tau
-// = 512, 32 slots 68.6 / 66.2; L = 16, L_tau = 512, 96 slots 50.1 / 50.2.
+// ring), else 72.  72 / 80, us per sweep: L = 18, L_tau = 2048, 92 slots 239 / 235; L = 16,
+// L_tau = 512, 96 slots 51.3 / 49.8 (heat bath), L_tau = 2048, 128 slots 205.6 / 202.3.
 __host__ __device__ constexpr int unit_regs(int L) {
     const int warps = (units_per_block(L) * L * L / 2 + 31) / 32;
     const int ring = 227 * 1024 / (units_per_block(L) * kRing * L * L * 8 + 1280);
