@@ -5,6 +5,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -205,6 +207,46 @@ uint64_t pt_factor(double delta, long long n) {
 
 }  // namespace
 
+// Host words for the contexts' copies of their device flag, in one page that is
+// page-locked once for the process: page-locked memory of a context's own would make
+// its destruction wait for all work on the device (cudaFreeHost).  A context past the
+// page's 512 takes ordinary memory, whose copies are slower.
+class FlagWords {
+public:
+    static int *take() {
+        std::lock_guard<std::mutex> lock(mutex());
+        if (!registered_) {
+            registered_ = true;
+            if (cudaHostRegister(page_, sizeof(page_), cudaHostRegisterPortable) != cudaSuccess) cudaGetLastError();
+        }
+        for (int i = 0; i < kSlots; ++i)
+            if (!used_[i]) {
+                used_[i] = true;
+                return page_ + kWords * i;
+            }
+        return new (std::nothrow) int[kWords];
+    }
+    static void give(int *p) {
+        if (p < page_ || p >= page_ + kWords * kSlots) {
+            delete[] p;
+            return;
+        }
+        std::lock_guard<std::mutex> lock(mutex());
+        used_[(p - page_) / kWords] = false;
+    }
+
+private:
+    static constexpr int kSlots = 512, kWords = 2;
+    static std::mutex &mutex() {
+        static std::mutex m;
+        return m;
+    }
+    alignas(4096) static int page_[kWords * kSlots];
+    static bool used_[kSlots], registered_;
+};
+alignas(4096) int FlagWords::page_[FlagWords::kWords * FlagWords::kSlots];
+bool FlagWords::used_[FlagWords::kSlots], FlagWords::registered_ = false;
+
 // Everything that a captured graph of sweeps holds by value.
 struct GraphKey {
     int batch = 0, kernel = 0, mode = 0, variant = 0, chunk = 0, tail = 0, upb = 0;
@@ -257,7 +299,7 @@ struct qsg_ctx {
     // writer of the correlator buffers waits for
     cudaEvent_t fin_ev = nullptr, copy_ev = nullptr;
     bool copy_pending = false;
-    // page-locked copies of the device flag: [0] taken with the copies of an
+    // copies of the device flag (FlagWords): [0] taken with the copies of an
     // asynchronous read, [1] as last read by fetch_flag
     int *h_flag = nullptr;
     // kernels that may set the device flag were queued since it was last read, or
@@ -269,7 +311,7 @@ struct qsg_ctx {
         if (copy_pending) cudaEventSynchronize(copy_ev);
         if (fin_ev) cudaEventDestroy(fin_ev);
         if (copy_ev) cudaEventDestroy(copy_ev);
-        if (h_flag) cudaFreeHost(h_flag);
+        if (h_flag) FlagWords::give(h_flag);
         if (graph_exec) cudaGraphExecDestroy(graph_exec);
         if (cap_stream) cudaStreamDestroy(cap_stream);
     }
@@ -392,11 +434,13 @@ qsg_status qsg_create(qsg_ctx **out, const qsg_shape *shapes, int32_t n_groups, 
     carve(c->groups, own_scratch, c->ws, &c->d_err, &c->scratch, &c->scratch_words, &c->pb);
     for (Group &g : c->groups) g.err = c->d_err;
     c->stream = (cudaStream_t)cuda_stream;
-    cudaError_t e = cudaHostAlloc((void **)&c->h_flag, 2 * sizeof(int), cudaHostAllocDefault);
-    if (e == cudaSuccess) {
-        c->h_flag[0] = c->h_flag[1] = DEVERR_NONE;
-        e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream);
+    c->h_flag = FlagWords::take();
+    if (!c->h_flag) {
+        delete c;
+        return QSG_ERR_CUDA;
     }
+    c->h_flag[0] = c->h_flag[1] = DEVERR_NONE;
+    cudaError_t e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * 4, c->stream);
     for (const Group &g : c->groups)
         if (e == cudaSuccess)
             e = cudaMemsetAsync(g.arrivals, 0, sizeof(unsigned) * (size_t)g.nslots * (g.Ltau / 4 > 0 ? g.Ltau / 4 : 1),

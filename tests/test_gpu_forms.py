@@ -373,3 +373,25 @@ def test_workspace_without_the_groups_own_scratch():
         for a, b in zip(got[0], other):
             assert all(np.array_equal(a[0][k], b[0][k]) for k in a[0])
             assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+
+
+def test_contexts_are_made_and_destroyed_beside_running_work():
+    """Neither waits for the device; the words of the flag's copies are given back and more
+    contexts than there are serve all the same."""
+    torch = pytest.importorskip("torch")
+    busy = _context(Q.Shape(24, 1024, 64, 4, 16, Q.HEATBATH), 1)
+    small = Q.Shape(8, 16, 1, 1, 1)
+    _context(small, 2).close()
+    torch.cuda.synchronize()
+    busy.qsg_sweep(3000)  # 0.2 s
+    done = torch.cuda.Event()
+    done.record()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for _ in range(3):
+            Q.Context([small]).close()
+    assert not done.query()
+    many = [Q.Context([small]) for _ in range(520)]
+    for ctx in (many[0], many[-1]):
+        ctx.qsg_init_samples(2, [[0.3]])
+        ctx.qsg_sweep(2)
+    assert np.array_equal(many[0].qsg_get_spins(0), many[-1].qsg_get_spins(0))
