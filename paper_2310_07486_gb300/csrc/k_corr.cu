@@ -326,9 +326,7 @@ struct Divisor {
         y = __drcp_rn(by);
         yl = __dmul_rn(__fma_rn(-d, y, 1.0), y);
     }
-    // (by zero, with the count of measurements set to zero: the infinity or NaN of a division)
     __device__ __forceinline__ double into(double x) const {
-        if (d == 0.0) return __ddiv_rn(x, d);
         const double q = __fma_rn(x, y, __dmul_rn(x, yl));
         return __fma_rn(__fma_rn(-q, d, x), y, q);
     }
@@ -349,6 +347,14 @@ __global__ void k_finish(Group g, double nm) {
     }
     __syncthreads();
     const Divisor c = by[0], q = by[1];
+    if (nm == 0.0) {  // a count set to zero: the infinities and NaN of a division
+        for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nc; i += (size_t)gridDim.x * blockDim.x) {
+            g.outC[i] = __ddiv_rn((double)g.Cacc[i], 0.0);
+            g.outQ[i] = __ddiv_rn((double)g.Qacc[i], 0.0);
+            if (i < np) g.outP[i] = __ddiv_rn((double)g.Pacc[i], 0.0);
+        }
+        return;
+    }
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nc; i += (size_t)gridDim.x * blockDim.x) {
         g.outC[i] = c.into((double)g.Cacc[i]);
         g.outQ[i] = q.into((double)g.Qacc[i]);
