@@ -568,12 +568,16 @@ constexpr int kMaxDevices = 64;
 
 __device__ __align__(256) unsigned g_static_arrivals[kStaticArrivals];
 __device__ __align__(256) uint32_t g_static_thr[kStaticMaxK * 16];
-__device__ int g_static_status;  // DEVERR_TIMEOUT after a wait of these sweeps gave up
+__device__ int g_static_status;  // DEVERR_TIMEOUT after a wait of these sweeps gave up, where the host word is not mapped
 
 std::mutex g_static_mutex;
 void *g_static_arrivals_ptr[kMaxDevices];
 void *g_static_thr_ptr[kMaxDevices];
 void *g_static_status_ptr[kMaxDevices];
+// The status words on the host, mapped for the kernels where that works: read after the
+// wait that a call makes anyway (a copy of a device word took 8 us of a call).
+alignas(4096) volatile int g_static_seen[kMaxDevices];
+bool g_static_registered = false, g_static_mapped[kMaxDevices];
 
 // Device addresses of the two arrays and the status word on device `dev`, which
 // must be current (looked up, and the counters cleared, on the first call on that
@@ -591,6 +595,18 @@ cudaError_t static_scratch(int dev, void **arrivals, void **thr, void **status) 
         if (e != cudaSuccess) return e;
         e = cudaMemset(a, 0, sizeof(unsigned) * kStaticArrivals);
         if (e != cudaSuccess) return e;
+        int *words = const_cast<int *>(g_static_seen);
+        void *mapped = nullptr;
+        if (!g_static_registered &&
+            cudaHostRegister(words, sizeof(g_static_seen), cudaHostRegisterPortable | cudaHostRegisterMapped) ==
+                cudaSuccess)
+            g_static_registered = true;
+        if (g_static_registered && cudaHostGetDevicePointer(&mapped, words, 0) == cudaSuccess) {
+            s = (int *)mapped + dev;
+            g_static_mapped[dev] = true;
+        } else {
+            cudaGetLastError();
+        }
         g_static_arrivals_ptr[dev] = a;
         g_static_thr_ptr[dev] = t;
         g_static_status_ptr[dev] = s;
@@ -655,15 +671,19 @@ extern "C" qsg_status qsg_internal_static_sweeps(uint64_t *d_spins, const uint64
     if (sdev != dev) return QSG_ERR_ARG;
     void *arr = nullptr, *thr = nullptr, *status = nullptr;
     if (static_scratch(dev, &arr, &thr, &status) != cudaSuccess) return QSG_ERR_CUDA;
-    // the table lives on this function's stack: copy it and wait for the copy; the
-    // status that earlier calls left comes back by the same wait
-    int earlier = DEVERR_NONE;
-    if (cudaMemcpyAsync(&earlier, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return QSG_ERR_CUDA;
+    // the table lives on this function's stack: copy it and wait for the copy, after
+    // which the status that earlier calls left is known, too
+    if (!g_static_mapped[dev] && cudaMemcpyAsync(const_cast<int *>(&g_static_seen[dev]), status, sizeof(int),
+                                                 cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        return QSG_ERR_CUDA;
     if (cudaMemcpyAsync(thr, table, sizeof(uint32_t) * 16 * (size_t)g.K, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return QSG_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return QSG_ERR_CUDA;
-    if (earlier != DEVERR_NONE)  // reported once
-        return cudaMemsetAsync(status, 0, sizeof(int), st) == cudaSuccess ? QSG_ERR_TIMEOUT : QSG_ERR_CUDA;
+    if (g_static_seen[dev] != DEVERR_NONE) {  // reported once
+        g_static_seen[dev] = DEVERR_NONE;
+        if (!g_static_mapped[dev] && cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return QSG_ERR_CUDA;
+        return QSG_ERR_TIMEOUT;
+    }
     // counters start at zero (each sweep leaves them at zero; cleared anyway)
     if (cudaMemsetAsync(arr, 0, sizeof(unsigned) * (size_t)g.nslots * (g.Ltau / C), st) != cudaSuccess)
         return QSG_ERR_CUDA;
